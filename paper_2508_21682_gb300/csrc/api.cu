@@ -14,8 +14,8 @@
 #include "hf_internal.cuh"
 
 size_t sort_status_words(int64_t n, int K, int tb);
-int tie_small_cap(int W, int d, int bits, int K, int K2);
-size_t tie_scratch_words(int W, int d, int bits, int K, int K2);
+int tie_big_min(int W);
+size_t tie_scratch_words(int W);
 
 namespace {
 
@@ -136,7 +136,6 @@ void free_build_scratch(hf_forest* f, cudaStream_t s) {
   dfree(f->sort.vals_b, s);
   dfree(f->sort.status, s);
   dfree(f->sort.hist, s);
-  dfree(f->tie.runs, s);
   dfree(f->tie.big_runs, s);
   dfree(f->tie.counters, s);
   dfree(f->tie.fk, s);
@@ -400,12 +399,10 @@ static int build_impl(const float* points, int64_t n, int32_t d, int32_t T, int3
   chk(dalloc(&f->sort.vals_b, (size_t)TB * n, s));
   chk(dalloc(&f->sort.status, sort_status_words(n, K, TB), s));
   chk(dalloc(&f->sort.hist, (size_t)TB * K * 8 * 256, s));
-  const int cap = tie_small_cap(f->W, d, bits, K, f->K2);
-  f->tie.big_cap = n / (cap + 1) + 1;
-  chk(dalloc(&f->tie.runs, (size_t)(n / 2 + 1), s));
+  f->tie.big_cap = n / (tie_big_min(f->W) + 1) + 1;
   chk(dalloc(&f->tie.big_runs, (size_t)T * f->tie.big_cap, s));
   chk(dalloc(&f->tie.counters, (size_t)T * 4, s));
-  chk(dalloc(&f->tie.fk, K < f->W ? tie_scratch_words(f->W, d, bits, K, f->K2) : 1, s));
+  chk(dalloc(&f->tie.fk, K < f->W ? tie_scratch_words(f->W) : 1, s));
   void* rscratch = nullptr;
   const size_t rbytes = range_scratch_bytes(n, d);
   chk(dalloc_bytes(&rscratch, rbytes, s));
@@ -478,10 +475,10 @@ static int build_impl(const float* points, int64_t n, int32_t d, int32_t T, int3
   dfree(seg64, s);
   if (rc == HF_OK) {
     tm.collect({0, 1, 2, 3});
-    // keys, prefix gather and tie kernels per tree; histogram, scan and 8K
-    // passes per batch
+    // keys per tree; histogram, scan, 8K passes, prefix gather and tie kernels
+    // per batch
     const int nb = (T + TB - 1) / TB;
-    f->timings[6] = (float)(T * (1 + (K > 1 ? 1 : 0) + (K < f->W ? 2 : 0)) + nb * (2 + 8 * K));
+    f->timings[6] = (float)(T + nb * (2 + 8 * K + (K > 1 ? 1 : 0) + (K < f->W ? 3 : 0)));
   }
   free_build_scratch(f, s);
   if (rc != HF_OK) {

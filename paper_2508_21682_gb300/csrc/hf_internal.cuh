@@ -37,11 +37,10 @@ struct SortScratch {  // for a batch of TB trees
 };
 
 struct TieScratch {
-  uint32_t* counters = nullptr;  // [0] runs, [1] big runs, [2] big elements
-  uint2* runs = nullptr;         // (start, len) of runs, capacity n/2 + 1
-  uint2* big_runs = nullptr;     // per tree: runs longer than the small cap
+  uint32_t* counters = nullptr;  // per tree: [0] tied positions, [1] big runs, [2] sub-runs
+  uint2* big_runs = nullptr;     // per tree: runs that the host settles
   int64_t big_cap = 0;           // entries per tree in big_runs
-  uint64_t* fk = nullptr;        // full-key scratch of the small-run fix-up
+  uint64_t* fk = nullptr;        // full-key scratch of the sub-runs
 };
 
 struct hf_forest {

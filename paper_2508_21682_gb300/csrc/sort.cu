@@ -301,11 +301,15 @@ __global__ void __launch_bounds__(NT, 5) onesweep_kernel(const PassArgs a) {
   }
 }
 
-// Sorted prefix words 1..K-1: out[w][p] = pk[w][sigma[p]].
-__global__ void gather_prefix_kernel(const uint64_t* __restrict__ pk, const uint32_t* __restrict__ sigma,
-                                     int64_t n, int K, uint64_t* __restrict__ out,
-                                     const int* __restrict__ err) {
+// Sorted prefix words 1..K-1: out[w][p] = pk[w][sigma[p]]. Tree blockIdx.y of
+// the batch (one launch for all of them).
+__global__ void gather_prefix_kernel(const uint64_t* __restrict__ pk0, int64_t pk_ts,
+                                     const uint32_t* __restrict__ sigma0, int64_t n, int K,
+                                     uint64_t* __restrict__ out0, const int* __restrict__ err) {
   if (*(volatile const int*)err) return;  // the order is not valid: skip
+  const uint64_t* pk = pk0 + blockIdx.y * pk_ts;
+  const uint32_t* sigma = sigma0 + blockIdx.y * n;
+  uint64_t* out = out0 + (size_t)blockIdx.y * K * n;
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n;
        p += (int64_t)gridDim.x * blockDim.x) {
     const uint32_t i = sigma[p];
@@ -317,32 +321,9 @@ __global__ void gather_prefix_kernel(const uint64_t* __restrict__ pk, const uint
 __device__ __forceinline__ bool prefix_eq(const uint64_t* __restrict__ pre, int64_t n, int K,
                                           int64_t a, int64_t b) {
   for (int w = 0; w < K; ++w)
-    if (pre[(size_t)w * n + a] != pre[(size_t)w * n + b]) return false;
+    if (__ldg(pre + (size_t)w * n + a) != __ldg(pre + (size_t)w * n + b)) return false;
   return true;
 }
-
-// Finds maximal runs of >= 2 equal prefixes. Small runs go to `runs`, runs
-// longer than small_cap to `big`.
-__global__ void tie_find_kernel(const uint64_t* __restrict__ pre, int64_t n, int K, int small_cap,
-                                uint2* __restrict__ runs, uint2* __restrict__ big, int64_t big_cap,
-                                uint32_t* __restrict__ counters) {
-  for (int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; m + 1 < n;
-       m += (int64_t)gridDim.x * blockDim.x) {
-    if (!prefix_eq(pre, n, K, m, m + 1)) continue;
-    if (m > 0 && prefix_eq(pre, n, K, m - 1, m)) continue;
-    int64_t len = 2;
-    while (m + len < n && prefix_eq(pre, n, K, m, m + len)) ++len;
-    if (len <= small_cap) {
-      const uint32_t r = atomicAdd(&counters[0], 1u);
-      runs[r] = make_uint2((uint32_t)m, (uint32_t)len);
-    } else {
-      const uint32_t r = atomicAdd(&counters[1], 1u);
-      if (r < big_cap) big[r] = make_uint2((uint32_t)m, (uint32_t)len);
-      atomicAdd(&counters[2], (uint32_t)len);
-    }
-  }
-}
-
 
 __device__ __forceinline__ bool full_less(const uint64_t* a, uint32_t ia, const uint64_t* b,
                                           uint32_t ib, int W) {
@@ -362,118 +343,277 @@ __device__ __forceinline__ uint32_t xor_scan_msb(uint32_t v) {
   return v;
 }
 
-// One block per small run (grid-stride over runs). The run's prefixes (words
-// 0..K-1) are equal, so the order inside it is decided by the following key
-// words K..K2-1. When the key kernel computed them (kpre > K) they are read
-// from pkx[w][point]; otherwise they are computed here: they lie in the top
-// Lf bit levels, and the top Lf levels of a key equal the Lf-bit key of the
-// coordinates' top Lf bits, so they cost a transform with Lf levels only
-// (with Lf = 1 a running XOR, which a warp forms with ballots).
-// Each point's rank = number of run members below it by (words K..K2-1,
-// index). Only if two members also tie on those words does the block compute
-// full keys (into its own slice of global scratch) and rank by (full key,
-// index). Shared layout: tk[cap][K2-K], pt[cap], rank[cap], Y[blockDim][d].
-__global__ void tie_small_kernel(const uint32_t* __restrict__ planes, int64_t n, int d, int W32,
-                                 int bits, int W, int K, int K2, int Lf, int cap,
-                                 const uint64_t* __restrict__ pkx, int kpre,
-                                 const int32_t* __restrict__ pi, const uint32_t* __restrict__ rbits,
-                                 const uint2* __restrict__ runs, const uint32_t* __restrict__ counters,
-                                 uint32_t* __restrict__ sigma, uint64_t* __restrict__ fk_scratch,
-                                 const int* __restrict__ err) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  __shared__ int s_tie;
-  if (*(volatile const int*)err) return;  // the order is not valid: skip
-  const int KT = K2 - K;
-  uint64_t* tk = reinterpret_cast<uint64_t*>(smraw);
-  uint32_t* pt = reinterpret_cast<uint32_t*>(tk + (size_t)cap * KT);
-  uint32_t* rank = pt + cap;
-  uint8_t* Y = reinterpret_cast<uint8_t*>(rank + cap) + (size_t)threadIdx.x * d;
-  uint64_t* fk = fk_scratch + (size_t)blockIdx.x * cap * W;
-  const uint32_t nruns = counters[0];
-  for (uint32_t r = blockIdx.x; r < nruns; r += gridDim.x) {
-    const uint2 run = runs[r];
-    const int len = (int)run.y;  // <= cap by construction
-    if (threadIdx.x == 0) s_tie = 0;
-    if (kpre <= K && Lf == 1) {
-      // Words K .. K2-1 lie in the top bit level: one warp per member forms
-      // them with ballots over the permuted, reflected top bits (plane 0),
-      // carrying the parity of the first 64K bits.
-      const int lane = threadIdx.x & 31;
-      for (int e = threadIdx.x >> 5; e < len; e += blockDim.x >> 5) {
-        const uint32_t p = sigma[run.x + e];
-        if (lane == 0) pt[e] = p;
-        if (p >= (uint64_t)n) continue;  // cannot happen for a valid order
-        const uint32_t* row = planes + (size_t)p * W32;
-        uint32_t carry = 0, hi = 0;
-        for (int h = 0; h < 2 * K2; ++h) {
+// ---------------------------------------------------------------------------
+// Runs of equal prefixes (the LSD passes left each run in index order). Three
+// launches cover every tree of the batch (tree blockIdx.y), with one thread
+// per tied position rather than one block per run: a run has about ten members
+// on clustered data, and a block that holds one run at a time keeps a handful
+// of its lanes busy (4M x 64, T = 16, mixture data with about half of the
+// points tied at 128 bits: 393 ms of kernels in that form; the whole build went
+// from 337 to 20.4 ms, and one of 1.2M x 128 rows with few ties lost 0.8 ms of
+// its 32 small launches).
+//   tie_mark   finds the tied positions, lists them, keeps their points and
+//              the first key word past the prefix (word K) where that is cheap;
+//   tie_words  word K by the transform of the top Lf levels, for the rest;
+//   tie_rank   each member counts the members of its run that precede it.
+// Members that also tie on every word at hand form sub-runs of the ranked
+// order; tie_hard orders those by the full key. Runs longer than TIE_RUN_CAP
+// and sub-runs longer than tie_hard_cap go to the list of big runs, which the
+// host settles after the build's sync.
+// The scratch is the sort's own, free after the last pass: words in keys_a,
+// sub-runs in keys_b, points in vals_a, listed positions in vals_b.
+// ---------------------------------------------------------------------------
+// A member's rank costs one pass over its run: 2^26 word compares for a run at
+// the cap, about 20 us of the whole chip.
+constexpr int TIE_RUN_CAP = 8192;
+// Sub-run members whose full keys fit a block's scratch slice: 304 slices of
+// 256 x 48 words at d = 384 are 30 MB; rows of more than 64 words keep 64.
+__host__ __device__ constexpr int tie_hard_cap(int W) { return W <= 64 ? 256 : 64; }
+
+struct TieArgs {  // the first tree of the batch; strides below
+  const uint64_t* prefix;  // [tb][K][n] sorted
+  const uint64_t* pk;      // [tb][K2][n] key words, point order
+  uint32_t* sigma;         // [tb][n]
+  uint64_t* word;          // [tb][n] word K by position
+  uint2* hard;             // [tb][n] sub-runs (start, len)
+  uint32_t* pt;            // [tb][n] points by position (the order before the fix-up)
+  uint32_t* list;          // [tb][n] tied positions
+  uint2* big;              // [tb][big_cap]
+  uint32_t* counters;      // [tb][4]: listed positions, big runs, sub-runs
+  const uint32_t* planes;
+  const int32_t* pi;       // [tb][d]
+  const uint32_t* rbits;   // [tb][W32]
+  const int* err;
+  int64_t n, big_cap;
+  int d, W32, bits, W, K, K2, Lf, tb, stride;
+};
+
+// WORDS: where word K comes from. 0: the key kernel computed it (K2 > K); 1:
+// it lies in the top bit level (d >= 64 (K + 1)), a warp forms it per tied
+// point with ballots over the permuted, reflected top bits, carrying the
+// parity of the first 64 K; 2: tie_words.
+template <int WORDS>
+__global__ void __launch_bounds__(256) tie_mark_kernel(const TieArgs a) {
+  if (*(volatile const int*)a.err) return;  // the order is not valid: skip
+  const int64_t n = a.n;
+  const int K = a.K, lane = threadIdx.x & 31;
+  const size_t tr = blockIdx.y;
+  const uint64_t* __restrict__ pre = a.prefix + tr * K * n;
+  const uint64_t* __restrict__ pkw = a.pk + tr * a.K2 * n + (size_t)K * n;
+  const uint32_t* __restrict__ sigma = a.sigma + tr * n;
+  uint64_t* __restrict__ word = a.word + tr * n;
+  uint32_t* __restrict__ pt = a.pt + tr * n;
+  uint32_t* __restrict__ list = a.list + tr * n;
+  uint32_t* ctr = a.counters + tr * 4;
+  const int32_t* __restrict__ pi = a.pi + tr * a.d;
+  const uint32_t* __restrict__ rb = a.rbits + tr * a.W32;
+  // whole warps take 32 consecutive positions
+  for (int64_t m0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); m0 < n;
+       m0 += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t m = m0 + lane;
+    const bool tied = m < n && ((m + 1 < n && prefix_eq(pre, n, K, m, m + 1)) ||
+                                (m > 0 && prefix_eq(pre, n, K, m - 1, m)));
+    const uint32_t mask = __ballot_sync(0xffffffffu, tied);
+    if (!mask) continue;
+    uint32_t slot = 0;
+    if (lane == 0) slot = atomicAdd(&ctr[0], (uint32_t)__popc(mask));
+    slot = __shfl_sync(0xffffffffu, slot, 0) + __popc(mask & lanemask_lt());
+    uint32_t p = 0;
+    if (tied) {
+      p = sigma[m];
+      if (p >= (uint64_t)n) p = 0;  // cannot happen for a valid order
+      pt[m] = p;
+      list[slot] = (uint32_t)m;
+      if (WORDS == 0) word[m] = __ldg(pkw + p);
+    }
+    if (WORDS == 1) {
+      for (uint32_t rest = mask; rest; rest &= rest - 1) {
+        const int src = __ffs(rest) - 1;
+        const uint32_t q = __shfl_sync(0xffffffffu, p, src);
+        const uint32_t* row = a.planes + (size_t)q * a.W32;
+        uint32_t carry = 0, half[2] = {0, 0};
+        for (int h = 0; h < 2 * K + 2; ++h) {
           const int c = __ldg(pi + 32 * h + lane);
-          const uint32_t bit = ((__ldg(row + (c >> 5)) >> (c & 31)) ^ (__ldg(rbits + h) >> lane)) & 1u;
+          const uint32_t bit = ((__ldg(row + (c >> 5)) >> (c & 31)) ^ (__ldg(rb + h) >> lane)) & 1u;
           const uint32_t bal = __ballot_sync(0xffffffffu, bit);
           if (h < 2 * K) {
             carry ^= __popc(bal) & 1u;
-            continue;
-          }
-          uint32_t v = xor_scan_msb(__brev(bal));
-          if (carry) v = ~v;
-          carry = v & 1u;
-          if (h & 1) {
-            if (lane == 0) tk[(size_t)e * KT + (h >> 1) - K] = ((uint64_t)hi << 32) | v;
           } else {
-            hi = v;
+            uint32_t v = xor_scan_msb(__brev(bal));
+            if (carry) v = ~v;
+            carry = v & 1u;
+            half[h & 1] = v;
           }
         }
+        if (lane == src) word[m] = ((uint64_t)half[0] << 32) | half[1];
       }
-    } else {
+    }
+  }
+}
+
+// Word K of the listed positions: one thread per member, its coordinates' top
+// Lf bits in shared memory (row stride 4 x odd bytes: the lanes of a warp, all
+// at the same coordinate, fall in distinct banks). The coordinates are filled
+// plane word by plane word (Lf loads per 32 of them) through the inverse
+// permutation. Bound by the transform's dependent shared-memory steps.
+__global__ void tie_words_kernel(const TieArgs a) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  if (*(volatile const int*)a.err) return;
+  const int64_t n = a.n;
+  const size_t tr = blockIdx.y;
+  const uint32_t cnt = a.counters[tr * 4];
+  if ((uint64_t)blockIdx.x * blockDim.x >= cnt) return;
+  const int d = a.d, Lf = a.Lf;
+  int32_t* inv = reinterpret_cast<int32_t*>(smraw);  // inv[pi[i]] = i, sign bit: reflected
+  uint8_t* Y = smraw + (size_t)d * 4 + (size_t)threadIdx.x * a.stride;
+  const uint32_t* __restrict__ rb = a.rbits + tr * a.W32;
+  for (int i = threadIdx.x; i < d; i += blockDim.x) {
+    const uint32_t refl = (__ldg(rb + (i >> 5)) >> (i & 31)) & 1u;
+    inv[__ldg(a.pi + tr * d + i)] = i | (int32_t)(refl << 31);
+  }
+  __syncthreads();
+  const uint32_t full = (1u << Lf) - 1u;
+  for (uint64_t e = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; e < cnt; e += (uint64_t)gridDim.x * blockDim.x) {
+    const uint32_t m = a.list[tr * n + e];
+    const uint32_t p = a.pt[tr * n + m];
+    for (int m32 = 0; m32 < a.W32; ++m32) {
+      uint32_t w[HF_MAX_BITS];
+#pragma unroll
+      for (int l = 0; l < HF_MAX_BITS; ++l)
+        w[l] = l < Lf ? __ldg(a.planes + ((size_t)l * n + p) * a.W32 + m32) : 0u;
+      const int cn = d - 32 * m32 < 32 ? d - 32 * m32 : 32;
+      for (int c = 0; c < cn; ++c) {
+        uint32_t v = 0;
+#pragma unroll
+        for (int l = 0; l < HF_MAX_BITS; ++l)
+          if (l < Lf) v = (v << 1) | ((w[l] >> c) & 1u);
+        const int32_t i = inv[32 * m32 + c];
+        Y[i & 0x7fffffff] = (uint8_t)(i < 0 ? v ^ full : v);
+      }
+    }
+    hf_skilling(Y, d, Lf);
+    a.word[tr * n + m] = hf_pack_word(Y, d, Lf, a.K);
+  }
+}
+
+// First position of the run of equal prefixes that holds m (dir = -1), or the
+// last one (dir = +1): galloping probes, then bisection; the prefixes are
+// sorted, so equality is monotone.
+__device__ __forceinline__ int64_t run_edge(const uint64_t* __restrict__ pre, int64_t n, int K, int64_t m, int dir) {
+  int64_t in = m, step = 1, out;  // `in` is inside the run, `out` the nearest known position outside
+  for (;;) {
+    out = in + dir * step;
+    if (out < 0 || out >= n) {
+      out = out < 0 ? -1 : n;
+      break;
+    }
+    if (!prefix_eq(pre, n, K, m, out)) break;
+    in = out;
+    step <<= 1;
+  }
+  while (out - in > 1 || in - out > 1) {
+    const int64_t mid = (in + out) >> 1;
+    if (mid >= 0 && mid < n && prefix_eq(pre, n, K, m, mid)) in = mid;
+    else out = mid;
+  }
+  return in;
+}
+
+// One thread per listed position. The run's words are read in order (the
+// lanes of a warp mostly share a run: broadcast loads). Ties on every word at
+// hand (word K, and words K+1 .. K2-1 when the key kernel formed them) stay in
+// index order, which is position order; the first of a tied group lists the
+// group as a sub-run when the key has more words.
+__global__ void __launch_bounds__(256) tie_rank_kernel(const TieArgs a) {
+  if (*(volatile const int*)a.err) return;
+  const int64_t n = a.n;
+  const size_t tr = blockIdx.y;
+  uint32_t* ctr = a.counters + tr * 4;
+  const uint32_t cnt = ctr[0];
+  const int K = a.K;
+  const uint64_t* __restrict__ pre = a.prefix + tr * K * n;
+  const uint64_t* __restrict__ pk = a.pk + tr * a.K2 * n;
+  const uint64_t* __restrict__ word = a.word + tr * n;
+  const uint32_t* __restrict__ pt = a.pt + tr * n;
+  uint32_t* __restrict__ sigma = a.sigma + tr * n;
+  uint2* big = a.big + tr * a.big_cap;
+  const int known = a.K2 > K + 1 ? a.K2 : K + 1;  // key words at hand
+  for (uint64_t e = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; e < cnt; e += (uint64_t)gridDim.x * blockDim.x) {
+    const int64_t m = a.list[tr * n + e];
+    const int64_t lo = run_edge(pre, n, K, m, -1), hi = run_edge(pre, n, K, m, 1);
+    if (hi - lo >= TIE_RUN_CAP) {
+      if (m == lo) {
+        const uint32_t r = atomicAdd(&ctr[1], 1u);
+        if (r < a.big_cap) big[r] = make_uint2((uint32_t)lo, (uint32_t)(hi - lo + 1));
+      }
+      continue;
+    }
+    const uint64_t own = word[m];
+    const uint32_t p = pt[m];
+    uint32_t rank = 0, before = 0, after = 0;
+    for (int64_t g = lo; g <= hi; ++g) {
+      const uint64_t v = word[g];
+      if (v < own) ++rank;
+      if (v == own && g != m) {
+        int c = 0;
+        for (int w = K + 1; w < a.K2 && c == 0; ++w) {
+          const uint64_t x = __ldg(pk + (size_t)w * n + pt[g]), y = __ldg(pk + (size_t)w * n + p);
+          c = x < y ? -1 : (x > y ? 1 : 0);
+        }
+        if (c < 0) ++rank;
+        else if (c == 0 && g < m) ++before;
+        else if (c == 0) ++after;
+      }
+    }
+    sigma[lo + rank + before] = p;
+    if (known < a.W && before == 0 && after > 0) {
+      const uint2 sub = make_uint2((uint32_t)(lo + rank), after + 1);
+      if ((int)after < tie_hard_cap(a.W)) {
+        a.hard[tr * n + atomicAdd(&ctr[2], 1u)] = sub;
+      } else {
+        const uint32_t r = atomicAdd(&ctr[1], 1u);
+        if (r < a.big_cap) big[r] = sub;
+      }
+    }
+  }
+}
+
+// Sub-runs that tie on every word at hand: one block each (few: the next 64
+// bits settle all but near-duplicate points), ranked by (full key, index) from
+// full keys in the block's slice of global scratch.
+__global__ void tie_hard_kernel(const TieArgs a, uint64_t* __restrict__ fk_scratch) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  if (*(volatile const int*)a.err) return;
+  const int64_t n = a.n;
+  const int d = a.d, W = a.W;
+  uint32_t* pt = reinterpret_cast<uint32_t*>(smraw);
+  const int cap = tie_hard_cap(W);
+  uint8_t* Y = reinterpret_cast<uint8_t*>(pt + cap) + (size_t)threadIdx.x * d;
+  uint64_t* fk = fk_scratch + (size_t)blockIdx.x * cap * W;
+  for (int tr = 0; tr < a.tb; ++tr) {
+    const uint32_t nruns = a.counters[(size_t)tr * 4 + 2];
+    uint32_t* sigma = a.sigma + (size_t)tr * n;
+    // trees start at different blocks, so that a few sub-runs per tree spread
+    for (uint32_t r = (blockIdx.x + (uint32_t)tr * 37u) % gridDim.x; r < nruns; r += gridDim.x) {
+      const uint2 run = a.hard[(size_t)tr * n + r];
+      const int len = (int)run.y;  // <= cap
       for (int e = threadIdx.x; e < len; e += blockDim.x) {
         const uint32_t p = sigma[run.x + e];
         pt[e] = p;
         if (p >= (uint64_t)n) continue;  // cannot happen for a valid order
-        if (kpre > K) {
-          for (int w = 0; w < KT; ++w) tk[(size_t)e * KT + w] = __ldg(pkx + (size_t)(K + w) * n + p);
-        } else {
-          hf_load_coords_planes(planes, n, d, W32, Lf, pi, rbits, p, Y);
-          hf_skilling(Y, d, Lf);
-          for (int w = 0; w < KT; ++w) tk[(size_t)e * KT + w] = hf_pack_word(Y, d, Lf, K + w);
-        }
-      }
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < len; e += blockDim.x) {
-      uint32_t rk = 0;
-      bool tie = false;
-      for (int g = 0; g < len; ++g) {
-        int c = 0;
-        for (int w = 0; w < KT && c == 0; ++w) {
-          const uint64_t a = tk[(size_t)g * KT + w], b = tk[(size_t)e * KT + w];
-          c = a < b ? -1 : (a > b ? 1 : 0);
-        }
-        if (c == 0 && g != e) tie = true;
-        rk += (c < 0 || (c == 0 && pt[g] < pt[e])) ? 1u : 0u;
-      }
-      rank[e] = rk;
-      if (tie) s_tie = 1;
-    }
-    __syncthreads();
-    if (s_tie && K2 < W) {
-      // rare: the next words tie as well, rank by full keys
-      for (int e = threadIdx.x; e < len; e += blockDim.x) {
-        const uint32_t p = pt[e];
-        if (p >= (uint64_t)n) continue;
-        hf_load_coords_planes(planes, n, d, W32, bits, pi, rbits, p, Y);
-        hf_skilling(Y, d, bits);
-        for (int w = 0; w < W; ++w) fk[(size_t)e * W + w] = hf_pack_word(Y, d, bits, w);
+        hf_load_coords_planes(a.planes, n, d, a.W32, a.bits, a.pi + (size_t)tr * d, a.rbits + (size_t)tr * a.W32, p, Y);
+        hf_skilling(Y, d, a.bits);
+        for (int w = 0; w < W; ++w) fk[(size_t)e * W + w] = hf_pack_word(Y, d, a.bits, w);
       }
       __syncthreads();
       for (int e = threadIdx.x; e < len; e += blockDim.x) {
         uint32_t rk = 0;
         for (int g = 0; g < len; ++g)
           rk += full_less(fk + (size_t)g * W, pt[g], fk + (size_t)e * W, pt[e], W) ? 1u : 0u;
-        rank[e] = rk;
+        sigma[run.x + rk] = pt[e];
       }
       __syncthreads();
     }
-    for (int e = threadIdx.x; e < len; e += blockDim.x) sigma[run.x + rank[e]] = pt[e];
-    __syncthreads();
   }
 }
 
@@ -543,30 +683,16 @@ __global__ void iota_kernel(uint32_t* a, uint32_t m) {
   if (i < m) a[i] = i;
 }
 
-constexpr int TIE_THREADS = 64;
 constexpr int TIE_BLOCKS = 152 * 2;
 
-struct TieGeom {
-  int K2, Lf, cap;
-  size_t smem;
-};
+// Threads of a tie_hard block: their coordinate rows (d bytes each) share the
+// block's shared memory.
+int tie_hard_threads(int d) { return d <= 2048 ? 64 : 32; }
 
-// Words K..K2-1 (up to four) break ties; they lie in the top Lf levels.
-// With kpre > K the key kernel already computed words K..kpre-1.
-TieGeom tie_geom(int W, int d, int bits, int K, int kpre) {
-  TieGeom g;
-  g.K2 = kpre > K ? kpre : (K + 4 < W ? K + 4 : W);
-  const int64_t lf = ((int64_t)64 * g.K2 + d - 1) / d;
-  g.Lf = (int)(lf < bits ? lf : bits);
-  const int KT = g.K2 - K;
-  const size_t y = (size_t)TIE_THREADS * d;
-  const size_t per = (size_t)KT * 8 + 8;
-  size_t cap = (96 * 1024 - (y < 96 * 1024 ? y : 96 * 1024)) / per;
-  if (cap > 256) cap = 256;
-  if (cap < 2) cap = 2;
-  g.cap = (int)cap;
-  g.smem = (size_t)g.cap * per + y;
-  return g;
+// Levels that word K needs, and the row stride of tie_words.
+int tie_levels(int d, int bits, int K) {
+  const int64_t lf = ((int64_t)64 * (K + 1) + d - 1) / d;
+  return (int)(lf < bits ? lf : bits);
 }
 
 }  // namespace
@@ -650,31 +776,65 @@ int sort_batch(hf_forest* f, int t0, int tb, cudaStream_t s) {
       a.vals_in_ts = a.vals_out_ts;
     }
   }
-  for (int j = 0; j < tb; ++j) {
-    const int t = t0 + j;
-    const uint64_t* pkt = f->pk + (size_t)j * pk_ts;
-    uint64_t* pre = f->prefix + (size_t)t * K * n;
-    uint32_t* sig = f->sigma + (size_t)t * n;
-    if (K > 1) {
-      gather_prefix_kernel<<<hf_blocks(n, 256, 152 * 8), 256, 0, s>>>(pkt, sig, n, K, pre, f->err);
-      hf_after_launch("gather_prefix_kernel", s);
+  // per tree blocks of the launches below: about 16 blocks per SM over all trees
+  const int64_t tree_cap = (152 * 16 + tb - 1) / tb;
+  if (K > 1) {
+    gather_prefix_kernel<<<dim3(hf_blocks(n, 256, tree_cap), (unsigned)tb), 256, 0, s>>>(
+        f->pk, pk_ts, f->sigma + (size_t)t0 * n, n, K, f->prefix + (size_t)t0 * K * n, f->err);
+    hf_after_launch("gather_prefix_kernel", s);
+  }
+  // Equal prefixes, settled on the device right away. With K == W the prefix
+  // is the whole key: equal prefixes are equal keys, already in index order.
+  if (K < f->W) {
+    TieArgs a{};
+    a.prefix = f->prefix + (size_t)t0 * K * n;
+    a.pk = f->pk;
+    a.sigma = f->sigma + (size_t)t0 * n;
+    a.word = f->sort.keys_a;
+    a.hard = reinterpret_cast<uint2*>(f->sort.keys_b);
+    a.pt = f->sort.vals_a;
+    a.list = f->sort.vals_b;
+    a.big = f->tie.big_runs + (size_t)t0 * f->tie.big_cap;
+    a.counters = f->tie.counters + (size_t)t0 * 4;
+    a.planes = f->planes;
+    a.pi = f->pi + (size_t)t0 * f->d;
+    a.rbits = f->rbits + (size_t)t0 * f->W32;
+    a.err = f->err;
+    a.n = n;
+    a.big_cap = f->tie.big_cap;
+    a.d = f->d;
+    a.W32 = f->W32;
+    a.bits = f->bits;
+    a.W = f->W;
+    a.K = K;
+    a.K2 = K2;
+    a.Lf = tie_levels(f->d, f->bits, K);
+    a.tb = tb;
+    a.stride = ((f->d + 3) / 4 | 1) * 4;
+    const dim3 grid(hf_blocks(n, 256, tree_cap), (unsigned)tb);
+    if (K2 > K) {
+      tie_mark_kernel<0><<<grid, 256, 0, s>>>(a);
+      hf_after_launch("tie_mark_kernel", s);
+    } else if (f->d >= 64 * (K + 1)) {
+      tie_mark_kernel<1><<<grid, 256, 0, s>>>(a);
+      hf_after_launch("tie_mark_kernel", s);
+    } else {
+      tie_mark_kernel<2><<<grid, 256, 0, s>>>(a);
+      hf_after_launch("tie_mark_kernel", s);
+      // d < 64 (K + 1) <= 576 here: a block of 128 rows holds 75 KB at most
+      const size_t sm = (size_t)f->d * 4 + (size_t)128 * a.stride;
+      set_attr((const void*)tie_words_kernel, sm);
+      tie_words_kernel<<<dim3(hf_blocks(n, 128, 2 * tree_cap), (unsigned)tb), 128, sm, s>>>(a);
+      hf_after_launch("tie_words_kernel", s);
     }
-    // Equal prefixes: find runs, fix the small ones on the device right
-    // away. With K == W the prefix is the whole key: equal prefixes are equal
-    // keys, already in index order.
-    if (K < f->W) {
-      const TieGeom tg = tie_geom(f->W, f->d, f->bits, K, K2);
-      uint32_t* ctr = f->tie.counters + (size_t)t * 4;
-      cudaMemsetAsync(ctr, 0, 4 * sizeof(uint32_t), s);
-      tie_find_kernel<<<hf_blocks(n, 256, 152 * 8), 256, 0, s>>>(pre, n, K, tg.cap, f->tie.runs,
-                                                                f->tie.big_runs + (size_t)t * f->tie.big_cap,
-                                                                f->tie.big_cap, ctr);
-      hf_after_launch("tie_find_kernel", s);
-      set_attr((const void*)tie_small_kernel, tg.smem);
-      tie_small_kernel<<<TIE_BLOCKS, TIE_THREADS, tg.smem, s>>>(
-          f->planes, n, f->d, f->W32, f->bits, f->W, K, tg.K2, tg.Lf, tg.cap, pkt, K2, f->pi + (size_t)t * f->d,
-          f->rbits + (size_t)t * f->W32, f->tie.runs, ctr, sig, f->tie.fk, f->err);
-      hf_after_launch("tie_small_kernel", s);
+    tie_rank_kernel<<<grid, 256, 0, s>>>(a);
+    hf_after_launch("tie_rank_kernel", s);
+    if ((K2 > K + 1 ? K2 : K + 1) < f->W) {
+      const int ht = tie_hard_threads(f->d);
+      const size_t sm = (size_t)tie_hard_cap(f->W) * 4 + (size_t)ht * f->d;
+      set_attr((const void*)tie_hard_kernel, sm);
+      tie_hard_kernel<<<TIE_BLOCKS, ht, sm, s>>>(a, f->tie.fk);
+      hf_after_launch("tie_hard_kernel", s);
     }
   }
   return cudaGetLastError() == cudaSuccess ? HF_OK : HF_ECUDA;
@@ -793,14 +953,13 @@ int tie_fixup_big(hf_forest* f, int t, uint32_t nbig, cudaStream_t s) {
   return rc;
 }
 
-size_t tie_scratch_words(int W, int d, int bits, int K, int K2) {
-  const TieGeom g = tie_geom(W, d, bits, K, K2);
-  return (size_t)TIE_BLOCKS * g.cap * W;
-}
+// Words of the sub-runs' full-key scratch.
+size_t tie_scratch_words(int W) { return (size_t)TIE_BLOCKS * tie_hard_cap(W) * W; }
+
+// Runs and sub-runs on the big list are longer than this.
+int tie_big_min(int W) { return tie_hard_cap(W); }
 
 size_t sort_status_words(int64_t n, int K, int tb) {
   const int64_t ntiles = (n + TILE - 1) / TILE;
   return ((size_t)tb * (ntiles + 1) * 256 + 1) * 8 * K;
 }
-
-int tie_small_cap(int W, int d, int bits, int K, int K2) { return tie_geom(W, d, bits, K, K2).cap; }
