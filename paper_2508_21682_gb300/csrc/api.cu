@@ -433,7 +433,7 @@ static int build_impl(const float* points, int64_t n, int32_t d, int32_t T, int3
 
   cudaEvent_t a0 = tm.mark();
   if (nseg > 1)
-    launch_seg_range(f->x, d, f->seg_off, nseg, bits, f->lo, f->scale, f->err, s);
+    launch_seg_range(f->x, n, d, f->seg_off, f->seg, nseg, bits, f->lo, f->scale, f->err, s);
   else
     launch_range(f->x, n, d, f->lo, f->scale, bits, f->err, rscratch, rbytes, s);
   launch_quantize_planes(f->x, n, d, f->lo, f->scale, bits, f->planes, f->err, s, nseg > 1 ? f->seg : nullptr);

@@ -119,8 +119,8 @@ void launch_range(const float* x, int64_t n, int d, float* lo, float* scale, int
 size_t range_scratch_bytes(int64_t n, int d);
 // segmented matrix (rows off[s] .. off[s+1]-1 form set s): per-set range
 // (lo / scale: nseg x d) and the set of every row
-void launch_seg_range(const float* x, int d, const int64_t* off, int nseg, int bits, float* lo, float* scale, int* err,
-                      cudaStream_t s);
+void launch_seg_range(const float* x, int64_t n, int d, const int64_t* off, const uint32_t* seg, int nseg, int bits,
+                      float* lo, float* scale, int* err, cudaStream_t s);
 void launch_seg_of_row(const int64_t* off, int nseg, int64_t n, uint32_t* seg, uint64_t* seg64, cudaStream_t s);
 void launch_quantize_planes(const float* x, int64_t n, int d, const float* lo, const float* scale,
                             int bits, uint32_t* planes, int* err, cudaStream_t s, const uint32_t* seg = nullptr);
