@@ -1194,6 +1194,11 @@ int hf_search(hf_forest* f, const float* queries, int64_t nq, int32_t k, int32_t
   if (e == cudaSuccess) e = dalloc(&qc, (size_t)nq * d, s);
   if (e == cudaSuccess && !li) e = dalloc(&li, cnt, s);
   if (e == cudaSuccess && !ldd) e = dalloc(&ldd, cnt, s);
+  const int64_t parts = f->mode == 3 ? 1 : search_parts(f, nq, w);
+  uint32_t* part_i = nullptr;
+  float* part_d = nullptr;
+  if (e == cudaSuccess && parts > 1) e = dalloc(&part_i, cnt * parts, s);
+  if (e == cudaSuccess && parts > 1) e = dalloc(&part_d, cnt * parts, s);
   int rc = map_cuda(e);
   Timer tm(f, s);
   if (rc == HF_OK) {
@@ -1204,7 +1209,7 @@ int hf_search(hf_forest* f, const float* queries, int64_t nq, int32_t k, int32_t
     if (rc == HF_OK && f->mode == 3)
       rc = sketch_search(f, qsrc, qc, nq, k, w, li, ldd, s);
     else if (rc == HF_OK)
-      rc = launch_search(f, qsrc, qc, nq, k, w, li, ldd, nullptr, -1, s);
+      rc = launch_search(f, qsrc, qc, nq, k, w, li, ldd, nullptr, -1, s, part_i, part_d);
     cudaEvent_t a1 = tm.mark();
     tm.span(5, a0, a1);
     if (rc == HF_OK && !dev_i) rc = map_cuda(cudaMemcpyAsync(out_idx, li, cnt * 4, cudaMemcpyDeviceToHost, s));
@@ -1215,6 +1220,8 @@ int hf_search(hf_forest* f, const float* queries, int64_t nq, int32_t k, int32_t
   }
   dfree(qd, s);
   dfree(qc, s);
+  dfree(part_i, s);
+  dfree(part_d, s);
   if (!dev_i) dfree(li, s);
   if (!dev_d) dfree(ldd, s);
   return rc;

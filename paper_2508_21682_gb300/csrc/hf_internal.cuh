@@ -204,7 +204,10 @@ void launch_f32_to_bf16(const float* x, int64_t rows, int cols, int ld, void* ou
 // search.cu
 int launch_search(const hf_forest* f, const float* q, const uint8_t* qcodes, int64_t nq, int k,
                   int w, uint32_t* out_idx, float* out_dist, int64_t* out_pos, int only_tree,
-                  cudaStream_t s);
+                  cudaStream_t s, uint32_t* part_idx = nullptr, float* part_dist = nullptr);
+// warps that share one query of a batch (1: no split); a split search keeps a
+// list of k per part in part_idx / part_dist (nq x parts x k)
+int64_t search_parts(const hf_forest* f, int64_t nq, int w);
 // sketch form of the search: positions of every tree (pos, T x nq) and query
 // sketches (qsk) first; needs f->sketch, f->xm and f->posm
 int launch_sketch_search(const hf_forest* f, const float* q, int64_t nq, const int64_t* pos, const uint64_t* qsk,

@@ -95,6 +95,11 @@ struct SearchArgs {
   int pos_all;  // positions of every tree into out_pos[t * nq + query], no lists
   int vec4;  // d % 4 == 0 and both matrices 16-byte aligned
   int top;   // the K prefix words lie in the top bit level (d >= 64K)
+  // parts of a query: warp `part` takes trees tp, tp + tsplit, ... and, in
+  // each window, the 32-candidate chunks cp, cp + csplit, ... (part = tp *
+  // csplit + cp). One part: out_idx / out_dist hold the result. More: they
+  // hold a list of k per part, which merge_parts_kernel merges.
+  int tsplit, csplit;
 };
 
 // Query prefix from the top bits, the warp taking 32 coordinates per ballot:
@@ -269,17 +274,21 @@ __global__ void __launch_bounds__(SWARPS * 32) search_kernel(SearchArgs a) {
   uint8_t* Yq = reinterpret_cast<uint8_t*>(cpid + 32);
   uint8_t* Yd = Yq + a.d;
 
-  const int64_t qi = (int64_t)blockIdx.x * SWARPS + wib;
+  const int parts = a.tsplit * a.csplit;
+  const int64_t li = (int64_t)blockIdx.x * SWARPS + wib;  // this warp's list
+  const int64_t qi = parts == 1 ? li : li / parts;
   if (qi >= a.nq) return;
+  const int part = (int)(li - qi * parts);
+  const int tp = part / a.csplit, cp = part - tp * a.csplit;
   const uint8_t* qc = a.qcodes + (size_t)qi * a.d;
   const float* qv = a.q + (size_t)qi * a.d;
 
   WarpList<S> list;
   list.init();
 
-  const int t_begin = a.only_tree >= 0 ? a.only_tree : 0;
+  const int t_begin = a.only_tree >= 0 ? a.only_tree : tp;
   const int t_end = a.only_tree >= 0 ? a.only_tree + 1 : a.T;
-  for (int t = t_begin; t < t_end; ++t) {
+  for (int t = t_begin; t < t_end; t += a.tsplit) {
     const int32_t* pi = a.pi + (size_t)t * a.d;
     const uint32_t* rb = a.rbits + (size_t)t * a.W32;
     const uint64_t* pre = a.prefix + (size_t)t * a.K * a.n;
@@ -319,7 +328,7 @@ __global__ void __launch_bounds__(SWARPS * 32) search_kernel(SearchArgs a) {
     }
     const int64_t c0 = pos - a.w > 0 ? pos - a.w : 0;
     const int64_t c1 = pos + a.w < a.n ? pos + a.w : a.n;
-    for (int64_t cb = c0; cb < c1; cb += 32) {
+    for (int64_t cb = c0 + 32 * cp; cb < c1; cb += 32 * a.csplit) {
       const int64_t c = cb + lane;
       uint32_t pid = c < c1 ? __ldg(sig + c) : 0xffffffffu;
       float dist;
@@ -389,8 +398,62 @@ __global__ void __launch_bounds__(SWARPS * 32) search_kernel(SearchArgs a) {
   for (int s = 0; s < S; ++s) {
     const int e = 32 * s + lane;
     if (e < a.k) {
-      a.out_idx[(size_t)qi * a.k + e] = list.iv[s];
-      a.out_dist[(size_t)qi * a.k + e] = list.dv[s];
+      a.out_idx[(size_t)li * a.k + e] = list.iv[s];
+      a.out_dist[(size_t)li * a.k + e] = list.dv[s];
+    }
+  }
+}
+
+// Top k of a query's part lists (each ascending): one warp per query, the
+// parts in turn, 32 entries at a time until the first that cannot enter. A
+// point found by several parts has the same distance in each; the insertion
+// drops the repeats.
+template <int S>
+__global__ void __launch_bounds__(SWARPS * 32)
+merge_parts_kernel(const uint32_t* __restrict__ pidx, const float* __restrict__ pdist, int64_t nq, int parts, int k,
+                   uint32_t* __restrict__ out_idx, float* __restrict__ out_dist) {
+  const int lane = threadIdx.x & 31;
+  const int64_t qi = (int64_t)blockIdx.x * SWARPS + (threadIdx.x >> 5);
+  if (qi >= nq) return;
+  WarpList<S> list;
+  list.init();
+  const int64_t total = (int64_t)parts * k;
+  const uint32_t* qidx = pidx + (size_t)qi * total;
+  const float* qdist = pdist + (size_t)qi * total;
+  uint32_t nid = lane < k ? __ldg(qidx + lane) : 0xffffffffu;  // the next part's first entries are in flight
+  float nd = lane < k ? __ldg(qdist + lane) : INFINITY;
+  for (int p = 0; p < parts; ++p) {
+    bool more = true;
+    for (int e0 = 0; e0 < k && more; e0 += 32) {
+      uint32_t id = nid;
+      float dv = nd;
+      if (e0) {
+        id = e0 + lane < k ? __ldg(qidx + (size_t)p * k + e0 + lane) : 0xffffffffu;
+        dv = e0 + lane < k ? __ldg(qdist + (size_t)p * k + e0 + lane) : INFINITY;
+      } else if (p + 1 < parts) {
+        nid = lane < k ? __ldg(qidx + (size_t)(p + 1) * k + lane) : 0xffffffffu;
+        nd = lane < k ? __ldg(qdist + (size_t)(p + 1) * k + lane) : INFINITY;
+      }
+      for (int u = 0; u < 32; ++u) {
+        const float cd = __shfl_sync(FULL, dv, u);
+        const uint32_t ci = __shfl_sync(FULL, id, u);
+        float kd;
+        uint32_t ki;
+        list.last(k, kd, ki);
+        if (ci == 0xffffffffu || !lessp(cd, ci, kd, ki)) {
+          more = false;
+          break;
+        }
+        list.insert(cd, ci, k, lane);
+      }
+    }
+  }
+#pragma unroll
+  for (int s = 0; s < S; ++s) {
+    const int e = 32 * s + lane;
+    if (e < k) {
+      out_idx[(size_t)qi * k + e] = list.iv[s];
+      out_dist[(size_t)qi * k + e] = list.dv[s];
     }
   }
 }
@@ -401,15 +464,48 @@ int launch_s(const SearchArgs& a, size_t smem, cudaStream_t s) {
       cudaFuncSetAttribute((const void*)search_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
           cudaSuccess)
     return HF_ECUDA;
-  search_kernel<S><<<hf_blocks(a.nq, SWARPS), SWARPS * 32, smem, s>>>(a);
+  search_kernel<S><<<hf_blocks(a.nq * a.tsplit * a.csplit, SWARPS), SWARPS * 32, smem, s>>>(a);
   hf_after_launch("search_kernel", s);
   return HF_OK;
 }
 
+template <int S>
+void launch_merge(const SearchArgs& a, uint32_t* out_idx, float* out_dist, cudaStream_t s) {
+  merge_parts_kernel<S><<<hf_blocks(a.nq, SWARPS), SWARPS * 32, 0, s>>>(a.out_idx, a.out_dist, a.nq,
+                                                                       a.tsplit * a.csplit, a.k, out_idx, out_dist);
+  hf_after_launch("merge_parts_kernel", s);
+}
+
+// Parts per query. One warp walks all T trees of a query in T dependent steps
+// (key, probes, rows: about 30 us each at 200,000 x 384), which is the whole
+// time of a small batch; the trees, then the chunks of a window, go to as many
+// time of a small batch (5 queries, T = 32, w = 32: 1001 us a call, 107 split
+// into 64 parts each); the trees, then the chunks of a window, go to as many
+// warps as give the chip SPLIT_WARPS of them. From half that many queries on
+// the batch fills the chip by itself.
+ int64_t SPLIT_WARPS = 152 * 16;
+
+void search_split(int64_t nq, int T, int w, int* tsplit, int* csplit) {
+  const int64_t want = SPLIT_WARPS / nq;
+  *tsplit = *csplit = 1;
+  if (want < 2) return;
+  *tsplit = (int)(want < T ? want : T);
+  const int64_t chunks = ((int64_t)2 * w + 31) / 32, rest = want / *tsplit;
+  *csplit = (int)(rest < chunks ? rest : chunks);
+  if (*csplit > 4) *csplit = 4;  // the merge walks the parts one by one
+}
+
 }  // namespace
 
+int64_t search_parts(const hf_forest* f, int64_t nq, int w) {
+  int ts, cs;
+  search_split(nq, f->T, w, &ts, &cs);
+  return (int64_t)ts * cs;
+}
+
 int launch_search(const hf_forest* f, const float* q, const uint8_t* qcodes, int64_t nq, int k, int w,
-                  uint32_t* out_idx, float* out_dist, int64_t* out_pos, int only_tree, cudaStream_t s) {
+                  uint32_t* out_idx, float* out_dist, int64_t* out_pos, int only_tree, cudaStream_t s,
+                  uint32_t* part_idx, float* part_dist) {
   if (k < 1 || k > 64) return HF_EINVAL;
   SearchArgs a;
   a.x = f->x;
@@ -440,9 +536,26 @@ int launch_search(const hf_forest* f, const float* q, const uint8_t* qcodes, int
   a.vec4 = (f->d % 4 == 0) && ((reinterpret_cast<uintptr_t>(f->x) & 15) == 0) &&
            ((reinterpret_cast<uintptr_t>(q) & 15) == 0);
   a.top = f->d >= 64 * f->K;
+  a.tsplit = a.csplit = 1;
+  if (a.pos_all) {
+    // positions only: trees are independent, nothing to merge
+    int cs;
+    search_split(nq, f->T, 1, &a.tsplit, &cs);
+  } else if (a.only_tree < 0 && part_idx) {
+    search_split(nq, f->T, w, &a.tsplit, &a.csplit);
+  }
+  const bool parts = !a.pos_all && a.tsplit * a.csplit > 1;
+  if (parts) {
+    a.out_idx = part_idx;
+    a.out_dist = part_dist;
+  }
   const size_t smem = search_per_warp(f->K, f->d) * SWARPS;
   const int rc = k <= 32 ? launch_s<1>(a, smem, s) : launch_s<2>(a, smem, s);
   if (rc != HF_OK) return rc;
+  if (parts) {
+    if (k <= 32) launch_merge<1>(a, out_idx, out_dist, s);
+    else launch_merge<2>(a, out_idx, out_dist, s);
+  }
   return cudaGetLastError() == cudaSuccess ? HF_OK : HF_ECUDA;
 }
 
