@@ -165,6 +165,7 @@ void destroy(hf_forest* f, cudaStream_t s) {
   dfree(f->plan_ld, s);
   dfree(f->plan_xs, s);
   dfree(f->plan_ms, s);
+  dfree(f->plan_band, s);
   if (f->side) {
     cudaStreamSynchronize(s);  // the stream-ordered frees above run before the side stream goes
     cudaStreamDestroy(f->side);
@@ -592,10 +593,12 @@ int knn_graph_impl(hf_forest* f, int32_t k, int32_t w, const int32_t* wpt, const
   // gathered on a side stream while the Gram band of this tree runs)
   void* xs[2] = {nullptr, nullptr};
   float2* ms[2] = {nullptr, nullptr};
+  float* band = nullptr;      // plain and sketch forms: pair distances of one row chunk
   uint16_t* pw = nullptr;     // per-point windows of one tree
   int32_t* tile_w = nullptr;  // per-tile windows of one tree
   cudaError_t e = dalloc(&li, (size_t)n * kp, s);
   if (e == cudaSuccess) e = dalloc(&ldd, (size_t)n * kp, s);
+  if (e == cudaSuccess && !tensor) e = dalloc(&band, window_band_bytes(n, w) / sizeof(float), s);
   if (e == cudaSuccess && budget) e = dalloc(&pw, (size_t)n, s);
   if (e == cudaSuccess && budget) e = dalloc(&tile_w, (size_t)(n + 127) / 128, s);
   for (int b = 0; b < (T_use > 1 ? 2 : 1) && tensor; ++b) {
@@ -625,6 +628,7 @@ int knn_graph_impl(hf_forest* f, int32_t k, int32_t w, const int32_t* wpt, const
       dfree(xs[b], s);
       dfree(ms[b], s);
     }
+    dfree(band, s);
     dfree(pw, s);
     dfree(tile_w, s);
     return map_cuda(e);
@@ -666,9 +670,9 @@ int knn_graph_impl(hf_forest* f, int32_t k, int32_t w, const int32_t* wpt, const
       }
     } else if (sketchf) {
       rc = launch_window_hamming(reinterpret_cast<const uint32_t*>(f->sketch), n, f->sketch_bits / 32,
-                                 f->sigma + (size_t)t * n, w, kp, li, ldd, s, f->seg, f->seg_off);
+                                 f->sigma + (size_t)t * n, w, kp, li, ldd, band, s, f->seg, f->seg_off);
     } else
-      rc = launch_window_graph(f->x, n, f->d, f->sigma + (size_t)t * n, w, kp, li, ldd, s, f->seg, f->seg_off);
+      rc = launch_window_graph(f->x, n, f->d, f->sigma + (size_t)t * n, w, kp, li, ldd, band, s, f->seg, f->seg_off);
   }
   if (tensor) {
     // nothing of the side stream may outlive the buffers freed on s
@@ -715,6 +719,7 @@ int knn_graph_impl(hf_forest* f, int32_t k, int32_t w, const int32_t* wpt, const
     dfree(xs[b], s);
     dfree(ms[b], s);
   }
+  dfree(band, s);
   dfree(pw, s);
   dfree(tile_w, s);
   return rc;
@@ -760,6 +765,12 @@ int hf_graph_plan(hf_forest* f, int32_t k, int32_t w, int32_t threads, void* str
     e = dalloc(&f->plan_li, (size_t)n * kp, s);
     if (e == cudaSuccess) e = dalloc(&f->plan_ld, (size_t)n * kp, s);
   }
+  if (e == cudaSuccess && !form && window_band_bytes(n, w) > f->plan_band_bytes) {
+    dfree(f->plan_band, s);
+    f->plan_band_bytes = 0;
+    e = dalloc(&f->plan_band, window_band_bytes(n, w) / sizeof(float), s);
+    if (e == cudaSuccess) f->plan_band_bytes = window_band_bytes(n, w);
+  }
   if (e == cudaSuccess && form && (form != f->plan_form || !f->plan_xs)) {
     dfree(f->plan_xs, s);
     dfree(f->plan_ms, s);
@@ -782,6 +793,8 @@ int hf_graph_plan(hf_forest* f, int32_t k, int32_t w, int32_t threads, void* str
     dfree(f->plan_ld, s);
     dfree(f->plan_xs, s);
     dfree(f->plan_ms, s);
+    dfree(f->plan_band, s);
+    f->plan_band_bytes = 0;
     f->plan_kp = 0;
     return map_cuda(e);
   }
@@ -808,8 +821,8 @@ static int enqueue_graph(hf_forest* f, int32_t* out_idx, float* out_dist, cudaSt
       rc = launch_gram_window(form, n, f->d, sig, f->plan_w, nullptr, nullptr, kp, f->plan_li, f->plan_ld, f->err,
                               f->plan_xs, f->plan_ms, s, f->seg, f->seg_off);
     } else {
-      rc = launch_window_graph(f->x, n, f->d, sig, f->plan_w, kp, f->plan_li, f->plan_ld, s, f->seg, f->seg_off,
-                               f->plan_nt);
+      rc = launch_window_graph(f->x, n, f->d, sig, f->plan_w, kp, f->plan_li, f->plan_ld, f->plan_band, s, f->seg,
+                               f->seg_off, f->plan_nt);
     }
   }
   if (rc == HF_OK) rc = launch_rerank(f->x, n, f->d, f->sigma, kp, kp, f->plan_li, f->plan_ld, s);

@@ -101,6 +101,8 @@ struct hf_forest {
   float* plan_ld = nullptr;
   void* plan_xs = nullptr;     // tensor forms: operand rows in tree order
   float2* plan_ms = nullptr;
+  float* plan_band = nullptr;  // plain form: pair distances of one row chunk
+  size_t plan_band_bytes = 0;
   int plan_k = 0, plan_w = 0, plan_kp = 0, plan_nt = 0, plan_form = 0;
   int sketch_k2 = 60;     // candidates kept by Hamming distance (mode 3)
   int expand_h = 2;       // master-order neighbours per survivor (mode 3 search)
@@ -152,13 +154,15 @@ int tie_fixup_big(hf_forest* f, int tree, uint32_t big_runs, cudaStream_t s);
 
 // window.cu
 int window_list_pitch(int k);  // list slots per point kept by the window kernel (>= k)
+// scratch of a tree's pair distances (one row chunk of it)
+size_t window_band_bytes(int64_t n, int w);
 int launch_window_graph(const float* x, int64_t n, int d, const uint32_t* sigma, int w, int kp,
-                        uint32_t* list_idx, float* list_dist, cudaStream_t s,
+                        uint32_t* list_idx, float* list_dist, float* band, cudaStream_t s,
                         const uint32_t* segr = nullptr, const int64_t* segoff = nullptr, int nt = 0);
 void launch_list_init(uint32_t* idx, float* dist, int64_t count, cudaStream_t s);
 // the same over binary sketches (words 32-bit words per point), Hamming distance
 int launch_window_hamming(const uint32_t* sketch, int64_t n, int words, const uint32_t* sigma, int w, int kp,
-                          uint32_t* list_idx, float* list_dist, cudaStream_t s,
+                          uint32_t* list_idx, float* list_dist, float* band, cudaStream_t s,
                           const uint32_t* segr = nullptr, const int64_t* segoff = nullptr);
 
 // gram.cu -- tensor-core window distances. form 1: BF16 operands; form 2:

@@ -451,11 +451,41 @@ __global__ void __launch_bounds__(256) tie_mark_kernel(const TieArgs a) {
   }
 }
 
+// inv[pi[i]] = i, sign bit set where permuted axis i is reflected; the whole
+// block, which synchronises before the table is used.
+__device__ __forceinline__ void tie_inverse(const int32_t* __restrict__ pi, const uint32_t* __restrict__ rb, int d,
+                                            int32_t* inv) {
+  for (int i = threadIdx.x; i < d; i += blockDim.x) {
+    const uint32_t refl = (__ldg(rb + (i >> 5)) >> (i & 31)) & 1u;
+    inv[__ldg(pi + i)] = i | (int32_t)(refl << 31);
+  }
+}
+
+// Y[i] = top Lf bits of permuted, reflected coordinate i of point p, filled
+// plane word by plane word (Lf loads per 32 coordinates).
+__device__ __forceinline__ void tie_load_row(const uint32_t* __restrict__ planes, int64_t n, int d, int W32, int Lf,
+                                             const int32_t* inv, uint32_t p, uint8_t* Y) {
+  const uint32_t full = (1u << Lf) - 1u;
+  for (int m32 = 0; m32 < W32; ++m32) {
+    uint32_t w[HF_MAX_BITS];
+#pragma unroll
+    for (int l = 0; l < HF_MAX_BITS; ++l) w[l] = l < Lf ? __ldg(planes + ((size_t)l * n + p) * W32 + m32) : 0u;
+    const int cn = d - 32 * m32 < 32 ? d - 32 * m32 : 32;
+    for (int c = 0; c < cn; ++c) {
+      uint32_t v = 0;
+#pragma unroll
+      for (int l = 0; l < HF_MAX_BITS; ++l)
+        if (l < Lf) v = (v << 1) | ((w[l] >> c) & 1u);
+      const int32_t i = inv[32 * m32 + c];
+      Y[i & 0x7fffffff] = (uint8_t)(i < 0 ? v ^ full : v);
+    }
+  }
+}
+
 // Word K of the listed positions: one thread per member, its coordinates' top
 // Lf bits in shared memory (row stride 4 x odd bytes: the lanes of a warp, all
-// at the same coordinate, fall in distinct banks). The coordinates are filled
-// plane word by plane word (Lf loads per 32 of them) through the inverse
-// permutation. Bound by the transform's dependent shared-memory steps.
+// at the same coordinate, fall in distinct banks). Bound by the transform's
+// dependent shared-memory steps.
 __global__ void tie_words_kernel(const TieArgs a) {
   extern __shared__ __align__(16) unsigned char smraw[];
   if (*(volatile const int*)a.err) return;
@@ -464,33 +494,14 @@ __global__ void tie_words_kernel(const TieArgs a) {
   const uint32_t cnt = a.counters[tr * 4];
   if ((uint64_t)blockIdx.x * blockDim.x >= cnt) return;
   const int d = a.d, Lf = a.Lf;
-  int32_t* inv = reinterpret_cast<int32_t*>(smraw);  // inv[pi[i]] = i, sign bit: reflected
+  int32_t* inv = reinterpret_cast<int32_t*>(smraw);
   uint8_t* Y = smraw + (size_t)d * 4 + (size_t)threadIdx.x * a.stride;
-  const uint32_t* __restrict__ rb = a.rbits + tr * a.W32;
-  for (int i = threadIdx.x; i < d; i += blockDim.x) {
-    const uint32_t refl = (__ldg(rb + (i >> 5)) >> (i & 31)) & 1u;
-    inv[__ldg(a.pi + tr * d + i)] = i | (int32_t)(refl << 31);
-  }
+  tie_inverse(a.pi + tr * d, a.rbits + tr * a.W32, d, inv);
   __syncthreads();
-  const uint32_t full = (1u << Lf) - 1u;
   for (uint64_t e = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; e < cnt; e += (uint64_t)gridDim.x * blockDim.x) {
     const uint32_t m = a.list[tr * n + e];
     const uint32_t p = a.pt[tr * n + m];
-    for (int m32 = 0; m32 < a.W32; ++m32) {
-      uint32_t w[HF_MAX_BITS];
-#pragma unroll
-      for (int l = 0; l < HF_MAX_BITS; ++l)
-        w[l] = l < Lf ? __ldg(a.planes + ((size_t)l * n + p) * a.W32 + m32) : 0u;
-      const int cn = d - 32 * m32 < 32 ? d - 32 * m32 : 32;
-      for (int c = 0; c < cn; ++c) {
-        uint32_t v = 0;
-#pragma unroll
-        for (int l = 0; l < HF_MAX_BITS; ++l)
-          if (l < Lf) v = (v << 1) | ((w[l] >> c) & 1u);
-        const int32_t i = inv[32 * m32 + c];
-        Y[i & 0x7fffffff] = (uint8_t)(i < 0 ? v ^ full : v);
-      }
-    }
+    tie_load_row(a.planes, n, d, a.W32, Lf, inv, p, Y);
     hf_skilling(Y, d, Lf);
     a.word[tr * n + m] = hf_pack_word(Y, d, Lf, a.K);
   }
@@ -580,7 +591,9 @@ __global__ void __launch_bounds__(256) tie_rank_kernel(const TieArgs a) {
 
 // Sub-runs that tie on every word at hand: one block each (few: the next 64
 // bits settle all but near-duplicate points), ranked by (full key, index) from
-// full keys in the block's slice of global scratch.
+// full keys in the block's slice of global scratch. The time is that of one
+// member's key, a serial chain: 0.49 ms at d = 384 with the coordinates read
+// bit by bit through the permutation.
 __global__ void tie_hard_kernel(const TieArgs a, uint64_t* __restrict__ fk_scratch) {
   extern __shared__ __align__(16) unsigned char smraw[];
   if (*(volatile const int*)a.err) return;
@@ -588,20 +601,25 @@ __global__ void tie_hard_kernel(const TieArgs a, uint64_t* __restrict__ fk_scrat
   const int d = a.d, W = a.W;
   uint32_t* pt = reinterpret_cast<uint32_t*>(smraw);
   const int cap = tie_hard_cap(W);
-  uint8_t* Y = reinterpret_cast<uint8_t*>(pt + cap) + (size_t)threadIdx.x * d;
+  int32_t* inv = reinterpret_cast<int32_t*>(pt + cap);
+  uint8_t* Y = reinterpret_cast<uint8_t*>(inv + d) + (size_t)threadIdx.x * a.stride;
   uint64_t* fk = fk_scratch + (size_t)blockIdx.x * cap * W;
   for (int tr = 0; tr < a.tb; ++tr) {
     const uint32_t nruns = a.counters[(size_t)tr * 4 + 2];
     uint32_t* sigma = a.sigma + (size_t)tr * n;
     // trees start at different blocks, so that a few sub-runs per tree spread
-    for (uint32_t r = (blockIdx.x + (uint32_t)tr * 37u) % gridDim.x; r < nruns; r += gridDim.x) {
+    const uint32_t first = (blockIdx.x + (uint32_t)tr * 37u) % gridDim.x;
+    if (first >= nruns) continue;
+    tie_inverse(a.pi + (size_t)tr * d, a.rbits + (size_t)tr * a.W32, d, inv);
+    __syncthreads();
+    for (uint32_t r = first; r < nruns; r += gridDim.x) {
       const uint2 run = a.hard[(size_t)tr * n + r];
       const int len = (int)run.y;  // <= cap
       for (int e = threadIdx.x; e < len; e += blockDim.x) {
         const uint32_t p = sigma[run.x + e];
         pt[e] = p;
         if (p >= (uint64_t)n) continue;  // cannot happen for a valid order
-        hf_load_coords_planes(a.planes, n, d, a.W32, a.bits, a.pi + (size_t)tr * d, a.rbits + (size_t)tr * a.W32, p, Y);
+        tie_load_row(a.planes, n, d, a.W32, a.bits, inv, p, Y);
         hf_skilling(Y, d, a.bits);
         for (int w = 0; w < W; ++w) fk[(size_t)e * W + w] = hf_pack_word(Y, d, a.bits, w);
       }
@@ -831,7 +849,7 @@ int sort_batch(hf_forest* f, int t0, int tb, cudaStream_t s) {
     hf_after_launch("tie_rank_kernel", s);
     if ((K2 > K + 1 ? K2 : K + 1) < f->W) {
       const int ht = tie_hard_threads(f->d);
-      const size_t sm = (size_t)tie_hard_cap(f->W) * 4 + (size_t)ht * f->d;
+      const size_t sm = (size_t)(tie_hard_cap(f->W) + f->d) * 4 + (size_t)ht * a.stride;
       set_attr((const void*)tie_hard_kernel, sm);
       tie_hard_kernel<<<TIE_BLOCKS, ht, sm, s>>>(a, f->tie.fk);
       hf_after_launch("tie_hard_kernel", s);
