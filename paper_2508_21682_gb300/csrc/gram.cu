@@ -25,8 +25,8 @@
 // tensor memory and merges the estimated distances into the point's top-KP
 // list (KP >= k + slack). Two halves of four warps share a tile: half h takes
 // the 32-column chunks of parity h, each half keeps its own list for the row,
-// and at the end of the tile half 1 hands its list to half 0 through shared
-// memory, which merges it and writes the point's list back.
+// and at the end of the tile half 1 hands the entries it added to half 0
+// through shared memory, which merges them and writes the point's list back.
 //
 // After the last tree, rerank_kernel recomputes every listed candidate's
 // distance in float32 with exact coordinate differences from the float32
@@ -74,45 +74,101 @@ __device__ __forceinline__ void tc_fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
-// Whole warp: allocates `ncols` tensor-memory columns, writes the base
-// address to *slot (shared memory).
+// Every tcgen05 wrapper below takes PAIR: false, one CTA works by itself
+// (cta_group::1); true, the two CTAs of a cluster work on one tile
+// (cta_group::2), each holding its half of the operands and the accumulator.
+
+// Whole warp (PAIR: one warp of each CTA): allocates `ncols` tensor-memory
+// columns, writes the base address to *slot (shared memory).
+template <bool PAIR>
 __device__ __forceinline__ void tmem_alloc(uint32_t* slot, uint32_t ncols) {
-  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)),
-               "r"(ncols)
-               : "memory");
-  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  if (PAIR) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)), "r"(ncols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  } else {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)), "r"(ncols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
 }
+template <bool PAIR>
 __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
-  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+  if (PAIR)
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+  else
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 
-// D[tmem] (+)= A * B^T, A: M x 16, B: N x 16, both K-major BF16 in shared memory.
-__device__ __forceinline__ void mma_bf16(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                         uint32_t accumulate) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dtmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
+// D[tmem] (+)= A * B^T over one 128-byte K chunk, both K-major in shared
+// memory: four instructions of 32 bytes a row (BF16 K = 16, e4m3 K = 32), two
+// descriptor units apart. The whole warp calls it and one elected lane issues:
+// called from a branch of one lane, each instruction's operands go through the
+// vector registers, about 200 cycles an instruction against the 128 that one
+// of M = 128, N = 256, K = 16 takes to execute.
+template <bool F8, bool PAIR>
+__device__ __forceinline__ void mma_chunk(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                          uint32_t accumulate) {
+#define HF_MMA(GROUP, KIND)                                                                                         \
+  asm volatile(                                                                                                     \
+      "{\n .reg .pred p, t, e;\n .reg .b64 a, b;\n elect.sync _|e, 0xffffffff;\n setp.ne.b32 p, %4, 0;\n"          \
+      " setp.eq.b32 t, 0, 0;\n @e tcgen05.mma.cta_group::" GROUP ".kind::" KIND " [%0], %1, %2, %3, p;\n"           \
+      " add.s64 a, %1, 2;\n add.s64 b, %2, 2;\n"                                                                    \
+      " @e tcgen05.mma.cta_group::" GROUP ".kind::" KIND " [%0], a, b, %3, t;\n"                                    \
+      " add.s64 a, %1, 4;\n add.s64 b, %2, 4;\n"                                                                    \
+      " @e tcgen05.mma.cta_group::" GROUP ".kind::" KIND " [%0], a, b, %3, t;\n"                                    \
+      " add.s64 a, %1, 6;\n add.s64 b, %2, 6;\n"                                                                    \
+      " @e tcgen05.mma.cta_group::" GROUP ".kind::" KIND " [%0], a, b, %3, t;\n}\n" ::"r"(dtmem),                   \
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)                                                           \
+      : "memory")
+  if (PAIR) {
+    if (F8) HF_MMA("2", "f8f6f4");
+    else HF_MMA("2", "f16");
+  } else {
+    if (F8) HF_MMA("1", "f8f6f4");
+    else HF_MMA("1", "f16");
+  }
+#undef HF_MMA
 }
-// The same with e4m3 A and B (K = 32 per instruction, 32 bytes per row).
-__device__ __forceinline__ void mma_f8(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                       uint32_t accumulate) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n}\n" ::"r"(dtmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-// Arrives on *bar once all MMAs issued so far by this thread have completed.
+// Whole warp: arrives on *bar (PAIR: on the barrier at that offset in both
+// CTAs) once all MMAs issued so far by the elected lane have completed.
+template <bool PAIR>
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                   smem_u32(bar))
-               : "memory");
+  if (PAIR)
+    asm volatile(
+        "{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n"
+        " @e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n}" ::"r"(
+            smem_u32(bar)),
+        "h"((uint16_t)3)
+        : "memory");
+  else
+    asm volatile(
+        "{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n"
+        " @e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}" ::"r"(smem_u32(bar))
+        : "memory");
 }
 
-// 32 consecutive FP32 columns of this thread's tensor-memory lane.
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* v) {
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Cluster-wide address of this CTA's shared-memory object in CTA `rank`.
+__device__ __forceinline__ uint32_t peer_addr(const void* p, uint32_t rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr) {
+  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+}
+
+// 32 consecutive FP32 columns of this thread's tensor-memory lane: issue, and
+// wait (the wait names the registers, so that no use moves above it).
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
       "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
@@ -124,7 +180,16 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* v) {
         "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
       : "r"(taddr)
       : "memory");
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_wait32(uint32_t (&v)[32]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]),
+                 "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]),
+                 "+r"(v[15]), "+r"(v[16]), "+r"(v[17]), "+r"(v[18]), "+r"(v[19]), "+r"(v[20]), "+r"(v[21]),
+                 "+r"(v[22]), "+r"(v[23]), "+r"(v[24]), "+r"(v[25]), "+r"(v[26]), "+r"(v[27]), "+r"(v[28]),
+                 "+r"(v[29]), "+r"(v[30]), "+r"(v[31])
+               :
+               : "memory");
 }
 
 // Shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups
@@ -223,6 +288,8 @@ struct GramArgs {
   int elem_per_chunk;      // 64 (BF16) or 128 (FP8) elements per chunk
   int w;                   // window when tile_w is null
   int stages;              // B ring stages
+  int box_rows;            // rows per TMA box
+  int solo;                // no tile has more than one unit
   uint32_t a_off, b_off, slot_off, x_off, bar_off;  // shared-memory layout
   uint32_t b_stage_bytes;
   uint32_t* lidx;
@@ -238,12 +305,12 @@ struct GramArgs {
 // operand rows are in the tree's position order (gather_rows_kernel), so a
 // unit's rows are positions [c_lo + 256 j, c_lo + 256 j + Nj) and the tile's
 // own rows positions [s, s + 128).
-//   warp 0      TMA producer (one lane): per K chunk of a unit, boxes of 32
-//               rows x 128 bytes into the B ring (128-byte swizzle, rows
-//               outside the matrix zero-filled);
-//   warp 1      MMA issuer (one lane): per unit, all K chunks into one of two
-//               tensor-memory accumulators (256 columns each); it also owns
-//               the tensor-memory allocation;
+//   warp 0      TMA producer (one lane): per K chunk of a unit, its rows x 128
+//               bytes into the B ring (128-byte swizzle, rows outside the
+//               matrix zero-filled);
+//   warp 1      MMA issuer: per unit, all K chunks into one of two tensor-
+//               memory accumulators (256 columns each); it also owns the
+//               tensor-memory allocation;
 //   warp 2      prep: per unit, the (norm, scale, id) of its columns (and, for
 //               the first unit, of the tile's own rows) into one of NSLOT
 //               slots;
@@ -252,7 +319,17 @@ struct GramArgs {
 //               tile's last MMA reading it has completed;
 //   warps 4..11 epilogue: a warp owns tensor-memory lanes 32 (warp % 4) ..
 //               + 31 (tile rows) and, in half h = (warp - 4) / 4, the
-//               32-column chunks of parity h.
+//               32-column chunks of parity h; where no tile has more than one
+//               unit (w <= 64), half h takes the whole units of accumulator h
+//               instead, so that no list is ever shared (1M x 128, w = 32,
+//               T = 16: 481 -> 310 us a tree).
+// PAIR: a cluster of two CTAs works on a tile of 256 positions, CTA r owning
+// rows 128 r .. 128 r + 127. Each stages its own rows (A) and half of every
+// unit's columns (B); the first CTA's MMA warp issues for both
+// (cta_group::2, M = 256), each accumulator half lies in its CTA's tensor
+// memory, and each CTA screens and merges its own rows. The full barriers and
+// the accumulators' empty barriers live in the first CTA, the commits arrive
+// in both.
 // Every barrier wait is bounded (spin_limit ns of %globaltimer); when one
 // gives up, the block raises the error word, every role leaves, and tensor
 // memory is freed after a bounded wait for MMAs in flight.
@@ -268,8 +345,7 @@ constexpr int AW = 3;              // A (own rows) producer warp
 constexpr int EW0 = 4;             // first epilogue warp
 constexpr int PT = (EW0 + 8) * 32;
 constexpr uint32_t TMEM_ALL = 512; // two accumulators of 256 columns
-constexpr int MAX_STAGES = 4;
-constexpr int BOX_ROWS = 32;       // rows per TMA box
+constexpr int MAX_STAGES = 8;      // ring stages (4 of a single CTA, 8 of half the size of a pair)
 
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("{\n .reg .b64 st;\n mbarrier.arrive.shared::cta.b64 st, [%0];\n}\n" ::"r"(smem_u32(bar)) : "memory");
@@ -280,14 +356,23 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t by
                "r"(bytes)
                : "memory");
 }
-// A 2-D box of the tensor map at (x elements, y rows) into shared memory;
-// completion is counted in bytes on *bar.
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
-          dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_u32(bar))
-      : "memory");
+// A 2-D box of the tensor map at (x elements, y rows) into this CTA's shared
+// memory; completion is counted in bytes on the barrier at `bar` (PAIR: a
+// cluster address, the first CTA's barrier counts both CTAs' boxes).
+template <bool PAIR>
+__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
+  if (PAIR)
+    asm volatile(
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
+        "[%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
+        : "memory");
+  else
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
+        "[%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
+        : "memory");
 }
 
 struct Bars {
@@ -353,15 +438,25 @@ __device__ __forceinline__ bool pwait(uint64_t* bar, uint32_t parity, uint64_t l
 struct TileGeom {
   int w, W8, ncol, J;
 };
+template <bool PAIR>
 __device__ __forceinline__ TileGeom tile_geom(const GramArgs& a, int64_t t) {
+  constexpr int TP = PAIR ? 2 * GB : GB;  // positions per tile
   TileGeom g;
-  g.w = a.tile_w ? __ldg(a.tile_w + t) : a.w;
+  g.w = a.w;
+  if (a.tile_w) {  // windows are given per 128 positions
+    if (PAIR) {
+      g.w = __ldg(a.tile_w + 2 * t);
+      if ((2 * t + 1) * GB < a.n) g.w = max(g.w, __ldg(a.tile_w + 2 * t + 1));
+    } else {
+      g.w = __ldg(a.tile_w + t);
+    }
+  }
   if (g.w <= 0) {
     g.w = g.W8 = g.ncol = g.J = 0;
     return g;
   }
   g.W8 = (g.w + 7) & ~7;
-  g.ncol = GB + 2 * g.W8;
+  g.ncol = TP + 2 * g.W8;
   g.J = (g.ncol + SLOT_COLS - 1) / SLOT_COLS;
   return g;
 }
@@ -381,7 +476,7 @@ __device__ __forceinline__ uint32_t pick32(const uint32_t (&v)[32], int j) {
   return (j & 1) ? a2[1] : a2[0];
 }
 
-template <int KP, bool F8>
+template <int KP, bool F8, bool PAIR>
 __global__ void __launch_bounds__(PT, 1) gram_band_kernel(GramArgs a, const __grid_constant__ CUtensorMap xmap) {
   extern __shared__ unsigned char smraw[];
   unsigned char* base = smraw + ((1024u - (smem_u32(smraw) & 1023u)) & 1023u);
@@ -390,14 +485,22 @@ __global__ void __launch_bounds__(PT, 1) gram_band_kernel(GramArgs a, const __gr
   unsigned char* slots = base + a.slot_off;
   float* xd = reinterpret_cast<float*>(base + a.x_off);            // [XE][128] distances
   uint32_t* xi = reinterpret_cast<uint32_t*>(xd + XE * GB);        // [XE][128] indices
+  uint32_t* xc = xi + XE * GB;                                     // [128] entries handed over
   Bars& S = *reinterpret_cast<Bars*>(base + a.bar_off);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int64_t ntiles = (a.n + GB - 1) / GB;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // known to be the same in every lane
+  constexpr int TP = PAIR ? 2 * GB : GB;  // positions per tile
+  const int rank = PAIR ? (int)cluster_rank() : 0;
+  const int64_t ntiles = (a.n + TP - 1) / TP;
+  const int64_t tile0 = PAIR ? blockIdx.x >> 1 : blockIdx.x, tstep = PAIR ? gridDim.x >> 1 : gridDim.x;
   const uint64_t lim = a.spin_limit;
   const int nk = a.nk, stages = a.stages;
+  // the barrier at the same place in the pair's first CTA, whose MMA warp
+  // issues for both
+  auto lead = [&](uint64_t* b) { return PAIR ? peer_addr(b, 0) : smem_u32(b); };
 
-  if (warp == MW) tmem_alloc(&S.tslot, TMEM_ALL);
+  if (warp == MW) tmem_alloc<PAIR>(&S.tslot, TMEM_ALL);
   if (tid == 0) {
     for (int i = 0; i < stages; ++i) {
       mbar_init(&S.full[i], 1);
@@ -409,11 +512,11 @@ __global__ void __launch_bounds__(PT, 1) gram_band_kernel(GramArgs a, const __gr
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(&S.tfull[i], 1);
-      mbar_init(&S.tempty[i], 8);
+      mbar_init(&S.tempty[i], PAIR ? 16 : (a.solo ? 4 : 8));
     }
     for (int i = 0; i < NSLOT; ++i) {
       mbar_init(&S.mfull[i], 32);
-      mbar_init(&S.mempty[i], 8);
+      mbar_init(&S.mempty[i], a.solo ? 4 : 8);
     }
     for (int i = 0; i < 4; ++i) {
       mbar_init(&S.xfull[i], 32);
@@ -424,6 +527,7 @@ __global__ void __launch_bounds__(PT, 1) gram_band_kernel(GramArgs a, const __gr
   }
   tc_fence_before();
   __syncthreads();
+  if (PAIR) cluster_sync();  // both CTAs' barriers exist before either is used
   tc_fence_after();
   const uint32_t tmem = S.tslot;
   volatile int* abort = &S.abort;
@@ -433,14 +537,16 @@ __global__ void __launch_bounds__(PT, 1) gram_band_kernel(GramArgs a, const __gr
     if (lane == 0) {
       uint32_t it = 0;
       bool ok = true;
-      const uint32_t chunk_box = (uint32_t)BOX_ROWS * 128u;
-      for (int64_t t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-        const TileGeom g = tile_geom(a, t);
-        const int64_t s = t * GB, c_lo = s - g.W8;
+      const int BR = a.box_rows;
+      const uint32_t chunk_box = (uint32_t)BR * 128u;
+      for (int64_t t = tile0; t < ntiles && ok; t += tstep) {
+        const TileGeom g = tile_geom<PAIR>(a, t);
+        const int64_t s = t * TP, c_lo = s - g.W8;
         for (int j = 0; j < g.J && ok; ++j) {
-          const int nj = min(SLOT_COLS, g.ncol - SLOT_COLS * j);
-          const int nbox = (nj + BOX_ROWS - 1) / BOX_ROWS;
-          const int y0 = (int)(c_lo + (int64_t)SLOT_COLS * j);
+          // a pair's CTA stages its half of the unit's columns
+          const int nj = min(SLOT_COLS, g.ncol - SLOT_COLS * j) / (PAIR ? 2 : 1);
+          const int nbox = (nj + BR - 1) / BR;
+          const int y0 = (int)(c_lo + (int64_t)SLOT_COLS * j) + rank * nj;
           for (int kc = 0; kc < nk; ++kc, ++it) {
             const int x = kc * a.elem_per_chunk;
             const int st = it % stages;
@@ -448,12 +554,17 @@ __global__ void __launch_bounds__(PT, 1) gram_band_kernel(GramArgs a, const __gr
               ok = false;
               break;
             }
-            mbar_arrive_expect_tx(&S.full[st], (uint32_t)nbox * chunk_box);
-            const uint32_t d0 = smem_u32(bring + (size_t)st * a.b_stage_bytes);
-            for (int b = 0; b < nbox; ++b) tma_load_2d(d0 + (uint32_t)b * chunk_box, &xmap, x, y0 + b * BOX_ROWS, &S.full[st]);
+            if (rank == 0) mbar_arrive_expect_tx(&S.full[st], (PAIR ? 2u : 1u) * (uint32_t)nbox * chunk_box);
+            const uint32_t d0 = smem_u32(bring + (size_t)st * a.b_stage_bytes), fb = lead(&S.full[st]);
+            for (int b = 0; b < nbox; ++b)
+              tma_load_2d<PAIR>(d0 + (uint32_t)b * chunk_box, &xmap, x, y0 + b * BR, fb);
           }
         }
       }
+      // the first CTA's commits still arrive here: wait until every stage is
+      // back before this CTA may end
+      for (int i = 0; PAIR && ok && i < stages; ++i, ++it)
+        ok = pwait(&S.empty[it % stages], ((it / stages) & 1) ^ 1, lim, abort, a.err);
     }
     __syncwarp();
   } else if (warp == AW) {
@@ -463,25 +574,26 @@ __global__ void __launch_bounds__(PT, 1) gram_band_kernel(GramArgs a, const __gr
     if (lane == 0) {
       uint32_t auses = 0;
       bool ok = true;
-      const uint32_t chunk_box = (uint32_t)BOX_ROWS * 128u;
-      for (int64_t t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-        const TileGeom g = tile_geom(a, t);
+      const int BR = a.box_rows;
+      const uint32_t chunk_box = (uint32_t)BR * 128u;
+      for (int64_t t = tile0; t < ntiles && ok; t += tstep) {
+        const TileGeom g = tile_geom<PAIR>(a, t);
         if (g.J <= 1) continue;
-        const int64_t s = t * GB;
+        const int64_t s = t * TP + rank * GB;
         for (int kc = 0; kc < nk; ++kc) {
           if (!pwait(&S.aempty[kc], (auses & 1) ^ 1, lim, abort, a.err)) {
             ok = false;
             break;
           }
-          mbar_arrive_expect_tx(&S.afull[kc], (uint32_t)GB * 128u);
-          const uint32_t d0 = smem_u32(aregion + (size_t)kc * GB * 128);
-#pragma unroll
-          for (int b = 0; b < GB / BOX_ROWS; ++b)
-            tma_load_2d(d0 + (uint32_t)b * chunk_box, &xmap, kc * a.elem_per_chunk, (int)s + b * BOX_ROWS,
-                        &S.afull[kc]);
+          if (rank == 0) mbar_arrive_expect_tx(&S.afull[kc], (PAIR ? 2u : 1u) * (uint32_t)GB * 128u);
+          const uint32_t d0 = smem_u32(aregion + (size_t)kc * GB * 128), fb = lead(&S.afull[kc]);
+          for (int b = 0; b < GB / BR; ++b)
+            tma_load_2d<PAIR>(d0 + (uint32_t)b * chunk_box, &xmap, kc * a.elem_per_chunk, (int)s + b * BR, fb);
         }
         ++auses;
       }
+      for (int kc = 0; PAIR && ok && auses && kc < nk; ++kc)
+        ok = pwait(&S.aempty[kc], (auses & 1) ^ 1, lim, abort, a.err);
     }
     __syncwarp();
   } else if (warp == PW) {
@@ -490,9 +602,9 @@ __global__ void __launch_bounds__(PT, 1) gram_band_kernel(GramArgs a, const __gr
     // the MMA and the epilogue (contiguous reads: the tree's order)
     uint32_t u = 0;
     bool ok = true;
-    for (int64_t t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-      const TileGeom g = tile_geom(a, t);
-      const int64_t s = t * GB, c_lo = s - g.W8;
+    for (int64_t t = tile0; t < ntiles && ok; t += tstep) {
+      const TileGeom g = tile_geom<PAIR>(a, t);
+      const int64_t c_lo = t * TP - g.W8, s = t * TP + rank * GB;
       for (int j = 0; j < g.J && ok; ++j, ++u) {
         const int sl = u % NSLOT;
         const int nj = min(SLOT_COLS, g.ncol - SLOT_COLS * j);
@@ -530,51 +642,48 @@ __global__ void __launch_bounds__(PT, 1) gram_band_kernel(GramArgs a, const __gr
       }
     }
   } else if (warp == MW) {
-    // ---------------- MMA issuer (one lane)
-    if (lane == 0) {
-      uint32_t it = 0, u = 0, auses = 0;
+    // ---------------- MMA issuer (of a pair, the first CTA's); the whole warp
+    // walks the loop, see mma_chunk
+    if (rank == 0) {
+      uint32_t st = 0, sphase = 0, u = 0, auses = 0;
       const uint32_t bb = smem_u32(bring), ab = smem_u32(aregion);
       // FP32 accumulator; BF16 A and B (kind::f16) or e4m3 A and B
       // (kind::f8f6f4); both K-major; M >> 4 at bit 24, N >> 3 at bit 17
-      const uint32_t id0 = (1u << 4) | (F8 ? 0u : ((1u << 7) | (1u << 10))) | ((uint32_t)(GB >> 4) << 24);
+      const uint32_t id0 = (1u << 4) | (F8 ? 0u : ((1u << 7) | (1u << 10))) | ((uint32_t)(TP >> 4) << 24);
       bool ok = true;
-      for (int64_t t = blockIdx.x; t < ntiles && ok && !*abort; t += gridDim.x) {
-        const TileGeom g = tile_geom(a, t);
+      auto wwait = [&](uint64_t* bar, uint32_t par) {
+        return __all_sync(0xffffffffu, pwait(bar, par, lim, abort, a.err));
+      };
+      for (int64_t t = tile0; t < ntiles && ok && !__any_sync(0xffffffffu, *abort); t += tstep) {
+        const TileGeom g = tile_geom<PAIR>(a, t);
         for (int j = 0; j < g.J; ++j, ++u) {
-          const int buf = u & 1;
-          const uint32_t use = u >> 1;
-          if (!pwait(&S.tempty[buf], (use & 1) ^ 1, lim, abort, a.err)) {
+          const uint32_t buf = u & 1;
+          if (!wwait(&S.tempty[buf], ((u >> 1) & 1) ^ 1)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t acc = tmem + (uint32_t)(buf * 256);
+          const uint32_t acc = tmem + buf * 256u;
           const int nj = min(SLOT_COLS, g.ncol - SLOT_COLS * j);
           const uint32_t idesc = id0 | ((uint32_t)(nj >> 3) << 17);
-          for (int kc = 0; kc < nk; ++kc, ++it) {
-            const int st = it % stages;
-            if (!pwait(&S.full[st], (it / stages) & 1, lim, abort, a.err) ||
-                (g.J > 1 && !pwait(&S.afull[kc], auses & 1, lim, abort, a.err))) {
+          for (int kc = 0; kc < nk; ++kc) {
+            if (!wwait(&S.full[st], sphase) || (g.J > 1 && !wwait(&S.afull[kc], auses & 1))) {
               ok = false;
               break;
             }
             tc_fence_after();
-            const uint32_t chunk = bb + (uint32_t)(st * a.b_stage_bytes);
+            const uint32_t chunk = bb + st * a.b_stage_bytes;
             const uint32_t achunk = g.J == 1 ? chunk + (uint32_t)(g.W8 >> 3) * 1024u : ab + (uint32_t)kc * GB * 128u;
-#pragma unroll
-            for (int ks = 0; ks < 4; ++ks) {
-              const uint64_t bdesc = smem_desc(chunk + ks * 32);
-              const uint64_t adesc = smem_desc(achunk + ks * 32);
-              if (F8)
-                mma_f8(acc, adesc, bdesc, idesc, (kc | ks) != 0);
-              else
-                mma_bf16(acc, adesc, bdesc, idesc, (kc | ks) != 0);
+            mma_chunk<F8, PAIR>(acc, smem_desc(achunk), smem_desc(chunk), idesc, kc != 0);
+            mma_commit<PAIR>(&S.empty[st]);
+            if (g.J > 1 && j == g.J - 1) mma_commit<PAIR>(&S.aempty[kc]);
+            if (++st == (uint32_t)stages) {
+              st = 0;
+              sphase ^= 1;
             }
-            mma_commit(&S.empty[st]);
-            if (g.J > 1 && j == g.J - 1) mma_commit(&S.aempty[kc]);
           }
           if (!ok) break;
-          mma_commit(&S.tfull[buf]);
+          mma_commit<PAIR>(&S.tfull[buf]);
         }
         if (g.J > 1) ++auses;
       }
@@ -584,20 +693,29 @@ __global__ void __launch_bounds__(PT, 1) gram_band_kernel(GramArgs a, const __gr
     // ---------------- epilogue: warp EW0 + q + 4 h owns tensor-memory lanes
     // 32 q .. 32 q + 31 (tile rows) and the 32-column chunks of parity h
     const int h = (warp - EW0) >> 2;
+    const bool solo = a.solo != 0;
     const int q = warp & 3;       // a warp may access TMEM lanes 32 (warp % 4) .. + 31
-    const int r = q * 32 + lane;  // tile row = TMEM lane
+    const int r = q * 32 + lane;  // this CTA's row = TMEM lane
+    const int rt = rank * GB + r;  // row of the tile
+    const int rq = rank * GB + 32 * q;  // the warp's first row of the tile
+    const uint32_t tempty0 = lead(&S.tempty[0]), tempty1 = lead(&S.tempty[1]);
     uint32_t u = 0, xr = 0;
     bool ok = true;
     // waits and exits are warp-uniform: tcgen05.ld is .sync.aligned
     auto wwait = [&](uint64_t* bar, uint32_t par) {
       return __all_sync(0xffffffffu, pwait(bar, par, lim, abort, a.err));
     };
-    for (int64_t t = blockIdx.x; t < ntiles && ok && !__any_sync(0xffffffffu, *abort); t += gridDim.x) {
-      const TileGeom g = tile_geom(a, t);
+    for (int64_t t = tile0; t < ntiles && ok && !__any_sync(0xffffffffu, *abort); t += tstep) {
+      const TileGeom g = tile_geom<PAIR>(a, t);
       if (g.J == 0) continue;
-      const int64_t p = t * GB + r;
+      if (solo && (int)(u & 1) != h) {  // the other half's tile
+        ++u;
+        continue;
+      }
+      const int64_t p = t * TP + rt;
       const bool rowok = p < a.n;
       ListK<KP> L;
+      uint32_t fresh = 0;  // list entries of this tile
       float ni = 0.f, c2 = 2.0f;
       uint32_t ip = 0xffffffffu;
       int wlo = 0, whi = -1;
@@ -615,14 +733,14 @@ __global__ void __launch_bounds__(PT, 1) gram_band_kernel(GramArgs a, const __gr
           c2 = F8 ? 2.0f * se.sc[SLOT_COLS + r] : 2.0f;
           int wr = g.w;
           if (rowok && a.pw) wr = min(wr, (int)__ldg(a.pw + ip));
-          // the row's band: columns [r + W8 - wr, r + W8 + wr] except r + W8
-          wlo = r + g.W8 - wr;
-          whi = rowok ? r + g.W8 + wr : -1;
+          // the row's band: columns [rt + W8 - wr, rt + W8 + wr] except rt + W8
+          wlo = rt + g.W8 - wr;
+          whi = rowok ? rt + g.W8 + wr : -1;
           if (rowok && a.segr) {
             // segmented forest: only the positions of the row's own set
-            // (column c is position t * GB - W8 + c)
+            // (column c is position t * TP - W8 + c)
             const uint32_t sg = __ldg(a.segr + ip);
-            const int64_t cbase = t * GB - g.W8;
+            const int64_t cbase = t * TP - g.W8;
             const int64_t plo = __ldg(a.segoff + sg) - cbase, phi = __ldg(a.segoff + sg + 1) - 1 - cbase;
             if (plo > wlo) wlo = (int)plo;
             if (phi < whi) whi = (int)phi;
@@ -641,15 +759,10 @@ __global__ void __launch_bounds__(PT, 1) gram_band_kernel(GramArgs a, const __gr
         }
         tc_fence_after();
         const int u0 = SLOT_COLS * j;
-        const int wb_hi = 32 * q + 31 + 2 * g.W8;  // last band column of the warp
-        const int diag = r + g.W8;
-        // chunks [c0, c0 + 32) of the warp's band inside this unit, parity h
-        int c0 = max(32 * q, u0);
-        if (((c0 >> 5) & 1) != h) c0 += 32;
-        for (; c0 <= wb_hi && c0 < u0 + SLOT_COLS; c0 += 64) {
-          __syncwarp();  // reconverge after the divergent inserts
-          uint32_t v[32];
-          tmem_ld32(tmem + (uint32_t)(buf * 256) + ((uint32_t)(32 * q) << 16) + (uint32_t)(c0 - u0), v);
+        const int wb_hi = rq + 31 + 2 * g.W8;  // last band column of the warp
+        const int diag = rt + g.W8;
+        // screens and merges chunk [c0, c0 + 32), whose products are in v
+        auto process = [&](uint32_t(&v)[32], int c0) {
           const int lo = wlo - c0 > 0 ? wlo - c0 : 0;
           const int hi = whi - c0 < 31 ? whi - c0 : 31;
           uint32_t wm = 0;
@@ -693,55 +806,94 @@ __global__ void __launch_bounds__(PT, 1) gram_band_kernel(GramArgs a, const __gr
           while (hm) {
             const int jj = __ffs(hm) - 1;
             hm &= hm - 1;
-            L.offer(__uint_as_float(pick32(v, jj)) + ni, se.id[(c0 - u0) + jj]);
+            const int at = L.offer(__uint_as_float(pick32(v, jj)) + ni, se.id[(c0 - u0) + jj]);
+            // the entries behind it move up by one, and so do their marks
+            if (at >= 0) fresh = (fresh & ((1u << at) - 1u)) | (1u << at) | (((fresh >> at) << 1) << at);
           }
+          __syncwarp();  // reconverge after the divergent inserts
+        };
+        // the chunks of the warp's band inside this unit that are this half's:
+        // all of them when a tile is one unit, else those of parity h
+        const int step = solo ? 32 : 64;
+        int c0 = max(rq, u0);
+        if (!solo && ((c0 >> 5) & 1) != h) c0 += 32;
+        const int cend = min(wb_hi + 1, u0 + SLOT_COLS);
+        const uint32_t tb = tmem + (uint32_t)(buf * 256) + ((uint32_t)(32 * q) << 16);
+        for (; c0 < cend; c0 += step) {
+          uint32_t v[32];
+          tmem_ld32(tb + (uint32_t)(c0 - u0), v);
+          tmem_wait32(v);
+          process(v, c0);
         }
         tc_fence_before();
         __syncwarp();
         if (lane == 0) {
-          mbar_arrive(&S.tempty[buf]);
+          if (PAIR) mbar_arrive_cluster(buf ? tempty1 : tempty0);
+          else mbar_arrive(&S.tempty[buf]);
           mbar_arrive(&S.mempty[sl]);
         }
       }
       if (!ok) break;
-      // half 1 hands its list to half 0 in rounds of XE entries
-      for (int e0 = 0; e0 < KP && ok; e0 += XE, ++xr) {
-        if (h == 1) {
-          if (!wwait(&S.xempty[q], (xr & 1) ^ 1)) {
-            ok = false;
-            break;
-          }
+      // Half 1 hands its entries of this tile to half 0, XE a round (a second
+      // round only while a list of 32 fills): on settled lists a warp's
+      // busiest row has two or three, where offering the whole list again cost
+      // 16 or 32 dependent steps a tile.
+      constexpr uint32_t MORE = 0x80000000u;
+      if (solo) {
+      } else if (h == 1) {
+        const int total = __popc(KP < 32 ? fresh & ((1u << (KP & 31)) - 1u) : fresh);  // those not pushed out since
+        bool more = true;
+        for (int base0 = 0; more; base0 += XE, ++xr) {
+          ok = wwait(&S.xempty[q], (xr & 1) ^ 1);
+          if (!ok) break;
+          int c = -base0;
 #pragma unroll
-          for (int e = 0; e < XE; ++e) {
-            xd[e * GB + r] = L.d[e0 + e];
-            xi[e * GB + r] = L.i[e0 + e];
-          }
+          for (int e = 0; e < KP; ++e)
+            if ((fresh >> e) & 1u) {
+              if (c >= 0 && c < XE) {
+                xd[c * GB + r] = L.d[e];
+                xi[c * GB + r] = L.i[e];
+              }
+              ++c;
+            }
+          more = __any_sync(0xffffffffu, total > base0 + XE);
+          xc[r] = (uint32_t)max(0, min(XE, total - base0)) | (more ? MORE : 0u);
           mbar_arrive(&S.xfull[q]);
-        } else {
-          if (!wwait(&S.xfull[q], xr & 1)) {
-            ok = false;
-            break;
-          }
-#pragma unroll 1
-          for (int e = 0; e < XE; ++e) L.offer(xd[e * GB + r], xi[e * GB + r]);
+        }
+      } else {
+        bool more = true;
+        for (; more; ++xr) {
+          ok = wwait(&S.xfull[q], xr & 1);
+          if (!ok) break;
+          const uint32_t hc = xc[r];
+          const int cnt = (int)(hc & ~MORE);
+          more = (hc & MORE) != 0;  // the same in every lane
+          for (int e = 0; __any_sync(0xffffffffu, e < cnt); ++e)
+            if (e < cnt) L.offer(xd[e * GB + r], xi[e * GB + r]);
           mbar_arrive(&S.xempty[q]);
         }
       }
-      if (ok && h == 0 && rowok) L.store(a.ldist + (size_t)ip * KP, a.lidx + (size_t)ip * KP);
+      if (ok && (h == 0 || solo) && rowok) L.store(a.ldist + (size_t)ip * KP, a.lidx + (size_t)ip * KP);
     }
   }
   // teardown: the last commit completes before tensor memory is freed
   tc_fence_before();
   __syncthreads();
-  if (warp == MW) {
-    if (*abort) {
-      // MMAs may still be in flight after an abort: give them a bounded time
-      const uint64_t t0 = gtimer();
-      while (gtimer() - t0 < lim) {
-      }
+  if (warp == MW && *abort) {
+    // MMAs may still be in flight after an abort: give them a bounded time
+    const uint64_t t0 = gtimer();
+    while (gtimer() - t0 < lim) {
     }
+  }
+  if (PAIR) {
+    // neither CTA ends (nor frees the pair's tensor memory) while the other
+    // may still reach its shared memory
+    __syncthreads();
+    cluster_sync();
+  }
+  if (warp == MW) {
     tc_fence_after();
-    tmem_dealloc(tmem, TMEM_ALL);
+    tmem_dealloc<PAIR>(tmem, TMEM_ALL);
   }
 }
 
@@ -864,7 +1016,8 @@ __global__ void __launch_bounds__(256, 6) rerank_kernel(const float* __restrict_
 // ---------------------------------------------------------------------------
 struct GramPlan {
   int ok = 0;
-  int rowb = 0, nk = 0, stages = 0;
+  int pair = 0;  // two CTAs per tile
+  int rowb = 0, nk = 0, stages = 0, box_rows = 0, solo = 0;
   uint32_t a_off = 0, b_off = 0, slot_off = 0, x_off = 0, bar_off = 0, b_stage_bytes = 0;
   size_t smem = 0;
 };
@@ -880,19 +1033,27 @@ int max_smem_optin() {
 }
 
 // Shared-memory layout for the widest window wmax of a launch.
-GramPlan gram_plan(int d, int wmax, bool f8, int smem_cap) {
+GramPlan gram_plan(int d, int wmax, bool f8, int smem_cap, bool pair = false) {
   GramPlan p;
+  p.pair = pair;
+  const int max_stages = pair ? MAX_STAGES : MAX_STAGES / 2;
   p.rowb = f8 ? (d + 127) / 128 * 128 : (d + 63) / 64 * 128;
   p.nk = p.rowb / 128;
   if (wmax < 1 || p.nk > 32) return p;
   const int W8 = (wmax + 7) & ~7;
-  const int ncol = GB + 2 * W8;
+  const int ncol = (pair ? 2 * GB : GB) + 2 * W8;
   const int J = (ncol + SLOT_COLS - 1) / SLOT_COLS;
-  const int stage_rows = (J == 1 ? ncol : SLOT_COLS) + BOX_ROWS - 1;  // whole boxes
-  p.b_stage_bytes = (uint32_t)(stage_rows / BOX_ROWS * BOX_ROWS) * 128u;
+  // whole boxes; a pair's CTA stages half of a unit's columns
+  // As few TMA boxes as possible (one lane issues them; 32-row boxes held a
+  // pair's K chunk to 840 cycles where its MMAs take 512): the whole unit when
+  // there is one, else 128 rows, which is a pair's half of a unit.
+  p.solo = J == 1;
+  p.box_rows = J == 1 ? ncol : GB;
+  const int stage_rows = pair ? SLOT_COLS / 2 : J == 1 ? ncol : SLOT_COLS;
+  p.b_stage_bytes = (uint32_t)stage_rows * 128u;
   const size_t a_bytes = J > 1 ? (size_t)p.nk * GB * 128 : 0;
   const size_t slot_bytes = (size_t)NSLOT * SLOT_ENTS * (f8 ? 12 : 8);
-  const size_t x_bytes = (size_t)2 * XE * GB * 4;
+  const size_t x_bytes = (size_t)(2 * XE + 1) * GB * 4;
   const size_t bar_bytes = (sizeof(Bars) + 127) / 128 * 128;
   size_t off = 0;
   p.a_off = (uint32_t)off;
@@ -901,7 +1062,7 @@ GramPlan gram_plan(int d, int wmax, bool f8, int smem_cap) {
   const size_t fixed = a_bytes + slot_bytes + x_bytes + bar_bytes + 1024;
   if ((size_t)smem_cap <= fixed) return p;
   int st = (int)(((size_t)smem_cap - fixed) / p.b_stage_bytes);
-  if (st > MAX_STAGES) st = MAX_STAGES;
+  if (st > max_stages) st = max_stages;
   if (st < 2) return p;
   p.stages = st;
   off += (size_t)st * p.b_stage_bytes;  // stage sizes are multiples of 4 KB
@@ -920,13 +1081,13 @@ GramPlan gram_plan(int d, int wmax, bool f8, int smem_cap) {
 }
 
 // Tensor map of the position-ordered operand rows xs [n][rowb bytes]: boxes
-// of 128 bytes x 32 rows, 128-byte swizzle (the layout the MMA descriptors
+// of 128 bytes x br rows, 128-byte swizzle (the layout the MMA descriptors
 // read), zero fill outside the matrix.
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-int make_row_map(CUtensorMap* map, const void* xs, int64_t n, int rowb, bool f8) {
+int make_row_map(CUtensorMap* map, const void* xs, int64_t n, int rowb, bool f8, int br) {
   static EncodeTiledFn fn = nullptr;
   if (!fn) {
     void* p = nullptr;
@@ -942,7 +1103,7 @@ int make_row_map(CUtensorMap* map, const void* xs, int64_t n, int rowb, bool f8)
   const int esz = f8 ? 1 : 2;
   const cuuint64_t gdim[2] = {(cuuint64_t)(rowb / esz), (cuuint64_t)n};
   const cuuint64_t gstride[1] = {(cuuint64_t)rowb};
-  const cuuint32_t box[2] = {(cuuint32_t)(128 / esz), (cuuint32_t)BOX_ROWS};
+  const cuuint32_t box[2] = {(cuuint32_t)(128 / esz), (cuuint32_t)br};
   const cuuint32_t estr[2] = {1, 1};
   const CUresult r = fn(map, f8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
                         const_cast<void*>(xs), gdim, gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -951,19 +1112,47 @@ int make_row_map(CUtensorMap* map, const void* xs, int64_t n, int rowb, bool f8)
   return r == CUDA_SUCCESS ? HF_OK : HF_ECUDA;
 }
 
-template <int KP, bool F8>
+template <int KP, bool F8, bool PAIR>
 int launch_band(const GramArgs& a, const CUtensorMap& map, size_t smem, cudaStream_t s) {
-  if (cudaFuncSetAttribute((const void*)gram_band_kernel<KP, F8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  if (cudaFuncSetAttribute((const void*)gram_band_kernel<KP, F8, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)smem) != cudaSuccess)
     return HF_ECUDA;
   int sms = 152;
   int dev = 0;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int64_t ntiles = (a.n + GB - 1) / GB;
-  const unsigned grid = (unsigned)(ntiles < sms ? ntiles : sms);
-  gram_band_kernel<KP, F8><<<grid, PT, smem, s>>>(a, map);
+  const int per = PAIR ? 2 : 1;
+  const int64_t ntiles = (a.n + per * GB - 1) / (per * GB);
+  const unsigned grid = (unsigned)(ntiles < sms / per ? ntiles : sms / per) * per;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(PT);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = 2;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = PAIR ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, gram_band_kernel<KP, F8, PAIR>, a, map);  // an error is the call's final check's to find
   hf_after_launch(F8 ? "gram_band_kernel<fp8>" : "gram_band_kernel<bf16>", s);
   return HF_OK;
+}
+
+// One CTA or two per tile. Two stage half of the B rows each (the operand
+// traffic through shared memory falls from 160 to 90 bytes a clock of MMA), at
+// the price of 128 more columns per 256 rows; it pays from five K chunks on,
+// and never where one CTA's column range is a single unit. One against two
+// CTAs, us per tree of 1M points (BF16) or 300,000 (FP8), band launch alone:
+// d = 384, w = 1024: 1538 / 1445 (1862 before both); w = 65: 549 / 535; d =
+// 256, w = 1024: 1251 / 1245; d = 128: 1124 / 1154; FP8 d = 768, w = 512: 758 /
+// 757, w = 1024: 1053 / 1045; FP8 d = 384, w = 512: 722 / 739.
+GramPlan choose_plan(int d, int w, bool f8) {
+  const int cap = max_smem_optin();
+  const GramPlan one = gram_plan(d, w, f8, cap);
+  if (!one.ok || one.solo || one.nk < 5) return one;
+  const GramPlan two = gram_plan(d, w, f8, cap, true);
+  return two.ok ? two : one;
 }
 
 }  // namespace
@@ -999,10 +1188,10 @@ int launch_gram_window(int form, int64_t n, int d, const uint32_t* sigma, int w,
                        const uint16_t* pw, int kp, uint32_t* li, float* ld, int* err, const void* xs, const float2* ms,
                        cudaStream_t s, const uint32_t* segr, const int64_t* segoff) {
   const bool f8 = form == 2;
-  const GramPlan p = gram_plan(d, w, f8, max_smem_optin());
+  const GramPlan p = choose_plan(d, w, f8);
   if (!p.ok) return HF_EINVAL;
   alignas(64) CUtensorMap map;
-  const int rc = make_row_map(&map, xs, n, p.rowb, f8);
+  const int rc = make_row_map(&map, xs, n, p.rowb, f8, p.box_rows);
   if (rc != HF_OK) return rc;
   GramArgs a;
   a.ms = ms;
@@ -1016,6 +1205,8 @@ int launch_gram_window(int form, int64_t n, int d, const uint32_t* sigma, int w,
   a.elem_per_chunk = f8 ? 128 : 64;
   a.w = w;
   a.stages = p.stages;
+  a.box_rows = p.box_rows;
+  a.solo = p.solo;
   a.a_off = p.a_off;
   a.b_off = p.b_off;
   a.slot_off = p.slot_off;
@@ -1026,11 +1217,15 @@ int launch_gram_window(int form, int64_t n, int d, const uint32_t* sigma, int w,
   a.ldist = ld;
   a.err = err;
   a.spin_limit = 2000000000ull;  // 2 s per wait (globaltimer nanoseconds)
-  switch (kp * 2 + (f8 ? 1 : 0)) {
-    case 32: return launch_band<16, false>(a, map, p.smem, s);
-    case 33: return launch_band<16, true>(a, map, p.smem, s);
-    case 64: return launch_band<32, false>(a, map, p.smem, s);
-    case 65: return launch_band<32, true>(a, map, p.smem, s);
+  switch (kp * 4 + (f8 ? 2 : 0) + (p.pair ? 1 : 0)) {
+    case 64: return launch_band<16, false, false>(a, map, p.smem, s);
+    case 65: return launch_band<16, false, true>(a, map, p.smem, s);
+    case 66: return launch_band<16, true, false>(a, map, p.smem, s);
+    case 67: return launch_band<16, true, true>(a, map, p.smem, s);
+    case 128: return launch_band<32, false, false>(a, map, p.smem, s);
+    case 129: return launch_band<32, false, true>(a, map, p.smem, s);
+    case 130: return launch_band<32, true, false>(a, map, p.smem, s);
+    case 131: return launch_band<32, true, true>(a, map, p.smem, s);
     default: return HF_EINVAL;
   }
 }

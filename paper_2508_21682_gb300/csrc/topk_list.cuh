@@ -50,9 +50,10 @@ struct ListK {
       i[j] = 0xffffffffu;
     }
   }
-  // Inserts (cd, ci) unless it is no better than the last slot or listed.
-  __device__ __forceinline__ void offer(float cd, uint32_t ci) {
-    if (!lessp(cd, ci, d[KP - 1], i[KP - 1])) return;
+  // Inserts (cd, ci) unless it is no better than the last slot or listed;
+  // returns its slot, or -1.
+  __device__ __forceinline__ int offer(float cd, uint32_t ci) {
+    if (!lessp(cd, ci, d[KP - 1], i[KP - 1])) return -1;
     // a listed candidate (the common case once lists have settled: the same
     // neighbour comes back in later trees) leaves before the insertion work
     uint32_t dupm[KP];
@@ -62,7 +63,7 @@ struct ListK {
     for (int w = 1; w < KP; w <<= 1)
 #pragma unroll
       for (int j = 0; j + w < KP; j += 2 * w) dupm[j] |= dupm[j + w];
-    if (dupm[0]) return;
+    if (dupm[0]) return -1;
     // insert position: the number of entries below the candidate (balanced
     // tree of bits: short dependency chains)
     uint32_t lowm[KP];
@@ -84,5 +85,6 @@ struct ListK {
       d[j] = shift ? pd : (here ? cd : d[j]);
       i[j] = shift ? pi : (here ? ci : i[j]);
     }
+    return (int)below;
   }
 };
