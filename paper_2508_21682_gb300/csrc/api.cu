@@ -444,11 +444,8 @@ static int build_impl(const float* points, int64_t n, int32_t d, int32_t T, int3
   for (int t0 = 0; t0 < T && rc == HF_OK; t0 += TB) {
     const int tb = T - t0 < TB ? T - t0 : TB;
     cudaEvent_t k0 = tm.mark();
-    for (int j = 0; j < tb; ++j) {
-      const int t = t0 + j;
-      launch_prefix_keys(f->planes, f->p0t, n, d, bits, f->K2, f->L, f->pi + (size_t)t * d, f->rbits + (size_t)t * W32,
-                         f->pk + (size_t)j * f->K2 * n, s);
-    }
+    launch_prefix_keys(f->planes, f->p0t, n, d, bits, f->K2, f->L, tb, f->pi + (size_t)t0 * d,
+                       f->rbits + (size_t)t0 * W32, f->pk, s);
     cudaEvent_t k1 = tm.mark();
     rc = sort_batch(f, t0, tb, s);
     cudaEvent_t k2 = tm.mark();
@@ -476,10 +473,9 @@ static int build_impl(const float* points, int64_t n, int32_t d, int32_t T, int3
   dfree(seg64, s);
   if (rc == HF_OK) {
     tm.collect({0, 1, 2, 3});
-    // keys per tree; histogram, scan, 8K passes, prefix gather and tie kernels
-    // per batch
+    // keys, histogram, scan, 8K passes, prefix gather and tie kernels per batch
     const int nb = (T + TB - 1) / TB;
-    f->timings[6] = (float)(T + nb * (2 + 8 * K + (K > 1 ? 1 : 0) + (K < f->W ? 3 : 0)));
+    f->timings[6] = (float)(nb * (3 + 8 * K + (K > 1 ? 1 : 0) + (K < f->W ? 3 : 0)));
   }
   free_build_scratch(f, s);
   if (rc != HF_OK) {
@@ -1293,7 +1289,7 @@ int hf_debug_prefix(hf_forest* f, int32_t tree, uint64_t* out_words, void* strea
     }
     launch_plane0_slice(f->planes, f->n, f->d, p0t, s);
   }
-  launch_prefix_keys(f->planes, p0t, f->n, f->d, f->bits, f->K2, f->L, f->pi + (size_t)tree * f->d,
+  launch_prefix_keys(f->planes, p0t, f->n, f->d, f->bits, f->K2, f->L, 1, f->pi + (size_t)tree * f->d,
                      f->rbits + (size_t)tree * f->W32, kk, s);
   int rc = HF_OK;
   if (!dev) rc = map_cuda(cudaMemcpyAsync(out_words, kk, cnt * 8, cudaMemcpyDeviceToHost, s));

@@ -81,10 +81,14 @@ __global__ void plane0_slice_kernel(const uint32_t* __restrict__ plane0, int64_t
 // plus the running carry of the earlier halves gives key bit i for all 32
 // points, and the transpose (bit-reversed: the key is packed most significant
 // bit first) gives point j its 32 bits 32h .. 32h+31.
+// Tree blockIdx.y of a batch: its axes at pi + y d, its words at pk + y K n.
 template <int H>
 __global__ void prefix_sliced_kernel(const uint32_t* __restrict__ p0t, int64_t n, int d, int K,
-                                     const int32_t* __restrict__ pi, const uint32_t* __restrict__ rbits,
+                                     const int32_t* __restrict__ pi, const uint32_t* __restrict__ rbits, int W32,
                                      uint64_t* __restrict__ pk) {
+  pi += (size_t)blockIdx.y * d;
+  rbits += (size_t)blockIdx.y * W32;
+  pk += (size_t)blockIdx.y * K * n;
   constexpr int GW = 2;  // point groups per warp and round: their loads are in flight together
   const int lane = threadIdx.x & 31;
   const int64_t G = (n + 31) / 32;
@@ -159,6 +163,9 @@ __global__ void prefix_bitsliced_kernel(const uint32_t* __restrict__ planes, int
                                         int gpw, int rs, const int32_t* __restrict__ pi,
                                         const uint32_t* __restrict__ rbits, uint64_t* __restrict__ pk) {
   extern __shared__ uint32_t smk[];
+  pi += (size_t)blockIdx.y * d;  // tree blockIdx.y of the batch
+  rbits += (size_t)blockIdx.y * W32;
+  pk += (size_t)blockIdx.y * K * n;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwb = blockDim.x >> 5;
   const int rows = L * d;
   int* inv = reinterpret_cast<int*>(smk);  // inv[pi[i]] = i
@@ -281,6 +288,9 @@ __global__ void prefix_general_kernel(const uint32_t* __restrict__ planes, int64
                                       const uint32_t* __restrict__ rbits,
                                       uint64_t* __restrict__ pk) {
   extern __shared__ uint8_t smb[];
+  pi += (size_t)blockIdx.y * d;  // tree blockIdx.y of the batch
+  rbits += (size_t)blockIdx.y * W32;
+  pk += (size_t)blockIdx.y * K * n;
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
   uint8_t* Y = smb + (size_t)threadIdx.x * d;
@@ -326,7 +336,7 @@ void set_smem(const void* fn, size_t bytes) {
 }
 
 template <int L>
-void bitsliced_launch(unsigned blocks, int threads, size_t smem, const uint32_t* planes, int64_t n, int d, int W32,
+void bitsliced_launch(dim3 blocks, int threads, size_t smem, const uint32_t* planes, int64_t n, int d, int W32,
                       int K, int gpw, int rs, const int32_t* pi, const uint32_t* rbits, uint64_t* pk, cudaStream_t s) {
   set_smem((const void*)prefix_bitsliced_kernel<L>, smem);
   prefix_bitsliced_kernel<L><<<blocks, threads, smem, s>>>(planes, n, d, W32, K, gpw, rs, pi, rbits, pk);
@@ -334,14 +344,14 @@ void bitsliced_launch(unsigned blocks, int threads, size_t smem, const uint32_t*
 
 // The bit-sliced general path; false (nothing launched) when one warp's tile
 // does not fit in shared memory. Groups per warp: as few as give about 16
-// warps per SM (the kernel is latency-bound: 8 or 32 per SM measured slower),
-// up to one per lane.
-bool launch_prefix_bitsliced(const uint32_t* planes, int64_t n, int d, int W32, int K, int L, const int32_t* pi,
-                             const uint32_t* rbits, uint64_t* pk, cudaStream_t s) {
+// warps per SM over the batch's trees (the kernel is latency-bound: 8 or 32 per
+// SM measured slower), up to one per lane.
+bool launch_prefix_bitsliced(const uint32_t* planes, int64_t n, int d, int W32, int K, int L, int trees,
+                             const int32_t* pi, const uint32_t* rbits, uint64_t* pk, cudaStream_t s) {
   constexpr int64_t kWarpsWanted = 152 * 16;
   constexpr size_t kSmemCap = 200 * 1024;
   const int64_t G = (n + 31) / 32;
-  const int64_t want = (G + kWarpsWanted - 1) / kWarpsWanted;
+  const int64_t want = (G * trees + kWarpsWanted - 1) / kWarpsWanted;
   const int gpw = want < 1 ? 1 : (want > 32 ? 32 : (int)want);
   const int rs = gpw | 1;
   const size_t per_warp = (size_t)L * d * rs * sizeof(uint32_t);
@@ -351,16 +361,18 @@ bool launch_prefix_bitsliced(const uint32_t* planes, int64_t n, int d, int W32, 
   if (smem > kSmemCap) return false;
   const int64_t warps = (G + gpw - 1) / gpw;
   int64_t blocks = (warps + nwb - 1) / nwb;
-  if (blocks > 152 * 32) blocks = 152 * 32;
+  const int64_t cap = (152 * 32 + trees - 1) / trees;
+  if (blocks > cap) blocks = cap;
   const int thr = 32 * nwb;
+  const dim3 grid((unsigned)blocks, (unsigned)trees);
   switch (L) {
-    case 2: bitsliced_launch<2>((unsigned)blocks, thr, smem, planes, n, d, W32, K, gpw, rs, pi, rbits, pk, s); break;
-    case 3: bitsliced_launch<3>((unsigned)blocks, thr, smem, planes, n, d, W32, K, gpw, rs, pi, rbits, pk, s); break;
-    case 4: bitsliced_launch<4>((unsigned)blocks, thr, smem, planes, n, d, W32, K, gpw, rs, pi, rbits, pk, s); break;
-    case 5: bitsliced_launch<5>((unsigned)blocks, thr, smem, planes, n, d, W32, K, gpw, rs, pi, rbits, pk, s); break;
-    case 6: bitsliced_launch<6>((unsigned)blocks, thr, smem, planes, n, d, W32, K, gpw, rs, pi, rbits, pk, s); break;
-    case 7: bitsliced_launch<7>((unsigned)blocks, thr, smem, planes, n, d, W32, K, gpw, rs, pi, rbits, pk, s); break;
-    default: bitsliced_launch<8>((unsigned)blocks, thr, smem, planes, n, d, W32, K, gpw, rs, pi, rbits, pk, s); break;
+    case 2: bitsliced_launch<2>(grid, thr, smem, planes, n, d, W32, K, gpw, rs, pi, rbits, pk, s); break;
+    case 3: bitsliced_launch<3>(grid, thr, smem, planes, n, d, W32, K, gpw, rs, pi, rbits, pk, s); break;
+    case 4: bitsliced_launch<4>(grid, thr, smem, planes, n, d, W32, K, gpw, rs, pi, rbits, pk, s); break;
+    case 5: bitsliced_launch<5>(grid, thr, smem, planes, n, d, W32, K, gpw, rs, pi, rbits, pk, s); break;
+    case 6: bitsliced_launch<6>(grid, thr, smem, planes, n, d, W32, K, gpw, rs, pi, rbits, pk, s); break;
+    case 7: bitsliced_launch<7>(grid, thr, smem, planes, n, d, W32, K, gpw, rs, pi, rbits, pk, s); break;
+    default: bitsliced_launch<8>(grid, thr, smem, planes, n, d, W32, K, gpw, rs, pi, rbits, pk, s); break;
   }
   hf_after_launch("prefix_bitsliced_kernel", s);
   return true;
@@ -377,26 +389,28 @@ void launch_plane0_slice(const uint32_t* planes, int64_t n, int d, uint32_t* p0t
   hf_after_launch("plane0_slice_kernel", s);
 }
 
+// One launch for all trees of a batch: with one per tree, eight trees of 20,000
+// points cost 147 us of launches that fill a fraction of the chip each.
 void launch_prefix_keys(const uint32_t* planes, const uint32_t* p0t, int64_t n, int d, int bits, int K, int L,
-                        const int32_t* pi, const uint32_t* rbits, uint64_t* pk, cudaStream_t s) {
+                        int trees, const int32_t* pi, const uint32_t* rbits, uint64_t* pk, cudaStream_t s) {
   const int W32 = (d + 31) / 32;
   if (prefix_top_path(d, K, L) && p0t) {
     const int64_t G = (n + 31) / 32;
-    const unsigned blocks = hf_blocks(G * 32, 256, 152 * 16);
+    const dim3 blocks(hf_blocks(G * 32, 256, (152 * 16 + trees - 1) / trees), (unsigned)trees);
     if (K <= 2)
-      prefix_sliced_kernel<4><<<blocks, 256, 0, s>>>(p0t, n, d, K, pi, rbits, pk);
+      prefix_sliced_kernel<4><<<blocks, 256, 0, s>>>(p0t, n, d, K, pi, rbits, W32, pk);
     else if (K <= 4)
-      prefix_sliced_kernel<8><<<blocks, 256, 0, s>>>(p0t, n, d, K, pi, rbits, pk);
+      prefix_sliced_kernel<8><<<blocks, 256, 0, s>>>(p0t, n, d, K, pi, rbits, W32, pk);
     else
-      prefix_sliced_kernel<16><<<blocks, 256, 0, s>>>(p0t, n, d, K, pi, rbits, pk);
+      prefix_sliced_kernel<16><<<blocks, 256, 0, s>>>(p0t, n, d, K, pi, rbits, W32, pk);
     hf_after_launch("prefix_sliced_kernel", s);
     return;
   }
-  if (L >= 2 && L <= 8 && launch_prefix_bitsliced(planes, n, d, W32, K, L, pi, rbits, pk, s)) return;
+  if (L >= 2 && L <= 8 && launch_prefix_bitsliced(planes, n, d, W32, K, L, trees, pi, rbits, pk, s)) return;
   const int t = threads_for_bytes_per_thread(d);
   const size_t smem = (size_t)t * d;
   set_smem((const void*)prefix_general_kernel, smem);
-  prefix_general_kernel<<<hf_blocks(n, t), t, smem, s>>>(planes, n, d, W32, K, L, pi, rbits, pk); hf_after_launch("prefix_general_kernel", s);
+  prefix_general_kernel<<<dim3(hf_blocks(n, t), (unsigned)trees), t, smem, s>>>(planes, n, d, W32, K, L, pi, rbits, pk); hf_after_launch("prefix_general_kernel", s);
   (void)bits;
 }
 

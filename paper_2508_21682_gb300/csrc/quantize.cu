@@ -118,74 +118,122 @@ __device__ __forceinline__ uint64_t transpose8x8(uint64_t x) {
   return x;
 }
 
-// One warp per point. The warp first copies the point's row into its
-// shared-memory slot (16-byte loads when rows are 16-byte aligned, all issued
-// before any is used). Lane j then takes groups of 8 consecutive coordinates
-// (8g .. 8g+7, g = j, j + 32, ...): it quantizes them, packs the 8 codes
+// A warp takes pb consecutive points at a time. Lane by lane it goes through
+// their groups of 8 consecutive coordinates (4 W32 groups a point, pb times
+// that many in a row: a multiple of 32, or nearly so, for every d): it loads
+// the group (32 bytes, one group ahead), quantizes it, packs the 8 codes
 // (aligned to 8 bits) into one 64-bit word and transposes it as an 8 x 8 bit
-// matrix, so that byte 7 - l holds bit plane l of the 8 coordinates: byte g
-// of the point's plane-l row. The plane rows (W32 words each) are collected
-// in shared memory and written out contiguously.
+// matrix, so that byte 7 - l holds bit plane l of the 8 coordinates: byte g of
+// the point's plane-l row. The plane rows (W32 words each) are collected in
+// shared memory, where the pb points' rows of a plane are adjacent as they are
+// in memory, and written out contiguously. One point per warp left half of the
+// lanes without a group at d = 64 and a quarter of the rounds at d = 384.
 constexpr int QP_THREADS = 256;
+
+// Points per warp: at least four rounds of 32 groups, within 2 KB per warp.
+int quantize_points(int W32, int bits) {
+  int pb = 1;
+  while (pb < 32 && pb * 4 * W32 < 128 && bits * pb * 2 * W32 * 4 <= 2048) pb <<= 1;
+  // an odd number of half rounds: one more doubling fills it
+  if ((pb * 4 * W32) % 32 != 0 && pb < 32 && bits * pb * 2 * W32 * 4 <= 4096) pb <<= 1;
+  return pb;
+}
 
 __global__ void __launch_bounds__(QP_THREADS)
 quantize_planes_kernel(const float* __restrict__ x, int64_t n, int d, int W32, const float* __restrict__ lo0,
-                       const float* __restrict__ scale0, int bits, int vec4, const uint32_t* __restrict__ seg,
+                       const float* __restrict__ scale0, int bits, int vec4, int pb, const uint32_t* __restrict__ seg,
                        uint32_t* __restrict__ planes) {
-  extern __shared__ __align__(16) float qsm[];
+  extern __shared__ __align__(16) uint32_t qsm[];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const int rowf = 32 * W32;                       // staged floats (>= d)
-  const int wstride = (rowf + bits * W32 + 3) & ~3;  // floats per warp, keeps 16-byte alignment
-  float* row_s = qsm + (size_t)wib * wstride;
-  uint32_t* word_s = reinterpret_cast<uint32_t*>(row_s + rowf);  // [bits][W32]
-  uint8_t* byte_s = reinterpret_cast<uint8_t*>(word_s);          // [bits][4 W32]
+  uint32_t* word_s = qsm + (size_t)wib * bits * pb * W32;  // [bits][pb][W32]
+  uint8_t* byte_s = reinterpret_cast<uint8_t*>(word_s);
+  const int groups = 4 * W32;
+  const int gstep = 32 % groups, pstep = 32 / groups;  // (point, group) of a lane's next item
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int groups = 4 * W32;
-  for (int64_t i = warp; i < n; i += nwarps) {
-    const float* row = x + (size_t)i * d;
-    // segmented rows take their own set's range
-    const size_t so = seg ? (size_t)__ldg(seg + i) * d : 0;
-    const float* __restrict__ lo = lo0 + so;
-    const float* __restrict__ scale = scale0 + so;
-    if (vec4) {
-      for (int f = lane; f < (d >> 2); f += 32)
-        reinterpret_cast<float4*>(row_s)[f] = __ldg(reinterpret_cast<const float4*>(row) + f);
-    } else {
-      for (int c = lane; c < d; c += 32) row_s[c] = __ldg(row + c);
-    }
-    __syncwarp();
-    for (int g = lane; g < groups; g += 32) {
+  const int64_t blocks = (n + pb - 1) / pb;
+  for (int64_t b = warp; b < blocks; b += nwarps) {
+    const int64_t i0 = b * pb;
+    const int np = (int)(n - i0 < pb ? n - i0 : pb);
+    float v[8];
+    auto load = [&](int pt, int g) {
       const int c0 = 8 * g;
-      uint32_t w0 = 0, w1 = 0;  // codes of coordinates c0 .. c0+3 and c0+4 .. c0+7, one per byte
-      if (vec4 && c0 + 8 <= d) {
-        const float4 xa = *reinterpret_cast<const float4*>(row_s + c0);
-        const float4 xb = *reinterpret_cast<const float4*>(row_s + c0 + 4);
-        const float4 la = __ldg(reinterpret_cast<const float4*>(lo + c0));
-        const float4 lb = __ldg(reinterpret_cast<const float4*>(lo + c0 + 4));
-        const float4 sa = __ldg(reinterpret_cast<const float4*>(scale + c0));
-        const float4 sb = __ldg(reinterpret_cast<const float4*>(scale + c0 + 4));
-        w0 = quantize_one(xa.x, la.x, sa.x, bits) | (quantize_one(xa.y, la.y, sa.y, bits) << 8) |
-             (quantize_one(xa.z, la.z, sa.z, bits) << 16) | (quantize_one(xa.w, la.w, sa.w, bits) << 24);
-        w1 = quantize_one(xb.x, lb.x, sb.x, bits) | (quantize_one(xb.y, lb.y, sb.y, bits) << 8) |
-             (quantize_one(xb.z, lb.z, sb.z, bits) << 16) | (quantize_one(xb.w, lb.w, sb.w, bits) << 24);
+      const float* src = x + (size_t)(i0 + pt) * d + c0;
+      if (vec4) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const float4 q = pt < np && c0 + 4 * h < d ? __ldcs(reinterpret_cast<const float4*>(src + 4 * h))
+                                                     : make_float4(0.f, 0.f, 0.f, 0.f);
+          v[4 * h] = q.x;
+          v[4 * h + 1] = q.y;
+          v[4 * h + 2] = q.z;
+          v[4 * h + 3] = q.w;
+        }
+      } else {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = pt < np && c0 + u < d ? __ldg(src + u) : 0.f;
+      }
+    };
+    int pt = lane / groups, g = lane % groups;
+    load(pt, g);
+    while (pt < np) {
+      float q[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) q[u] = v[u];
+      const int cpt = pt, cg = g;
+      pt += pstep;
+      g += gstep;
+      if (g >= groups) {
+        g -= groups;
+        ++pt;
+      }
+      load(pt, g);
+      const int c0 = 8 * cg;
+      // segmented rows take their own set's range
+      const size_t so = seg ? (size_t)__ldg(seg + i0 + cpt) * d : 0;
+      const float* __restrict__ lo = lo0 + so + c0;
+      const float* __restrict__ scale = scale0 + so + c0;
+      float lov[8], scv[8];
+      if (vec4) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const bool in = c0 + 4 * h < d;
+          const float4 l = in ? __ldg(reinterpret_cast<const float4*>(lo + 4 * h)) : make_float4(0.f, 0.f, 0.f, 0.f);
+          const float4 c = in ? __ldg(reinterpret_cast<const float4*>(scale + 4 * h)) : make_float4(0.f, 0.f, 0.f, 0.f);
+          lov[4 * h] = l.x;
+          lov[4 * h + 1] = l.y;
+          lov[4 * h + 2] = l.z;
+          lov[4 * h + 3] = l.w;
+          scv[4 * h] = c.x;
+          scv[4 * h + 1] = c.y;
+          scv[4 * h + 2] = c.z;
+          scv[4 * h + 3] = c.w;
+        }
       } else {
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-          const int c = c0 + u;
-          const uint32_t code = c < d ? quantize_one(row_s[c], __ldg(lo + c), __ldg(scale + c), bits) : 0u;
-          if (u < 4) w0 |= code << (8 * u);
-          else w1 |= code << (8 * (u - 4));
+          lov[u] = c0 + u < d ? __ldg(lo + u) : 0.f;
+          scv[u] = c0 + u < d ? __ldg(scale + u) : 0.f;
         }
+      }
+      // coordinates past d have scale 0: code 0
+      uint32_t w0 = 0, w1 = 0;  // codes of coordinates c0 .. c0+3 and c0+4 .. c0+7, one per byte
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        w0 |= quantize_one(q[u], lov[u], scv[u], bits) << (8 * u);
+        w1 |= quantize_one(q[u + 4], lov[u + 4], scv[u + 4], bits) << (8 * u);
       }
       // align every code to 8 bits (the shift stays inside each byte)
       const uint64_t packed = ((uint64_t)w1 << 32 | w0) << (8 - bits);
       const uint64_t tr = transpose8x8(packed);
-      for (int l = 0; l < bits; ++l) byte_s[l * groups + g] = (uint8_t)(tr >> (8 * (7 - l)));
+#pragma unroll
+      for (int l = 0; l < 8; ++l)
+        if (l < bits) byte_s[(l * pb + cpt) * groups + cg] = (uint8_t)(tr >> (8 * (7 - l)));
     }
     __syncwarp();
+    const int words = np * W32;
     for (int l = 0; l < bits; ++l)
-      for (int m = lane; m < W32; m += 32) planes[((size_t)l * n + i) * W32 + m] = word_s[l * W32 + m];
+      for (int m = lane; m < words; m += 32) planes[((size_t)l * n + i0) * W32 + m] = word_s[l * pb * W32 + m];
     __syncwarp();
   }
 }
@@ -416,11 +464,12 @@ void launch_quantize_planes(const float* x, int64_t n, int d, const float* lo, c
   (void)err;
   const int W32 = (d + 31) / 32;
   const int vec4 = d % 4 == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0;
-  const size_t smem = (size_t)(QP_THREADS / 32) * ((32 * W32 + bits * W32 + 3) & ~3) * 4;
+  const int pb = quantize_points(W32, bits);
+  const size_t smem = (size_t)(QP_THREADS / 32) * bits * pb * W32 * 4;
   if (smem > 48 * 1024)
     cudaFuncSetAttribute((const void*)quantize_planes_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  quantize_planes_kernel<<<hf_blocks(n * 32, QP_THREADS, 152 * 16), QP_THREADS, smem, s>>>(x, n, d, W32, lo, scale,
-                                                                                          bits, vec4, seg, planes);
+  quantize_planes_kernel<<<hf_blocks((n + pb - 1) / pb * 32, QP_THREADS, 152 * 16), QP_THREADS, smem, s>>>(
+      x, n, d, W32, lo, scale, bits, vec4, pb, seg, planes);
   hf_after_launch("quantize_planes_kernel", s);
 }
 
