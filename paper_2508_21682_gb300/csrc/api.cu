@@ -136,6 +136,7 @@ void free_build_scratch(hf_forest* f, cudaStream_t s) {
   dfree(f->sort.vals_b, s);
   dfree(f->sort.status, s);
   dfree(f->sort.hist, s);
+  dfree(f->sort.skip, s);
   dfree(f->tie.big_runs, s);
   dfree(f->tie.counters, s);
   dfree(f->tie.fk, s);
@@ -400,6 +401,7 @@ static int build_impl(const float* points, int64_t n, int32_t d, int32_t T, int3
   chk(dalloc(&f->sort.vals_b, (size_t)TB * n, s));
   chk(dalloc(&f->sort.status, sort_status_words(n, K, TB), s));
   chk(dalloc(&f->sort.hist, (size_t)TB * K * 8 * 256, s));
+  chk(dalloc(&f->sort.skip, (size_t)TB + 1, s));
   f->tie.big_cap = n / (tie_big_min(f->W) + 1) + 1;
   chk(dalloc(&f->tie.big_runs, (size_t)T * f->tie.big_cap, s));
   chk(dalloc(&f->tie.counters, (size_t)T * 4, s));
@@ -475,7 +477,7 @@ static int build_impl(const float* points, int64_t n, int32_t d, int32_t T, int3
     tm.collect({0, 1, 2, 3});
     // keys, histogram, scan, 8K passes, prefix gather and tie kernels per batch
     const int nb = (T + TB - 1) / TB;
-    f->timings[6] = (float)(nb * (3 + 8 * K + (K > 1 ? 1 : 0) + (K < f->W ? 3 : 0)));
+    f->timings[6] = (float)(nb * (4 + 8 * K + (K <= 2 ? 3 : 0) + (K < f->W ? 3 : 0)));
   }
   free_build_scratch(f, s);
   if (rc != HF_OK) {

@@ -34,10 +34,11 @@ struct SortScratch {  // for a batch of TB trees
   uint32_t* vals_b = nullptr;  // [TB][n]
   uint32_t* status = nullptr;  // [passes]([TB][tiles + 1][256] look-back words, ticket)
   uint32_t* hist = nullptr;    // [TB][K*8][256] digit counts -> exclusive offsets
+  uint32_t* skip = nullptr;    // [TB + 1] first pass of each tree, the least of them
 };
 
 struct TieScratch {
-  uint32_t* counters = nullptr;  // per tree: [0] tied positions, [1] big runs, [2] sub-runs
+  uint32_t* counters = nullptr;  // per tree: [0] tied positions, [1] big runs, [2] sub-runs, [3] refined positions
   uint2* big_runs = nullptr;     // per tree: runs that the host settles
   int64_t big_cap = 0;           // entries per tree in big_runs
   uint64_t* fk = nullptr;        // full-key scratch of the sub-runs

@@ -98,6 +98,111 @@ __global__ void hist_scan_kernel(uint32_t* __restrict__ hist) {
   h[threadIdx.x] = s[threadIdx.x];
 }
 
+// ---------------------------------------------------------------------------
+// How many of the low digits a tree's sort can leave out. On most data a
+// prefix of 32 to 64 bits already tells nearly all points apart, and the few
+// runs that share it are cheaper to order by counting (refine_warp_kernel)
+// than by the passes over every point that the remaining digits cost. The
+// runs' sizes are estimated from a sample: C pairs of equal top bits among S
+// points mean about n + 2 C (n / S)^2 word compares in the ranking. One block
+// per tree sorts S evenly spread, jittered points' first words and prices the
+// choices: start at pass 0 (every digit of the K <= 2 words), or order by the
+// first word's top 64, 56, 48, 40 or 32 bits.
+// Prices in picoseconds (3M x 384, 4M x 64, 1.2M x 128): a pass 11 per point
+// (or its launch's latency, on small inputs), refining 24 per point and 60 per
+// point of a run that reaches past a warp's 32 positions, a compare 0.5,
+// fetching the first word again in the final order 9. A run that the sample
+// misses costs time, not order. Per sort: 3M x 384, T = 64: 33.2 -> 25.9 ms of
+// kernels; 4M x 64, T = 16, where half of the points tie at 128 bits, keeps
+// every pass; 200,001 x 384, T = 16: 3.88 -> 3.74 ms, build and narrow graph.
+// A sample of 4096 takes 70 us, one block's sort, and one of 1024 24 us, which
+// misjudges the runs of large inputs (3M x 384: 6.7 ms lost, 4M x 64: 2.5).
+// ---------------------------------------------------------------------------
+constexpr int64_t PLAN_LARGE = (int64_t)1 << 18;  // points from which the sample is 4096
+constexpr int PLAN_LEVELS = 5;
+
+template <int PLAN_S>
+__global__ void __launch_bounds__(1024) sort_plan_kernel(const uint64_t* __restrict__ pk, int64_t pk_ts, int64_t n,
+                                                         int K, int TB, uint32_t* __restrict__ skip) {
+  constexpr int E = PLAN_S / 1024;
+  __shared__ uint64_t s[PLAN_S];
+  __shared__ unsigned long long pairs[PLAN_LEVELS];
+  const uint64_t* word = pk + blockIdx.x * pk_ts;
+  const int tid = threadIdx.x;
+  const int S = n < PLAN_S ? (int)n : PLAN_S;
+  const int64_t stride = n / S;
+  // bitonic sort of element e * 1024 + tid in register e, padded with the
+  // largest word: partners less than 32 apart by shuffles
+  uint64_t v[E];
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const int j = e * 1024 + tid;
+    const uint32_t h = (uint32_t)j * 0x9E3779B1u;
+    v[e] = j < S ? __ldg(word + (int64_t)j * stride + (int64_t)((h >> 8) % (uint64_t)stride)) : ~0ull;
+  }
+  if (tid < PLAN_LEVELS) pairs[tid] = 0;
+#pragma unroll 1
+  for (int kk = 2; kk <= PLAN_S; kk <<= 1)
+#pragma unroll 1
+    for (int j = kk >> 1; j > 0; j >>= 1) {
+      if (j >= 32) {
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < E; ++e) s[e * 1024 + tid] = v[e];
+        __syncthreads();
+      }
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const int i = e * 1024 + tid;
+        const uint64_t o = j >= 32 ? s[i ^ j] : __shfl_xor_sync(0xffffffffu, v[e], j);
+        const bool small = ((i & kk) == 0) == ((i & j) == 0);  // this place keeps the smaller
+        if (small ? o < v[e] : o > v[e]) v[e] = o;
+      }
+    }
+  __syncthreads();
+#pragma unroll
+  for (int e = 0; e < E; ++e) s[e * 1024 + tid] = v[e];
+  __syncthreads();
+  for (int l = 0; l < PLAN_LEVELS; ++l) {
+    unsigned long long mine = 0;
+    for (int i = tid; i < S; i += 1024) {  // (padding sorts last)
+      const uint64_t v = s[i] >> (8 * l);
+      int lo = 0, hi = i;  // first point with these top bits
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if ((s[mid] >> (8 * l)) < v) lo = mid + 1;
+        else hi = mid;
+      }
+      mine += (unsigned long long)(i - lo);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mine += __shfl_down_sync(0xffffffffu, mine, o);
+    if ((tid & 31) == 0 && mine) atomicAdd(&pairs[l], mine);
+  }
+  __syncthreads();
+  if (tid == 0) {
+    const double dn = (double)n, grow = (dn / S) * (dn / S);
+    const double pass = fmax(11.0 * dn, 8e6 / TB);  // a launch takes 8 us at least, shared by the trees
+    double best = pass * 8 * K;
+    uint32_t s0 = 0;
+    for (int l = 0; l < PLAN_LEVELS; ++l) {
+      const double compares = 2.0 * (double)pairs[l] * grow;
+      // mates per point; a run of m crosses a 32-position boundary with
+      // probability about m / 32
+      const double mates = compares / dn, cross = mates / (mates + 32.0);
+      const double cost =
+          pass * (8 - l) + 24.0 * dn + cross * 60.0 * dn + 0.5 * cross * compares + (l ? 9.0 * dn : 0.0);
+      const uint32_t st = (uint32_t)(8 * (K - 1) + l);
+      if (st && cost < best) {
+        best = cost;
+        s0 = st;
+      }
+    }
+    skip[blockIdx.x] = s0;
+    atomicMin(&skip[TB], s0);
+  }
+}
+
 struct PassSmem {
   uint64_t keys[TILE];
   uint32_t vals[TILE];
@@ -113,7 +218,7 @@ struct PassSmem {
 struct PassArgs {
   const uint64_t* keys_in;
   int64_t keys_in_ts;
-  const uint32_t* vals_in;  // null: identity (first pass)
+  const uint32_t* vals_in;
   int64_t vals_in_ts;
   const uint64_t* gather_src;
   int64_t gather_src_ts;
@@ -129,6 +234,12 @@ struct PassArgs {
   int64_t n, ntiles;
   uint64_t spin_ns;
   int shift, TB, stall;
+  // first pass of each tree, then the least of them (null: every pass runs);
+  // a tree's first pass reads the digit's word in point order
+  const uint32_t* skip;
+  const uint64_t* first_src;
+  int64_t first_src_ts;
+  uint32_t pass;
 };
 
 // One LSD pass: bins the keys of one tile by `digit = key >> shift & 255`.
@@ -139,6 +250,7 @@ __global__ void __launch_bounds__(NT, 5) onesweep_kernel(const PassArgs a) {
   extern __shared__ __align__(16) unsigned char smraw[];
   PassSmem& S = *reinterpret_cast<PassSmem*>(smraw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (a.skip && a.pass < __ldg(a.skip + a.TB)) return;  // no tree needs this digit
 
   if (tid == 0) S.tile = atomicAdd(a.ticket, 1u);
   for (int i = tid; i < WARPS * 256; i += NT) (&S.whist[0][0])[i] = 0;
@@ -147,9 +259,14 @@ __global__ void __launch_bounds__(NT, 5) onesweep_kernel(const PassArgs a) {
   const int64_t tile = S.tile / (uint32_t)a.TB;
   const int64_t n = a.n, ntiles = a.ntiles;
   const int shift = a.shift;
-  const uint64_t* __restrict__ keys_in = GATHER ? nullptr : a.keys_in + tr * a.keys_in_ts;
-  const uint32_t* __restrict__ vals_in = a.vals_in ? a.vals_in + tr * a.vals_in_ts : nullptr;
-  const uint64_t* __restrict__ gather_src = GATHER ? a.gather_src + tr * a.gather_src_ts : nullptr;
+  const uint32_t s0 = a.skip ? __ldg(a.skip + tr) : 0u;
+  if (a.pass < s0) return;
+  // a tree's first pass reads the word in point order (vals_in null: identity)
+  const bool first = a.skip && a.pass == s0;
+  const uint32_t* __restrict__ vals_in = first ? nullptr : a.vals_in + tr * a.vals_in_ts;
+  const uint64_t* __restrict__ src = first    ? a.first_src + tr * a.first_src_ts
+                                     : GATHER ? a.gather_src + tr * a.gather_src_ts
+                                              : a.keys_in + tr * a.keys_in_ts;
   uint64_t* __restrict__ keys_out = a.keys_out + tr * a.keys_out_ts;
   uint32_t* __restrict__ vals_out = a.vals_out + tr * a.vals_out_ts;
   const uint32_t* __restrict__ goff = a.goff + tr * a.goff_ts;
@@ -167,16 +284,16 @@ __global__ void __launch_bounds__(NT, 5) onesweep_kernel(const PassArgs a) {
     if (e < n) {
       // read once per pass: streaming loads leave L2 to the pass's output
       v[j] = vals_in ? __ldcs(vals_in + e) : (uint32_t)e;
-      if (GATHER) {
+      if (GATHER && vals_in) {
         // values are point indices < n unless an earlier pass gave up its
         // look-back (error word set); never read outside the source then
         if (v[j] >= (uint64_t)n) {
           hf_raise(err, HF_ERRBIT_TIMEOUT);
           v[j] = 0;
         }
-        k[j] = __ldg(gather_src + v[j]);
+        k[j] = __ldg(src + v[j]);
       } else {
-        k[j] = __ldcs(reinterpret_cast<const unsigned long long*>(keys_in) + e);
+        k[j] = __ldcs(reinterpret_cast<const unsigned long long*>(src) + e);
       }
       dg[j] = (uint32_t)(k[j] >> shift) & 255u;
     } else {
@@ -301,12 +418,16 @@ __global__ void __launch_bounds__(NT, 5) onesweep_kernel(const PassArgs a) {
   }
 }
 
-// Sorted prefix words 1..K-1: out[w][p] = pk[w][sigma[p]]. Tree blockIdx.y of
-// the batch (one launch for all of them).
+// Sorted prefix words: out[w][p] = pk[w][sigma[p]], w = 1 .. K-1, and word 0
+// of the trees that were not sorted by all of it. Tree blockIdx.y of the batch
+// (one launch for all of them).
 __global__ void gather_prefix_kernel(const uint64_t* __restrict__ pk0, int64_t pk_ts,
                                      const uint32_t* __restrict__ sigma0, int64_t n, int K,
-                                     uint64_t* __restrict__ out0, const int* __restrict__ err) {
+                                     const uint32_t* __restrict__ skip, uint64_t* __restrict__ out0,
+                                     const int* __restrict__ err) {
   if (*(volatile const int*)err) return;  // the order is not valid: skip
+  const int w0 = __ldg(skip + blockIdx.y) > 8u * (K - 1) ? 0 : 1;
+  if (w0 >= K) return;
   const uint64_t* pk = pk0 + blockIdx.y * pk_ts;
   const uint32_t* sigma = sigma0 + blockIdx.y * n;
   uint64_t* out = out0 + (size_t)blockIdx.y * K * n;
@@ -314,7 +435,7 @@ __global__ void gather_prefix_kernel(const uint64_t* __restrict__ pk0, int64_t p
        p += (int64_t)gridDim.x * blockDim.x) {
     const uint32_t i = sigma[p];
     if (i >= (uint64_t)n) continue;
-    for (int w = 1; w < K; ++w) out[(size_t)w * n + p] = __ldg(pk + (size_t)w * n + i);
+    for (int w = w0; w < K; ++w) out[(size_t)w * n + p] = __ldg(pk + (size_t)w * n + i);
   }
 }
 
@@ -380,6 +501,7 @@ struct TieArgs {  // the first tree of the batch; strides below
   uint32_t* list;          // [tb][n] tied positions
   uint2* big;              // [tb][big_cap]
   uint32_t* counters;      // [tb][4]: listed positions, big runs, sub-runs
+  const uint32_t* skip;    // [tb] first pass of each tree's sort
   const uint32_t* planes;
   const int32_t* pi;       // [tb][d]
   const uint32_t* rbits;   // [tb][W32]
@@ -528,6 +650,135 @@ __device__ __forceinline__ int64_t run_edge(const uint64_t* __restrict__ pre, in
     else out = mid;
   }
   return in;
+}
+
+// Trees sorted by the first word's top 64 - sh bits only (sort_plan_kernel):
+// their runs of equal top bits are ordered by the rest of the K words, points
+// in index order among equals, before anything else looks at the order.
+// A warp takes 32 positions: a run that lies within them is ordered right
+// there, each lane counting its predecessors by shuffles. The positions of the
+// other runs are listed (their points and second words by position), and
+// refine_rank counts their predecessors, one thread per position; those runs
+// are as long as the plan's price allowed, so there is no cap. The first word
+// is fetched again in the final order by gather_prefix_kernel.
+__global__ void __launch_bounds__(256) refine_warp_kernel(const TieArgs a) {
+  if (*(volatile const int*)a.err) return;
+  const size_t tr = blockIdx.y;
+  const uint32_t s0 = __ldg(a.skip + tr);
+  if (!s0) return;
+  const int64_t n = a.n;
+  const int K = a.K, sh = (int)(s0 - 8u * (K - 1)) * 8, lane = threadIdx.x & 31;
+  const uint64_t* __restrict__ w0 = a.prefix + tr * K * n;
+  const uint64_t* __restrict__ pk1 = a.pk + tr * a.K2 * n + n;
+  uint32_t* __restrict__ sigma = a.sigma + tr * n;
+  for (int64_t m0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); m0 < n;
+       m0 += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t m = m0 + lane;
+    const bool in = m < n;
+    const uint64_t v0 = in ? __ldg(w0 + m) : 0;
+    // tie with the next position, the last lane's against the next warp's first
+    uint64_t nx = __shfl_down_sync(0xffffffffu, v0, 1);
+    if (lane == 31 && m + 1 < n) nx = __ldg(w0 + m + 1);
+    const uint32_t eq = __ballot_sync(0xffffffffu, in && m + 1 < n && (v0 >> sh) == (nx >> sh));
+    bool enter = false;  // the first position continues the previous warp's run
+    if (lane == 0 && m > 0) enter = (__ldg(w0 + m - 1) >> sh) == (v0 >> sh);
+    enter = __shfl_sync(0xffffffffu, enter, 0);
+    if (!eq && !enter) continue;
+    // run [lo, hi] of this lane: the ties below end at the nearest clear bit
+    const uint32_t below = ~eq & ((1u << lane) - 1u);  // lanes that do not tie with their next
+    const int lo = below ? 32 - __clz(below) : 0;
+    const uint32_t above = ~eq >> lane;
+    const int hi = above ? lane + __ffs(above) - 1 : 32;  // 32: past the warp
+    const bool cross = (lo == 0 && enter) || hi == 32;
+    const bool tied = in && (hi > lo || cross);
+    uint32_t p = 0;
+    uint64_t v1 = 0;
+    if (tied) {
+      p = sigma[m];
+      if (p >= (uint64_t)n) p = 0;  // cannot happen for a valid order
+      if (K > 1) v1 = __ldg(pk1 + p);
+    }
+    const uint32_t far = __ballot_sync(0xffffffffu, tied && cross);
+    if (far) {
+      uint32_t slot = 0;
+      if (lane == 0) slot = atomicAdd(&a.counters[tr * 4 + 3], (uint32_t)__popc(far));
+      slot = __shfl_sync(0xffffffffu, slot, 0) + __popc(far & lanemask_lt());
+      if (tied && cross) {
+        a.pt[tr * n + m] = p;
+        a.list[tr * n + slot] = (uint32_t)m;
+        if (K > 1) a.word[tr * n + m] = v1;
+      }
+    }
+    const bool near = tied && !cross;
+    const int len = near ? hi - lo + 1 : 1;
+    const int most = __reduce_max_sync(0xffffffffu, len);
+    int rank = 0, other = lane;
+    for (int it = 1; it < most; ++it) {
+      other = other == hi ? lo : other + 1;  // around the run
+      const int src = near ? other : lane;
+      const uint64_t x = __shfl_sync(0xffffffffu, v0, src), y = __shfl_sync(0xffffffffu, v1, src);
+      if (it < len && (x < v0 || (x == v0 && (y < v1 || (y == v1 && src < lane))))) ++rank;
+    }
+    if (near) sigma[m0 + lo + rank] = p;  // every member's point was read above
+  }
+}
+
+// Edge of the run of equal top bits that holds position m (dir = -1: first,
+// +1: last), by galloping probes and bisection.
+__device__ __forceinline__ int64_t bits_edge(const uint64_t* __restrict__ w0, int64_t n, int sh, int64_t m, int dir) {
+  const uint64_t v = __ldg(w0 + m) >> sh;
+  int64_t in = m, step = 1, out;
+  for (;;) {
+    out = in + dir * step;
+    if (out < 0 || out >= n) {
+      out = out < 0 ? -1 : n;
+      break;
+    }
+    if ((__ldg(w0 + out) >> sh) != v) break;
+    in = out;
+    step <<= 1;
+  }
+  while (out - in > 1 || in - out > 1) {
+    const int64_t mid = (in + out) >> 1;
+    if (mid >= 0 && mid < n && (__ldg(w0 + mid) >> sh) == v) in = mid;
+    else out = mid;
+  }
+  return in;
+}
+
+__global__ void __launch_bounds__(256) refine_rank_kernel(const TieArgs a) {
+  if (*(volatile const int*)a.err) return;
+  const size_t tr = blockIdx.y;
+  const uint32_t s0 = __ldg(a.skip + tr);
+  if (!s0) return;
+  const int64_t n = a.n;
+  const int K = a.K, sh = (int)(s0 - 8u * (K - 1)) * 8;
+  const uint64_t* __restrict__ w0 = a.prefix + tr * K * n;
+  const uint64_t* __restrict__ w1 = a.word + tr * n;
+  const uint32_t cnt = a.counters[tr * 4 + 3];
+  for (uint64_t e = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; e < cnt; e += (uint64_t)gridDim.x * blockDim.x) {
+    const int64_t m = a.list[tr * n + e];
+    const int64_t lo = bits_edge(w0, n, sh, m, -1), hi = bits_edge(w0, n, sh, m, 1);
+    const uint64_t v0 = __ldg(w0 + m), v1 = K > 1 ? w1[m] : 0;
+    uint32_t below = 0;
+    if (sh == 0) {  // the first words are equal throughout
+      for (int64_t g = lo; g <= hi; ++g) {
+        const uint64_t y = K > 1 ? w1[g] : 0;
+        below += (y < v1 || (y == v1 && g < m)) ? 1u : 0u;
+      }
+    } else {
+      for (int64_t g = lo; g <= hi; ++g) {
+        const uint64_t x = __ldg(w0 + g);
+        if (x < v0) {
+          ++below;
+        } else if (x == v0) {
+          const uint64_t y = K > 1 ? w1[g] : 0;
+          below += (y < v1 || (y == v1 && g < m)) ? 1u : 0u;
+        }
+      }
+    }
+    a.sigma[tr * n + lo + below] = a.pt[tr * n + m];
+  }
 }
 
 // One thread per listed position. The run's words are read in order (the
@@ -746,7 +997,21 @@ int sort_batch(hf_forest* f, int t0, int tb, cudaStream_t s) {
   set_attr((const void*)onesweep_kernel<false>, psm);
   set_attr((const void*)onesweep_kernel<true>, psm);
 
+  // first pass of each tree: the plan handles one or two words; the stall test
+  // needs its first pass
+  uint32_t* skip = f->sort.skip;
+  cudaMemsetAsync(skip, 0, (size_t)(tb + 1) * sizeof(uint32_t), s);
+  if (K <= 2 && !f->test_stall) {
+    cudaMemsetAsync(skip + tb, 0xff, sizeof(uint32_t), s);
+    if (n >= PLAN_LARGE)
+      sort_plan_kernel<4096><<<(unsigned)tb, 1024, 0, s>>>(f->pk, pk_ts, n, K, tb, skip);
+    else
+      sort_plan_kernel<1024><<<(unsigned)tb, 1024, 0, s>>>(f->pk, pk_ts, n, K, tb, skip);
+    hf_after_launch("sort_plan_kernel", s);
+  }
+
   PassArgs a{};
+  a.skip = skip;
   a.err = f->err;
   a.n = n;
   a.ntiles = ntiles;
@@ -760,12 +1025,9 @@ int sort_batch(hf_forest* f, int t0, int tb, cudaStream_t s) {
     for (int b = 0; b < 8; ++b, ++pass) {
       const bool gather = (w < K - 1) && b == 0;
       const bool last = pass == passes - 1;
-      if (pass == 0) {
-        a.keys_in = f->pk + (size_t)(K - 1) * n;
-        a.keys_in_ts = pk_ts;
-        a.vals_in = nullptr;
-        a.vals_in_ts = 0;
-      }
+      a.pass = (uint32_t)pass;
+      a.first_src = f->pk + (size_t)w * n;
+      a.first_src_ts = pk_ts;
       a.gather_src = gather ? f->pk + (size_t)w * n : nullptr;
       if (last) {
         a.keys_out = f->prefix + (size_t)t0 * K * n;  // word 0 of each tree's prefix
@@ -796,15 +1058,10 @@ int sort_batch(hf_forest* f, int t0, int tb, cudaStream_t s) {
   }
   // per tree blocks of the launches below: about 16 blocks per SM over all trees
   const int64_t tree_cap = (152 * 16 + tb - 1) / tb;
-  if (K > 1) {
-    gather_prefix_kernel<<<dim3(hf_blocks(n, 256, tree_cap), (unsigned)tb), 256, 0, s>>>(
-        f->pk, pk_ts, f->sigma + (size_t)t0 * n, n, K, f->prefix + (size_t)t0 * K * n, f->err);
-    hf_after_launch("gather_prefix_kernel", s);
-  }
-  // Equal prefixes, settled on the device right away. With K == W the prefix
-  // is the whole key: equal prefixes are equal keys, already in index order.
-  if (K < f->W) {
+  const dim3 grid16(hf_blocks(n, 256, tree_cap), (unsigned)tb);
+  {
     TieArgs a{};
+    a.skip = skip;
     a.prefix = f->prefix + (size_t)t0 * K * n;
     a.pk = f->pk;
     a.sigma = f->sigma + (size_t)t0 * n;
@@ -829,7 +1086,19 @@ int sort_batch(hf_forest* f, int t0, int tb, cudaStream_t s) {
     a.Lf = tie_levels(f->d, f->bits, K);
     a.tb = tb;
     a.stride = ((f->d + 3) / 4 | 1) * 4;
-    const dim3 grid(hf_blocks(n, 256, tree_cap), (unsigned)tb);
+    if (K <= 2) {
+      refine_warp_kernel<<<grid16, 256, 0, s>>>(a);
+      hf_after_launch("refine_warp_kernel", s);
+      refine_rank_kernel<<<grid16, 256, 0, s>>>(a);
+      hf_after_launch("refine_rank_kernel", s);
+    }
+    gather_prefix_kernel<<<grid16, 256, 0, s>>>(f->pk, pk_ts, f->sigma + (size_t)t0 * n, n, K, skip,
+                                               f->prefix + (size_t)t0 * K * n, f->err);
+    hf_after_launch("gather_prefix_kernel", s);
+    // Equal prefixes, settled on the device right away. With K == W the prefix
+    // is the whole key: equal prefixes are equal keys, already in index order.
+    if (K >= f->W) return cudaGetLastError() == cudaSuccess ? HF_OK : HF_ECUDA;
+    const dim3 grid = grid16;
     if (K2 > K) {
       tie_mark_kernel<0><<<grid, 256, 0, s>>>(a);
       hf_after_launch("tie_mark_kernel", s);
