@@ -167,6 +167,7 @@ void destroy(hf_forest* f, cudaStream_t s) {
   dfree(f->plan_xs, s);
   dfree(f->plan_ms, s);
   dfree(f->plan_band, s);
+  dfree(f->plan_thr, s);
   if (f->side) {
     cudaStreamSynchronize(s);  // the stream-ordered frees above run before the side stream goes
     cudaStreamDestroy(f->side);
@@ -592,11 +593,13 @@ int knn_graph_impl(hf_forest* f, int32_t k, int32_t w, const int32_t* wpt, const
   void* xs[2] = {nullptr, nullptr};
   float2* ms[2] = {nullptr, nullptr};
   float* band = nullptr;      // plain and sketch forms: pair distances of one row chunk
+  float* thr = nullptr;       // tensor forms: the first tree's bounds
   uint16_t* pw = nullptr;     // per-point windows of one tree
   int32_t* tile_w = nullptr;  // per-tile windows of one tree
   cudaError_t e = dalloc(&li, (size_t)n * kp, s);
   if (e == cudaSuccess) e = dalloc(&ldd, (size_t)n * kp, s);
   if (e == cudaSuccess && !tensor) e = dalloc(&band, window_band_bytes(n, w) / sizeof(float), s);
+  if (e == cudaSuccess && tensor) e = dalloc(&thr, (size_t)n, s);
   if (e == cudaSuccess && budget) e = dalloc(&pw, (size_t)n, s);
   if (e == cudaSuccess && budget) e = dalloc(&tile_w, (size_t)(n + 127) / 128, s);
   for (int b = 0; b < (T_use > 1 ? 2 : 1) && tensor; ++b) {
@@ -627,6 +630,7 @@ int knn_graph_impl(hf_forest* f, int32_t k, int32_t w, const int32_t* wpt, const
       dfree(ms[b], s);
     }
     dfree(band, s);
+    dfree(thr, s);
     dfree(pw, s);
     dfree(tile_w, s);
     return map_cuda(e);
@@ -657,7 +661,7 @@ int knn_graph_impl(hf_forest* f, int32_t k, int32_t w, const int32_t* wpt, const
       cudaStreamWaitEvent(s, ev[b], 0);
       cudaEvent_t m0 = tm.mark();
       rc = launch_gram_window(form, n, f->d, sig, w, tile_w, pw, kp, li, ldd, f->err, xs[b], ms[b], s, f->seg,
-                              f->seg_off);
+                              f->seg_off, t == 0 ? thr : nullptr);
       cudaEvent_t m1 = tm.mark();
       tm.span(10, m0, m1);
       cudaEventRecord(ev[2 + b], s);
@@ -718,6 +722,7 @@ int knn_graph_impl(hf_forest* f, int32_t k, int32_t w, const int32_t* wpt, const
     dfree(ms[b], s);
   }
   dfree(band, s);
+  dfree(thr, s);
   dfree(pw, s);
   dfree(tile_w, s);
   return rc;
@@ -774,6 +779,8 @@ int hf_graph_plan(hf_forest* f, int32_t k, int32_t w, int32_t threads, void* str
     dfree(f->plan_ms, s);
     e = dalloc_bytes(&f->plan_xs, (size_t)n * gram_row_bytes(f->d, form), s);
     if (e == cudaSuccess) e = dalloc(&f->plan_ms, (size_t)n, s);
+    dfree(f->plan_thr, s);
+    if (e == cudaSuccess) e = dalloc(&f->plan_thr, (size_t)n, s);
   }
   if (e == cudaSuccess && form && f->xform != form) {
     dfree(f->xb, s);
@@ -791,6 +798,7 @@ int hf_graph_plan(hf_forest* f, int32_t k, int32_t w, int32_t threads, void* str
     dfree(f->plan_ld, s);
     dfree(f->plan_xs, s);
     dfree(f->plan_ms, s);
+    dfree(f->plan_thr, s);
     dfree(f->plan_band, s);
     f->plan_band_bytes = 0;
     f->plan_kp = 0;
@@ -817,7 +825,7 @@ static int enqueue_graph(hf_forest* f, int32_t* out_idx, float* out_dist, cudaSt
     if (form) {
       launch_gather_rows(f->xb, f->xmeta, form, n, f->d, sig, f->plan_xs, f->plan_ms, s);
       rc = launch_gram_window(form, n, f->d, sig, f->plan_w, nullptr, nullptr, kp, f->plan_li, f->plan_ld, f->err,
-                              f->plan_xs, f->plan_ms, s, f->seg, f->seg_off);
+                              f->plan_xs, f->plan_ms, s, f->seg, f->seg_off, t == 0 ? f->plan_thr : nullptr);
     } else {
       rc = launch_window_graph(f->x, n, f->d, sig, f->plan_w, kp, f->plan_li, f->plan_ld, f->plan_band, s, f->seg,
                                f->seg_off, f->plan_nt);

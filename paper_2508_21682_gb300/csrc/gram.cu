@@ -294,6 +294,8 @@ struct GramArgs {
   uint32_t b_stage_bytes;
   uint32_t* lidx;
   float* ldist;
+  float* thr;              // per position: a bound on the KP-th smallest estimate, or null
+  int group;               // columns per group of the bound's pass
   int* err;
   uint64_t spin_limit;
 };
@@ -476,7 +478,15 @@ __device__ __forceinline__ uint32_t pick32(const uint32_t (&v)[32], int j) {
   return (j & 1) ? a2[1] : a2[0];
 }
 
-template <int KP, bool F8, bool PAIR>
+// THR: the first tree's extra pass. Its lists are empty, and a list that fills
+// from nothing takes an insertion for nearly every row at nearly every step (1M
+// x 384, w = 1024: 12.2M clocks a block against 3M on settled lists). This
+// pass leaves the lists alone and finds a bound for every row instead: the
+// KP-th smallest of the minima over groups of `group` columns, which at least
+// KP candidates of the row do not exceed. With it as their first screen the
+// band's rows insert about 20 candidates each. Branch-free: per chunk the
+// groups' minima go through a sorted list of KP values.
+template <int KP, bool F8, bool PAIR, bool THR>
 __global__ void __launch_bounds__(PT, 1) gram_band_kernel(GramArgs a, const __grid_constant__ CUtensorMap xmap) {
   extern __shared__ unsigned char smraw[];
   unsigned char* base = smraw + ((1024u - (smem_u32(smraw) & 1023u)) & 1023u);
@@ -705,6 +715,136 @@ __global__ void __launch_bounds__(PT, 1) gram_band_kernel(GramArgs a, const __gr
     auto wwait = [&](uint64_t* bar, uint32_t par) {
       return __all_sync(0xffffffffu, pwait(bar, par, lim, abort, a.err));
     };
+    // the row's band of a tile, columns [wlo, whi] of its range except the row
+    // itself: its window, within its set in a segmented forest (column c is
+    // position t * TP - W8 + c)
+    auto row_band = [&](const TileGeom& g, int64_t t, bool rowok, uint32_t ip, int& wlo, int& whi) {
+      int wr = g.w;
+      if (rowok && a.pw) wr = min(wr, (int)__ldg(a.pw + ip));
+      wlo = rt + g.W8 - wr;
+      whi = rowok ? rt + g.W8 + wr : -1;
+      if (rowok && a.segr) {
+        const uint32_t sg = __ldg(a.segr + ip);
+        const int64_t cbase = t * TP - g.W8;
+        const int64_t plo = __ldg(a.segoff + sg) - cbase, phi = __ldg(a.segoff + sg + 1) - 1 - cbase;
+        if (plo > wlo) wlo = (int)plo;
+        if (phi < whi) whi = (int)phi;
+      }
+    };
+    // chunk [c0, c0 + 32) of it as a bit mask
+    auto band_mask = [&](int c0, int wlo, int whi, int diag) {
+      const int lo = wlo - c0 > 0 ? wlo - c0 : 0;
+      const int hi = whi - c0 < 31 ? whi - c0 : 31;
+      uint32_t wm = 0;
+      if (lo <= hi) wm = (0xffffffffu >> (31 - hi + lo)) << lo;
+      if (diag >= c0 && diag < c0 + 32) wm &= ~(1u << (diag - c0));
+      return wm;
+    };
+    if constexpr (THR) {
+      for (int64_t t = tile0; t < ntiles && ok && !__any_sync(0xffffffffu, *abort); t += tstep) {
+        const TileGeom g = tile_geom<PAIR>(a, t);
+        if (g.J == 0) continue;
+        const int64_t p = t * TP + rt;
+        const bool rowok = p < a.n;
+        float m[KP];  // smallest group minima, ascending
+#pragma unroll
+        for (int e = 0; e < KP; ++e) m[e] = INFINITY;
+        auto ins = [&](float x) {
+#pragma unroll
+          for (int e = 0; e < KP; ++e) {
+            const float lo = fminf(m[e], x);
+            x = fmaxf(m[e], x);
+            m[e] = lo;
+          }
+        };
+        float ni = 0.f, c2 = 2.0f;
+        int wlo = 0, whi = -1;
+        for (int j = 0; j < g.J; ++j, ++u) {
+          const int sl = u % NSLOT, buf = u & 1;
+          if (!wwait(&S.mfull[sl], (u / NSLOT) & 1)) {
+            ok = false;
+            break;
+          }
+          const SlotView se = slot_view<F8>(slots, sl);
+          if (j == 0) {
+            ni = se.nrm[SLOT_COLS + r];
+            c2 = F8 ? 2.0f * se.sc[SLOT_COLS + r] : 2.0f;
+            row_band(g, t, rowok, se.id[SLOT_COLS + r], wlo, whi);
+          }
+          if (!wwait(&S.tfull[buf], (u >> 1) & 1)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const int u0 = SLOT_COLS * j;
+          const int cend = min(rq + 32 + 2 * g.W8, u0 + SLOT_COLS);
+          int c0 = max(rq, u0);
+          if (((c0 >> 5) & 1) != h) c0 += 32;
+          for (; c0 < cend; c0 += 64) {
+            uint32_t v[32];
+            tmem_ld32(tmem + (uint32_t)(buf * 256) + ((uint32_t)(32 * q) << 16) + (uint32_t)(c0 - u0), v);
+            const uint32_t wm = band_mask(c0, wlo, whi, rt + g.W8);
+            tmem_wait32(v);
+            const float* cn = se.nrm + (c0 - u0);
+            float e[32];
+#pragma unroll
+            for (int c = 0; c < 32; ++c) {
+              const float mc = F8 ? -c2 * se.sc[c0 - u0 + c] : -2.0f;
+              e[c] = fmaf(__uint_as_float(v[c]), mc, cn[c]);
+            }
+            if (__any_sync(0xffffffffu, wm != 0xffffffffu)) {
+#pragma unroll
+              for (int c = 0; c < 32; ++c)
+                if (!((wm >> c) & 1u)) e[c] = INFINITY;
+            }
+            float m4[8];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) m4[c] = fminf(fminf(e[4 * c], e[4 * c + 1]), fminf(e[4 * c + 2], e[4 * c + 3]));
+            if (a.group == 4) {
+#pragma unroll
+              for (int c = 0; c < 8; ++c) ins(m4[c]);
+            } else if (a.group == 8) {
+#pragma unroll
+              for (int c = 0; c < 4; ++c) ins(fminf(m4[2 * c], m4[2 * c + 1]));
+            } else {
+#pragma unroll
+              for (int c = 0; c < 2; ++c)
+                ins(fminf(fminf(m4[4 * c], m4[4 * c + 1]), fminf(m4[4 * c + 2], m4[4 * c + 3])));
+            }
+          }
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) {
+            if (PAIR) mbar_arrive_cluster(buf ? tempty1 : tempty0);
+            else mbar_arrive(&S.tempty[buf]);
+            mbar_arrive(&S.mempty[sl]);
+          }
+        }
+        if (!ok) break;
+        // half 1's values into half 0's
+#pragma unroll
+        for (int e0 = 0; e0 < KP; e0 += XE) {
+          if (!ok) continue;
+          if (h == 1) {
+            ok = wwait(&S.xempty[q], (xr & 1) ^ 1);
+            if (!ok) continue;
+#pragma unroll
+            for (int e = 0; e < XE; ++e) xd[e * GB + r] = m[e0 + e];
+            mbar_arrive(&S.xfull[q]);
+          } else {
+            ok = wwait(&S.xfull[q], xr & 1);
+            if (!ok) continue;
+#pragma unroll
+            for (int e = 0; e < XE; ++e) ins(xd[e * GB + r]);
+            mbar_arrive(&S.xempty[q]);
+          }
+          ++xr;
+        }
+        // the estimates' own rounding (n_i + partial) and the screen's (bound
+        // - n_i) stay below the margin
+        if (ok && h == 0 && rowok) a.thr[p] = m[KP - 1] + ni + 1e-6f * (fabsf(m[KP - 1]) + ni);
+      }
+    } else {
     for (int64_t t = tile0; t < ntiles && ok && !__any_sync(0xffffffffu, *abort); t += tstep) {
       const TileGeom g = tile_geom<PAIR>(a, t);
       if (g.J == 0) continue;
@@ -716,6 +856,7 @@ __global__ void __launch_bounds__(PT, 1) gram_band_kernel(GramArgs a, const __gr
       const bool rowok = p < a.n;
       ListK<KP> L;
       uint32_t fresh = 0;  // list entries of this tile
+      float bound = INFINITY;
       float ni = 0.f, c2 = 2.0f;
       uint32_t ip = 0xffffffffu;
       int wlo = 0, whi = -1;
@@ -731,20 +872,8 @@ __global__ void __launch_bounds__(PT, 1) gram_band_kernel(GramArgs a, const __gr
           ip = se.id[SLOT_COLS + r];
           ni = se.nrm[SLOT_COLS + r];
           c2 = F8 ? 2.0f * se.sc[SLOT_COLS + r] : 2.0f;
-          int wr = g.w;
-          if (rowok && a.pw) wr = min(wr, (int)__ldg(a.pw + ip));
-          // the row's band: columns [rt + W8 - wr, rt + W8 + wr] except rt + W8
-          wlo = rt + g.W8 - wr;
-          whi = rowok ? rt + g.W8 + wr : -1;
-          if (rowok && a.segr) {
-            // segmented forest: only the positions of the row's own set
-            // (column c is position t * TP - W8 + c)
-            const uint32_t sg = __ldg(a.segr + ip);
-            const int64_t cbase = t * TP - g.W8;
-            const int64_t plo = __ldg(a.segoff + sg) - cbase, phi = __ldg(a.segoff + sg + 1) - 1 - cbase;
-            if (plo > wlo) wlo = (int)plo;
-            if (phi < whi) whi = (int)phi;
-          }
+          row_band(g, t, rowok, ip, wlo, whi);
+          bound = rowok && a.thr ? __ldg(a.thr + p) : INFINITY;
           // both halves start from the point's list (fetched while the MMAs
           // run), so both screen against its current last entry; half 0
           // writes the merged list back
@@ -763,17 +892,13 @@ __global__ void __launch_bounds__(PT, 1) gram_band_kernel(GramArgs a, const __gr
         const int diag = rt + g.W8;
         // screens and merges chunk [c0, c0 + 32), whose products are in v
         auto process = [&](uint32_t(&v)[32], int c0) {
-          const int lo = wlo - c0 > 0 ? wlo - c0 : 0;
-          const int hi = whi - c0 < 31 ? whi - c0 : 31;
-          uint32_t wm = 0;
-          if (lo <= hi) wm = (0xffffffffu >> (31 - hi + lo)) << lo;
-          if (diag >= c0 && diag < c0 + 32) wm &= ~(1u << (diag - c0));
+          const uint32_t wm = band_mask(c0, wlo, whi, diag);
           // screen: column c passes when its estimate d2 = ni + (n_c - 2 c2' dot)
-          // is at most the list's current last entry (ties pass; the offer
-          // decides); with ti = last - ni (finite even for an unfilled list),
+          // is at most the list's current last entry, or the row's bound where
+          // that is lower (ties pass; the offer decides); with ti = last - ni (finite even for an unfilled list),
           // the sign bit of ti - (n_c - ...) marks a miss, and the misses of
           // the 32 columns are gathered by funnel shifts
-          const float ti = fminf(L.d[KP - 1], 3.0e38f) - ni;
+          const float ti = fminf(fminf(L.d[KP - 1], bound), 3.0e38f) - ni;
           const float* cn = se.nrm + (c0 - u0);
           uint32_t miss = 0;
 #pragma unroll
@@ -874,6 +999,7 @@ __global__ void __launch_bounds__(PT, 1) gram_band_kernel(GramArgs a, const __gr
         }
       }
       if (ok && (h == 0 || solo) && rowok) L.store(a.ldist + (size_t)ip * KP, a.lidx + (size_t)ip * KP);
+    }
     }
   }
   // teardown: the last commit completes before tensor memory is freed
@@ -1112,9 +1238,9 @@ int make_row_map(CUtensorMap* map, const void* xs, int64_t n, int rowb, bool f8,
   return r == CUDA_SUCCESS ? HF_OK : HF_ECUDA;
 }
 
-template <int KP, bool F8, bool PAIR>
+template <int KP, bool F8, bool PAIR, bool THR>
 int launch_band(const GramArgs& a, const CUtensorMap& map, size_t smem, cudaStream_t s) {
-  if (cudaFuncSetAttribute((const void*)gram_band_kernel<KP, F8, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  if (cudaFuncSetAttribute((const void*)gram_band_kernel<KP, F8, PAIR, THR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)smem) != cudaSuccess)
     return HF_ECUDA;
   int sms = 152;
@@ -1134,9 +1260,21 @@ int launch_band(const GramArgs& a, const CUtensorMap& map, size_t smem, cudaStre
   at.val.clusterDim.y = at.val.clusterDim.z = 1;
   cfg.attrs = &at;
   cfg.numAttrs = PAIR ? 1 : 0;
-  cudaLaunchKernelEx(&cfg, gram_band_kernel<KP, F8, PAIR>, a, map);  // an error is the call's final check's to find
+  cudaLaunchKernelEx(&cfg, gram_band_kernel<KP, F8, PAIR, THR>, a, map);  // an error is the call's final check's to find
   hf_after_launch(F8 ? "gram_band_kernel<fp8>" : "gram_band_kernel<bf16>", s);
   return HF_OK;
+}
+
+// The band of one tree, after the bounds' pass when `bounds` is set.
+template <int KP, bool F8, bool PAIR>
+int launch_tree(GramArgs a, bool bounds, const CUtensorMap& map, size_t smem, cudaStream_t s) {
+  if (bounds) {
+    const int rc = launch_band<KP, F8, PAIR, true>(a, map, smem, s);
+    if (rc != HF_OK) return rc;
+  } else {
+    a.thr = nullptr;
+  }
+  return launch_band<KP, F8, PAIR, false>(a, map, smem, s);
 }
 
 // One CTA or two per tile. Two stage half of the B rows each (the operand
@@ -1186,7 +1324,7 @@ void launch_gather_rows(const void* xq, const float2* meta, int form, int64_t n,
 
 int launch_gram_window(int form, int64_t n, int d, const uint32_t* sigma, int w, const int32_t* tile_w,
                        const uint16_t* pw, int kp, uint32_t* li, float* ld, int* err, const void* xs, const float2* ms,
-                       cudaStream_t s, const uint32_t* segr, const int64_t* segoff) {
+                       cudaStream_t s, const uint32_t* segr, const int64_t* segoff, float* thr) {
   const bool f8 = form == 2;
   const GramPlan p = choose_plan(d, w, f8);
   if (!p.ok) return HF_EINVAL;
@@ -1217,15 +1355,22 @@ int launch_gram_window(int form, int64_t n, int d, const uint32_t* sigma, int w,
   a.ldist = ld;
   a.err = err;
   a.spin_limit = 2000000000ull;  // 2 s per wait (globaltimer nanoseconds)
+  // Bounds for a first tree: groups small enough for 4 KP of them in the
+  // window, of 4 columns at least; not worth a pass below 2 KP groups, nor
+  // where a tile is one unit.
+  a.thr = thr;
+  a.group = 16;
+  while (a.group > 4 && 2 * w < 4 * kp * a.group) a.group >>= 1;
+  const bool bounds = thr && !p.solo && 2 * w >= 2 * kp * a.group;
   switch (kp * 4 + (f8 ? 2 : 0) + (p.pair ? 1 : 0)) {
-    case 64: return launch_band<16, false, false>(a, map, p.smem, s);
-    case 65: return launch_band<16, false, true>(a, map, p.smem, s);
-    case 66: return launch_band<16, true, false>(a, map, p.smem, s);
-    case 67: return launch_band<16, true, true>(a, map, p.smem, s);
-    case 128: return launch_band<32, false, false>(a, map, p.smem, s);
-    case 129: return launch_band<32, false, true>(a, map, p.smem, s);
-    case 130: return launch_band<32, true, false>(a, map, p.smem, s);
-    case 131: return launch_band<32, true, true>(a, map, p.smem, s);
+    case 64: return launch_tree<16, false, false>(a, bounds, map, p.smem, s);
+    case 65: return launch_tree<16, false, true>(a, bounds, map, p.smem, s);
+    case 66: return launch_tree<16, true, false>(a, bounds, map, p.smem, s);
+    case 67: return launch_tree<16, true, true>(a, bounds, map, p.smem, s);
+    case 128: return launch_tree<32, false, false>(a, bounds, map, p.smem, s);
+    case 129: return launch_tree<32, false, true>(a, bounds, map, p.smem, s);
+    case 130: return launch_tree<32, true, false>(a, bounds, map, p.smem, s);
+    case 131: return launch_tree<32, true, true>(a, bounds, map, p.smem, s);
     default: return HF_EINVAL;
   }
 }

@@ -102,6 +102,7 @@ struct hf_forest {
   float* plan_ld = nullptr;
   void* plan_xs = nullptr;     // tensor forms: operand rows in tree order
   float2* plan_ms = nullptr;
+  float* plan_thr = nullptr;   // tensor forms: the first tree's bounds
   float* plan_band = nullptr;  // plain form: pair distances of one row chunk
   size_t plan_band_bytes = 0;
   int plan_k = 0, plan_w = 0, plan_kp = 0, plan_nt = 0, plan_form = 0;
@@ -179,13 +180,14 @@ void launch_prepare_operands(const float* x, int64_t n, int d, int form, void* x
 // xs[p] = xq[sigma[p]] (n x gram_row_bytes), ms[p] = meta[sigma[p]]
 void launch_gather_rows(const void* xq, const float2* meta, int form, int64_t n, int d, const uint32_t* sigma,
                         void* xs, float2* ms, cudaStream_t s);
-// one tree from its gathered rows; tile_w (per tile of 128 positions, this
+// one tree from its gathered rows; thr (n floats of scratch) while the lists
+// are empty: a pass of its own finds a bound per row first; tile_w (per tile of 128 positions, this
 // tree's window; 0 skips the tile) and pw (per point window) may be null,
 // then every point uses w
 int launch_gram_window(int form, int64_t n, int d, const uint32_t* sigma, int w, const int32_t* tile_w,
                        const uint16_t* pw, int kp, uint32_t* li, float* ld, int* err, const void* xs, const float2* ms,
-                       cudaStream_t s,
-                       const uint32_t* segr = nullptr, const int64_t* segoff = nullptr);
+                       cudaStream_t s, const uint32_t* segr = nullptr, const int64_t* segoff = nullptr,
+                       float* thr = nullptr);
 // exact float32 re-rank of the first kc slots of each KP-slot list
 int launch_rerank(const float* x, int64_t n, int d, const uint32_t* order, int kp, int kc, uint32_t* li, float* ld,
                   cudaStream_t s);
