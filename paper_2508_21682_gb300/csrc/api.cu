@@ -160,6 +160,8 @@ void destroy(hf_forest* f, cudaStream_t s) {
   dfree(f->sketch_r, s);
   dfree(f->xm, s);
   dfree(f->posm, s);
+  dfree(f->x16, s);
+  dfree(f->r16, s);
   dfree(f->seg_off, s);
   dfree(f->seg, s);
   dfree(f->plan_li, s);
@@ -1192,6 +1194,38 @@ static int sketch_search(hf_forest* f, const float* q, const uint8_t* qc, int64_
   return rc;
 }
 
+// Whether this search screens against the half-width copy of the points
+// (search.cu), which the first search that reads enough rows makes: copying
+// costs 1.5 reads of the matrix and saves half of every row scored, so four
+// rows scored per point pay for it within the same call. Without room for the
+// copy, or with rows that are not 16-byte aligned, the search reads the float32
+// rows as before. 10,000 queries, 3M x 384, T = 64, w = 50: 21 rows per point.
+static bool search_uses16(hf_forest* f, const float* q, int64_t nq, int w, cudaStream_t s) {
+  if (f->d % 4 || (reinterpret_cast<uintptr_t>(f->x) & 15) || (reinterpret_cast<uintptr_t>(q) & 15)) return false;
+  // below 64 coordinates a row is two sectors or fewer, which halves save little of
+  const double rows = (double)nq * 2.0 * w * f->T;
+  if (f->d < 64 || rows < 4.0 * (double)f->n || nq < 1024) return false;
+  std::lock_guard<std::mutex> lock(f->x16_mu);
+  if (f->x16) return true;
+  void* x16 = nullptr;
+  float* r16 = nullptr;
+  cudaError_t e = dalloc_bytes(&x16, (size_t)f->n * ((f->d + 63) / 64 * 64) * 2, s);
+  if (e == cudaSuccess) e = dalloc(&r16, (size_t)f->n, s);
+  if (e == cudaSuccess) {
+    launch_prepare16(f->x, f->n, f->d, x16, r16, s);
+    e = cudaStreamSynchronize(s);  // complete on every stream from here on
+  }
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    dfree(x16, s);
+    dfree(r16, s);
+    return false;
+  }
+  f->r16 = r16;
+  f->x16 = x16;
+  return true;
+}
+
 int hf_search(hf_forest* f, const float* queries, int64_t nq, int32_t k, int32_t w, int32_t* out_idx,
               float* out_dist, void* stream) {
   if (!f || nq < 0 || k < 1 || k > HF_MAX_K || w < 1) return HF_EINVAL;
@@ -1228,7 +1262,8 @@ int hf_search(hf_forest* f, const float* queries, int64_t nq, int32_t k, int32_t
     if (rc == HF_OK && f->mode == 3)
       rc = sketch_search(f, qsrc, qc, nq, k, w, li, ldd, s);
     else if (rc == HF_OK)
-      rc = launch_search(f, qsrc, qc, nq, k, w, li, ldd, nullptr, -1, s, part_i, part_d);
+      rc = launch_search(f, qsrc, qc, nq, k, w, li, ldd, nullptr, -1, s, part_i, part_d,
+                         search_uses16(f, qsrc, nq, w, s));
     cudaEvent_t a1 = tm.mark();
     tm.span(5, a0, a1);
     if (rc == HF_OK && !dev_i) rc = map_cuda(cudaMemcpyAsync(out_idx, li, cnt * 4, cudaMemcpyDeviceToHost, s));

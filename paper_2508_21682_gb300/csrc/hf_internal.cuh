@@ -6,6 +6,7 @@
 #include <vector>
 #include <stdint.h>
 
+#include <mutex>
 #include <string>
 
 #include "../../include/hf.h"
@@ -74,6 +75,12 @@ struct hf_forest {
   uint64_t* sketch = nullptr;
   int sketch_bits = 0;
   void* sketch_r = nullptr;   // BF16 projection (bits x dp) for query sketches
+  // search: half-width copy of the points and each one's distance from it,
+  // made by the first search large enough, under the lock, and complete before
+  // it is published
+  std::mutex x16_mu;
+  void* x16 = nullptr;
+  float* r16 = nullptr;
   float* xm = nullptr;        // master-ordered points (n x d), built on demand
   uint32_t* posm = nullptr;   // inverse of the master order
 
@@ -212,7 +219,9 @@ void launch_f32_to_bf16(const float* x, int64_t rows, int cols, int ld, void* ou
 // search.cu
 int launch_search(const hf_forest* f, const float* q, const uint8_t* qcodes, int64_t nq, int k,
                   int w, uint32_t* out_idx, float* out_dist, int64_t* out_pos, int only_tree,
-                  cudaStream_t s, uint32_t* part_idx = nullptr, float* part_dist = nullptr);
+                  cudaStream_t s, uint32_t* part_idx = nullptr, float* part_dist = nullptr, bool use16 = false);
+// the search's half-width copy of the points: x16 n x 64-padded d BF16, r16 n
+void launch_prepare16(const float* x, int64_t n, int d, void* x16, float* r16, cudaStream_t s);
 // warps that share one query of a batch (1: no split); a split search keeps a
 // list of k per part in part_idx / part_dist (nq x parts x k)
 int64_t search_parts(const hf_forest* f, int64_t nq, int w);

@@ -24,6 +24,15 @@
 //    (query, point) pair gets the same value in every tree.
 //  * Merge: the 32 scored candidates are sorted across the warp and inserted
 //    in ascending order until the first one that cannot enter.
+//  * Large batches read a half-width copy of the points first (B16 below):
+//    the distance to a point's BF16 copy, less the copy's distance from the
+//    point, bounds the point's distance from below, and only candidates whose
+//    bound does not exceed the list's last entry are scored, from the float32
+//    rows and in the arithmetic above. The lists are the same. 10,000 queries,
+//    3M x 384, T = 64, w = 50 (98 GB of float32 rows): 18.2 -> 12.4 ms, 13.5
+//    with the copy's making; bound by the screen's instructions (about 12 per
+//    row and four coordinates), no longer by HBM.
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -95,6 +104,11 @@ struct SearchArgs {
   int pos_all;  // positions of every tree into out_pos[t * nq + query], no lists
   int vec4;  // d % 4 == 0 and both matrices 16-byte aligned
   int top;   // the K prefix words lie in the top bit level (d >= 64K)
+  // half-width screen, or null: the points in BF16 (row pitch dp) and an upper
+  // bound of each one's distance from its copy
+  const __nv_bfloat16* x16;
+  const float* r16;
+  int dp;
   // parts of a query: warp `part` takes trees tp, tp + tsplit, ... and, in
   // each window, the 32-candidate chunks cp, cp + csplit, ... (part = tp *
   // csplit + cp). One part: out_idx / out_dist hold the result. More: they
@@ -221,6 +235,12 @@ struct WarpList {
     d = __shfl_sync(FULL, ds, l);
     i = __shfl_sync(FULL, is, l);
   }
+  __device__ __forceinline__ bool holds(uint32_t ci, int k, int lane) const {
+    bool dup = false;
+#pragma unroll
+    for (int s = 0; s < S; ++s) dup |= 32 * s + lane < k && iv[s] == ci;
+    return __any_sync(FULL, dup);
+  }
   // Inserts (cd, ci) unless ci is already listed; entries at or beyond k are
   // scratch.
   __device__ __forceinline__ void insert(float cd, uint32_t ci, int k, int lane) {
@@ -263,7 +283,56 @@ struct WarpList {
   }
 };
 
-template <int S>
+__device__ __forceinline__ float bf16_lo(uint32_t u) { return __uint_as_float(u << 16); }
+__device__ __forceinline__ float bf16_hi(uint32_t u) { return __uint_as_float(u & 0xffff0000u); }
+
+// acc + (q - (lo, hi))^2 on a pair of floats.
+__device__ __forceinline__ uint64_t sq_diff2(uint64_t q, float lo, float hi, uint64_t acc) {
+  uint64_t r;
+  asm("{\n .reg .b64 v, e;\n mov.b64 v, {%2, %3};\n sub.rn.f32x2 e, %1, v;\n fma.rn.f32x2 %0, e, e, %4;\n}"
+      : "=l"(r)
+      : "l"(q), "f"(lo), "f"(hi), "l"(acc));
+  return r;
+}
+__device__ __forceinline__ float pair_sum(uint64_t v) {
+  return __uint_as_float((uint32_t)v) + __uint_as_float((uint32_t)(v >> 32));
+}
+
+// BF16 copy of the points (row pitch dp, a multiple of 64, zero padded) and per
+// point an upper bound of |x - copy| (1e-5 above the float32 sum's value; inf
+// where a coordinate rounds to inf). One warp per point; d % 4 == 0, rows
+// 16-byte aligned.
+__global__ void prepare16_kernel(const float* __restrict__ x, int64_t n, int d, int dp, __nv_bfloat16* __restrict__ x16,
+                                 float* __restrict__ r16) {
+  const int lane = threadIdx.x & 31;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += nw) {
+    float s = 0.f;
+    for (int c = 4 * lane; c < dp; c += 128) {
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (c < d) v = __ldcs(reinterpret_cast<const float4*>(x + i * d + c));
+      const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
+      uint2 o;
+      o.x = *reinterpret_cast<const uint32_t*>(&a);
+      o.y = *reinterpret_cast<const uint32_t*>(&b);
+      *reinterpret_cast<uint2*>(x16 + i * dp + c) = o;
+      float e = v.x - bf16_lo(o.x);
+      s = fmaf(e, e, s);
+      e = v.y - bf16_hi(o.x);
+      s = fmaf(e, e, s);
+      e = v.z - bf16_lo(o.y);
+      s = fmaf(e, e, s);
+      e = v.w - bf16_hi(o.y);
+      s = fmaf(e, e, s);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(FULL, s, o);
+    // squares below the float32 range vanish from the sum: 2^-74 sqrt(d) covers them
+    if (lane == 0) r16[i] = sqrtf(s) * 1.00001f + 1e-20f;
+  }
+}
+
+template <int S, bool B16>
 __global__ void __launch_bounds__(SWARPS * 32) search_kernel(SearchArgs a) {
   extern __shared__ __align__(16) unsigned char smraw[];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -332,6 +401,79 @@ __global__ void __launch_bounds__(SWARPS * 32) search_kernel(SearchArgs a) {
       const int64_t c = cb + lane;
       uint32_t pid = c < c1 ? __ldg(sig + c) : 0xffffffffu;
       float dist;
+      if (B16) {
+        cpid[lane] = pid;
+        const float res = pid != 0xffffffffu ? __ldg(a.r16 + pid) : 0.f;
+        __syncwarp();
+        const int cnt = (int)(c1 - cb < 32 ? c1 - cb : 32);
+        float part[32];
+        // 16 rows at a time (none for an empty half): their loads are issued
+        // before any is used (an empty slot reads row 0; its result is
+        // discarded), two coordinates to an instruction (f32x2), the even and
+        // the odd ones' sums apart until the end
+#pragma unroll
+        for (int u0 = 0; u0 < 32; u0 += 16) {
+          uint64_t acc[16];
+#pragma unroll
+          for (int u = 0; u < 16; ++u) acc[u] = 0;
+          if (u0 < cnt) {
+            for (int m = 4 * lane; m < a.d; m += 128) {
+              const ulonglong2 qa = __ldg(reinterpret_cast<const ulonglong2*>(qv + m));
+              uint2 xb[16];
+#pragma unroll
+              for (int u = 0; u < 16; ++u) {
+                const uint32_t p = cpid[u0 + u];
+                xb[u] = __ldg(reinterpret_cast<const uint2*>(a.x16 + (size_t)(p != 0xffffffffu ? p : 0u) * a.dp + m));
+              }
+#pragma unroll
+              for (int u = 0; u < 16; ++u) {
+                acc[u] = sq_diff2(qa.x, bf16_lo(xb[u].x), bf16_hi(xb[u].x), acc[u]);
+                acc[u] = sq_diff2(qa.y, bf16_lo(xb[u].y), bf16_hi(xb[u].y), acc[u]);
+              }
+            }
+          }
+#pragma unroll
+          for (int u = 0; u < 16; ++u) part[u0 + u] = pair_sum(acc[u]);
+        }
+        const float near = warp_transpose_sum(part, lane);
+        __syncwarp();
+        // |q - x| >= |q - copy| - |x - copy|; the sums are within 1e-5 of
+        // their values up to d = 4096, also the exact one. A sum that
+        // overflowed, or whose squares leave the float32 range, says nothing.
+        const float gap = sqrtf(near) * 0.99999f - res;
+        const float bound = gap > 1e-12f && near < 1e38f ? gap * gap * 0.99998f : 0.f;
+        float kd;
+        uint32_t ki;
+        list.last(a.k, kd, ki);
+        uint32_t todo = __ballot_sync(FULL, pid != 0xffffffffu && !(bound > kd));
+        while (todo) {
+          const int src = __ffs(todo) - 1;
+          todo &= todo - 1;
+          const uint32_t ci = __shfl_sync(FULL, pid, src);
+          if (__shfl_sync(FULL, bound, src) > kd || list.holds(ci, a.k, lane)) continue;
+          float cd = 0.f;
+          for (int m = 4 * lane; m < a.d; m += 128) {
+            const float4 qa = __ldg(reinterpret_cast<const float4*>(qv + m));
+            const float4 xv = __ldg(reinterpret_cast<const float4*>(a.x + (size_t)ci * a.d + m));
+            float e = qa.x - xv.x;
+            cd = fmaf(e, e, cd);
+            e = qa.y - xv.y;
+            cd = fmaf(e, e, cd);
+            e = qa.z - xv.z;
+            cd = fmaf(e, e, cd);
+            e = qa.w - xv.w;
+            cd = fmaf(e, e, cd);
+          }
+          // the lanes' partials in warp_transpose_sum's tree
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) cd += __shfl_xor_sync(FULL, cd, o);
+          if (lessp(cd, ci, kd, ki)) {
+            list.insert(cd, ci, a.k, lane);
+            list.last(a.k, kd, ki);
+          }
+        }
+        continue;
+      }
       if (a.vec4) {
         cpid[lane] = pid;
         __syncwarp();
@@ -458,13 +600,12 @@ merge_parts_kernel(const uint32_t* __restrict__ pidx, const float* __restrict__ 
   }
 }
 
-template <int S>
+template <int S, bool B16>
 int launch_s(const SearchArgs& a, size_t smem, cudaStream_t s) {
-  if (smem > 48 * 1024 &&
-      cudaFuncSetAttribute((const void*)search_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-          cudaSuccess)
+  if (smem > 48 * 1024 && cudaFuncSetAttribute((const void*)search_kernel<S, B16>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return HF_ECUDA;
-  search_kernel<S><<<hf_blocks(a.nq * a.tsplit * a.csplit, SWARPS), SWARPS * 32, smem, s>>>(a);
+  search_kernel<S, B16><<<hf_blocks(a.nq * a.tsplit * a.csplit, SWARPS), SWARPS * 32, smem, s>>>(a);
   hf_after_launch("search_kernel", s);
   return HF_OK;
 }
@@ -497,6 +638,12 @@ void search_split(int64_t nq, int T, int w, int* tsplit, int* csplit) {
 
 }  // namespace
 
+void launch_prepare16(const float* x, int64_t n, int d, void* x16, float* r16, cudaStream_t s) {
+  prepare16_kernel<<<hf_blocks(n * 32, 256, 152 * 16), 256, 0, s>>>(x, n, d, (d + 63) / 64 * 64,
+                                                                   static_cast<__nv_bfloat16*>(x16), r16);
+  hf_after_launch("prepare16_kernel", s);
+}
+
 int64_t search_parts(const hf_forest* f, int64_t nq, int w) {
   int ts, cs;
   search_split(nq, f->T, w, &ts, &cs);
@@ -505,7 +652,7 @@ int64_t search_parts(const hf_forest* f, int64_t nq, int w) {
 
 int launch_search(const hf_forest* f, const float* q, const uint8_t* qcodes, int64_t nq, int k, int w,
                   uint32_t* out_idx, float* out_dist, int64_t* out_pos, int only_tree, cudaStream_t s,
-                  uint32_t* part_idx, float* part_dist) {
+                  uint32_t* part_idx, float* part_dist, bool use16) {
   if (k < 1 || k > 64) return HF_EINVAL;
   SearchArgs a;
   a.x = f->x;
@@ -550,7 +697,12 @@ int launch_search(const hf_forest* f, const float* q, const uint8_t* qcodes, int
     a.out_dist = part_dist;
   }
   const size_t smem = search_per_warp(f->K, f->d) * SWARPS;
-  const int rc = k <= 32 ? launch_s<1>(a, smem, s) : launch_s<2>(a, smem, s);
+  const bool b16 = a.vec4 && f->x16 && use16 && !a.pos_all && a.only_tree < 0;
+  a.x16 = b16 ? static_cast<const __nv_bfloat16*>(f->x16) : nullptr;
+  a.r16 = f->r16;
+  a.dp = (f->d + 63) / 64 * 64;
+  const int rc = b16 ? (k <= 32 ? launch_s<1, true>(a, smem, s) : launch_s<2, true>(a, smem, s))
+                     : (k <= 32 ? launch_s<1, false>(a, smem, s) : launch_s<2, false>(a, smem, s));
   if (rc != HF_OK) return rc;
   if (parts) {
     if (k <= 32) launch_merge<1>(a, out_idx, out_dist, s);
