@@ -110,50 +110,60 @@ int map_cuda(cudaError_t e) {
 }  // namespace
 
 // Synchronises, reads and clears the error word, maps to a status.
-int hf_finish(hf_forest* f, cudaStream_t s) {
+// With `words`, the error word and what lies behind it are read into
+// out[0 .. words).
+static int finish(hf_forest* f, cudaStream_t s, uint32_t* out = nullptr, size_t words = 1) {
   cudaError_t e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return map_cuda(e);
   e = cudaGetLastError();
   if (e != cudaSuccess) return map_cuda(e);
-  int word = 0;
-  if (cudaMemcpy(&word, f->err, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return HF_ECUDA;
+  uint32_t own = 0;
+  if (!out) out = &own;
+  if (cudaMemcpy(out, f->err, words * sizeof(uint32_t), cudaMemcpyDeviceToHost) != cudaSuccess) return HF_ECUDA;
+  const int word = (int)out[0];
   if (word) cudaMemset(f->err, 0, sizeof(int));
   if (word & HF_ERRBIT_NONFINITE) return HF_ENONFINITE;
   if (word & HF_ERRBIT_TIMEOUT) return HF_ETIMEOUT;
   return HF_OK;
 }
 
+int hf_finish(hf_forest* f, cudaStream_t s) { return finish(f, s); }
+
 namespace {
 
-int finish(hf_forest* f, cudaStream_t s) { return hf_finish(f, s); }
-
 void free_build_scratch(hf_forest* f, cudaStream_t s) {
-  dfree(f->pk, s);
-  dfree(f->p0t, s);
-  dfree(f->sort.keys_a, s);
-  dfree(f->sort.keys_b, s);
-  dfree(f->sort.vals_a, s);
-  dfree(f->sort.vals_b, s);
-  dfree(f->sort.status, s);
-  dfree(f->sort.hist, s);
-  dfree(f->sort.skip, s);
-  dfree(f->tie.big_runs, s);
-  dfree(f->tie.counters, s);
-  dfree(f->tie.fk, s);
+  dfree(f->scratch, s);
+  f->pk = nullptr;
+  f->p0t = nullptr;
+  f->sort = SortScratch{};
+  f->tie = TieScratch{};
 }
+
+// Several arrays of one lifetime in one allocation, each 256-byte aligned: a
+// small build spends more on its two dozen trips to the allocator and back than
+// on some of its kernels.
+struct Arena {
+  std::vector<std::pair<void**, size_t>> parts;  // where the pointer goes, offset
+  size_t bytes = 0;
+  template <typename T>
+  void add(T** p, size_t count) {
+    *p = nullptr;
+    parts.push_back({reinterpret_cast<void**>(p), bytes});
+    bytes += (count * sizeof(T) + 255) / 256 * 256;
+  }
+  cudaError_t take(uint8_t** block, cudaStream_t s) {
+    const cudaError_t e = dalloc(block, bytes, s);
+    if (e == cudaSuccess)
+      for (auto& p : parts) *p.first = *block + p.second;
+    return e;
+  }
+};
 
 void destroy(hf_forest* f, cudaStream_t s) {
   if (!f) return;
   free_build_scratch(f, s);
   dfree(f->x_owned, s);
-  dfree(f->lo, s);
-  dfree(f->scale, s);
-  dfree(f->planes, s);
-  dfree(f->pi, s);
-  dfree(f->rbits, s);
-  dfree(f->prefix, s);
-  dfree(f->sigma, s);
-  dfree(f->err, s);
+  dfree(f->block, s);
   dfree(f->xb, s);
   dfree(f->xmeta, s);
   dfree(f->sketch, s);
@@ -162,8 +172,6 @@ void destroy(hf_forest* f, cudaStream_t s) {
   dfree(f->posm, s);
   dfree(f->x16, s);
   dfree(f->r16, s);
-  dfree(f->seg_off, s);
-  dfree(f->seg, s);
   dfree(f->plan_li, s);
   dfree(f->plan_ld, s);
   dfree(f->plan_xs, s);
@@ -374,60 +382,66 @@ static int build_impl(const float* points, int64_t n, int32_t d, int32_t T, int3
     const double per_tree = (double)n * (8.0 * f->K2 + 24.0) + (double)(ntiles + 1) * 256 * 4 * 8 * K;
     size_t fr = 0, tot = 0;
     double budget = 16.0 * (1ull << 30);
-    if (cudaMemGetInfo(&fr, &tot) == cudaSuccess && 0.5 * (double)fr < budget) budget = 0.5 * (double)fr;
-    else cudaGetLastError();
+    // (a batch of 64 MB at most does not ask for the free memory, a slow call)
+    if (per_tree * T > (double)(64 << 20)) {
+      if (cudaMemGetInfo(&fr, &tot) == cudaSuccess && 0.5 * (double)fr < budget) budget = 0.5 * (double)fr;
+      else cudaGetLastError();
+    }
     const double tbd = budget / per_tree;
     f->TB = tbd >= T ? T : (tbd < 1.0 ? 1 : (int)tbd);
     if (f->sort_batch_max > 0 && f->TB > f->sort_batch_max) f->TB = f->sort_batch_max;
   }
   const int TB = f->TB;
-  chk(dalloc(&f->lo, (size_t)nseg * d, s));
-  chk(dalloc(&f->scale, (size_t)nseg * d, s));
+  // what the forest keeps, and the build's scratch
+  Arena keep, tmp;
+  keep.add(&f->lo, (size_t)nseg * d);
+  keep.add(&f->scale, (size_t)nseg * d);
   uint64_t* seg64 = nullptr;
   if (nseg > 1) {
-    chk(dalloc(&f->seg_off, (size_t)nseg + 1, s));
-    chk(dalloc(&f->seg, (size_t)n, s));
-    chk(dalloc(&seg64, (size_t)n, s));
+    keep.add(&f->seg_off, (size_t)nseg + 1);
+    keep.add(&f->seg, (size_t)n);
+    tmp.add(&seg64, (size_t)n);
   }
-  chk(dalloc(&f->planes, (size_t)bits * n * W32, s));
-  chk(dalloc(&f->pi, (size_t)T * d, s));
-  chk(dalloc(&f->rbits, (size_t)T * W32, s));
-  chk(dalloc(&f->prefix, (size_t)T * K * n, s));
-  chk(dalloc(&f->sigma, (size_t)T * n, s));
-  chk(dalloc(&f->err, 1, s));
-  chk(dalloc(&f->pk, (size_t)TB * f->K2 * n, s));
+  keep.add(&f->planes, (size_t)bits * n * W32);
+  keep.add(&f->pi, (size_t)T * (d + W32));  // the reflection masks behind the axes: one upload
+  keep.add(&f->prefix, (size_t)T * K * n);
+  keep.add(&f->sigma, (size_t)T * n);
+  keep.add(&f->err, 4 + (size_t)T * 4);  // the tie counters behind the error word: one read
+  tmp.add(&f->pk, (size_t)TB * f->K2 * n);
   const bool sliced = prefix_top_path(d, f->K2, f->L);
-  if (sliced) chk(dalloc(&f->p0t, (size_t)((n + 31) / 32) * d, s));
-  chk(dalloc(&f->sort.keys_a, (size_t)TB * n, s));
-  chk(dalloc(&f->sort.keys_b, (size_t)TB * n, s));
-  chk(dalloc(&f->sort.vals_a, (size_t)TB * n, s));
-  chk(dalloc(&f->sort.vals_b, (size_t)TB * n, s));
-  chk(dalloc(&f->sort.status, sort_status_words(n, K, TB), s));
-  chk(dalloc(&f->sort.hist, (size_t)TB * K * 8 * 256, s));
-  chk(dalloc(&f->sort.skip, (size_t)TB + 1, s));
+  if (sliced) tmp.add(&f->p0t, (size_t)((n + 31) / 32) * d);
+  tmp.add(&f->sort.keys_a, (size_t)TB * n);
+  tmp.add(&f->sort.keys_b, (size_t)TB * n);
+  tmp.add(&f->sort.vals_a, (size_t)TB * n);
+  tmp.add(&f->sort.vals_b, (size_t)TB * n);
+  // one run of words, cleared together per batch
+  const size_t skip_words = ((size_t)TB + 1 + 63) / 64 * 64, hist_words = (size_t)TB * K * 8 * 256;
+  tmp.add(&f->sort.skip, skip_words + hist_words + sort_status_words(n, K, TB));
   f->tie.big_cap = n / (tie_big_min(f->W) + 1) + 1;
-  chk(dalloc(&f->tie.big_runs, (size_t)T * f->tie.big_cap, s));
-  chk(dalloc(&f->tie.counters, (size_t)T * 4, s));
-  chk(dalloc(&f->tie.fk, K < f->W ? tie_scratch_words(f->W) : 1, s));
-  void* rscratch = nullptr;
+  tmp.add(&f->tie.big_runs, (size_t)T * f->tie.big_cap);
+  tmp.add(&f->tie.fk, K < f->W ? tie_scratch_words(f->W) : 1);
+  uint8_t* rscratch = nullptr;
   const size_t rbytes = range_scratch_bytes(n, d);
-  chk(dalloc_bytes(&rscratch, rbytes, s));
+  tmp.add(&rscratch, rbytes);
+  if (e == cudaSuccess) chk(keep.take(&f->block, s));
+  if (e == cudaSuccess) chk(tmp.take(&f->scratch, s));
   if (e != cudaSuccess) {
-    dfree(rscratch, s);
-    dfree(seg64, s);
     destroy(f, s);
     return map_cuda(e);
   }
-  cudaMemsetAsync(f->err, 0, sizeof(int), s);
+  f->rbits = reinterpret_cast<uint32_t*>(f->pi) + (size_t)T * d;
+  f->tie.counters = reinterpret_cast<uint32_t*>(f->err) + 4;
+  f->sort.hist = f->sort.skip + skip_words;
+  f->sort.status = f->sort.hist + hist_words;
+  cudaMemsetAsync(f->err, 0, (4 + (size_t)T * 4) * sizeof(uint32_t), s);
   if (nseg > 1) {
     cudaMemcpyAsync(f->seg_off, f->seg_off_h.data(), (size_t)(nseg + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s);
     launch_seg_of_row(f->seg_off, nseg, n, f->seg, seg64, s);
   }
-  cudaMemsetAsync(f->tie.counters, 0, (size_t)T * 4 * sizeof(uint32_t), s);
 
   // per-tree permutations and reflection masks (host, then one upload)
-  std::vector<int32_t> hpi((size_t)T * d);
-  std::vector<uint32_t> hr((size_t)T * W32, 0u);
+  std::vector<int32_t> hpi((size_t)T * (d + W32), 0);
+  uint32_t* hr = reinterpret_cast<uint32_t*>(hpi.data()) + (size_t)T * d;
   std::vector<uint8_t> r(d);
   for (int t = 0; t < T; ++t) {
     hf_tree_params_host(seed, t, d, hpi.data() + (size_t)t * d, r.data());
@@ -435,7 +449,6 @@ static int build_impl(const float* points, int64_t n, int32_t d, int32_t T, int3
       if (r[j]) hr[(size_t)t * W32 + (j >> 5)] |= 1u << (j & 31);
   }
   cudaMemcpyAsync(f->pi, hpi.data(), hpi.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s);
-  cudaMemcpyAsync(f->rbits, hr.data(), hr.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, s);
 
   cudaEvent_t a0 = tm.mark();
   if (nseg > 1)
@@ -457,13 +470,17 @@ static int build_impl(const float* points, int64_t n, int32_t d, int32_t T, int3
     tm.span(1, k0, k1);
     tm.span(2, k1, k2);
   }
-  if (rc == HF_OK) rc = finish(f, s);
+  // the error word and the tie counters in one read
+  std::vector<uint32_t> ctr(4 + (size_t)T * 4);
+  if (rc == HF_OK) rc = finish(f, s, ctr.data(), ctr.size());
   // runs of equal prefixes longer than the on-device cap
   if (rc == HF_OK) {
-    std::vector<uint32_t> ctr((size_t)T * 4);
-    if (cudaMemcpy(ctr.data(), f->tie.counters, ctr.size() * 4, cudaMemcpyDeviceToHost) != cudaSuccess) rc = HF_ECUDA;
+    bool more = nseg > 1;
     cudaEvent_t b0 = tm.mark();
-    for (int t = 0; t < T && rc == HF_OK; ++t) rc = tie_fixup_big(f, t, ctr[(size_t)t * 4 + 1], s);
+    for (int t = 0; t < T && rc == HF_OK; ++t) {
+      more |= ctr[4 + (size_t)t * 4 + 1] != 0;
+      rc = tie_fixup_big(f, t, ctr[4 + (size_t)t * 4 + 1], s);
+    }
     cudaEvent_t b1 = tm.mark();
     tm.span(3, b0, b1);
     if (rc == HF_OK && nseg > 1) {
@@ -472,10 +489,9 @@ static int build_impl(const float* points, int64_t n, int32_t d, int32_t T, int3
       cudaEvent_t c1 = tm.mark();
       tm.span(2, c0, c1);
     }
-    if (rc == HF_OK) rc = finish(f, s);
+    if (rc == HF_OK && more) rc = finish(f, s);
+    else if (b1) cudaEventSynchronize(b1);
   }
-  dfree(rscratch, s);
-  dfree(seg64, s);
   if (rc == HF_OK) {
     tm.collect({0, 1, 2, 3});
     // keys, histogram, scan, 8K passes, prefix gather and tie kernels per batch

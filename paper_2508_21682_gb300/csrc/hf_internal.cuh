@@ -35,7 +35,8 @@ struct SortScratch {  // for a batch of TB trees
   uint32_t* vals_b = nullptr;  // [TB][n]
   uint32_t* status = nullptr;  // [passes]([TB][tiles + 1][256] look-back words, ticket)
   uint32_t* hist = nullptr;    // [TB][K*8][256] digit counts -> exclusive offsets
-  uint32_t* skip = nullptr;    // [TB + 1] first pass of each tree, the least of them
+  uint32_t* skip = nullptr;    // [TB + 1] first pass of each tree, 255 less the least of them (0: none);
+                               // hist and status follow in the same run of words
 };
 
 struct TieScratch {
@@ -64,7 +65,9 @@ struct hf_forest {
   uint64_t* prefix = nullptr; // [T][K][n] key prefixes in sorted order
   uint32_t* sigma = nullptr;  // [T][n] position -> point
 
-  int* err = nullptr;         // device error word
+  int* err = nullptr;         // device error word (the build's tie counters lie behind it)
+  uint8_t* block = nullptr;   // the allocation that holds the arrays above and seg_off, seg
+  uint8_t* scratch = nullptr; // the build's scratch arrays (pk .. tie), freed when it ends
 
   // tensor mode: operand copy of the points (BF16 or e4m3 rows, pitch
   // gram_row_bytes) and per point (squared norm, scale), made on first use

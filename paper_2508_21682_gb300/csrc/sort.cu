@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(1024) sort_plan_kernel(const uint64_t* __restr
       }
     }
     skip[blockIdx.x] = s0;
-    atomicMin(&skip[TB], s0);
+    atomicMax(&skip[TB], 255u - s0);
   }
 }
 
@@ -234,7 +234,8 @@ struct PassArgs {
   int64_t n, ntiles;
   uint64_t spin_ns;
   int shift, TB, stall;
-  // first pass of each tree, then the least of them (null: every pass runs);
+  // first pass of each tree, then 255 less the least of them (0: every pass
+  // runs, as without the array);
   // a tree's first pass reads the digit's word in point order
   const uint32_t* skip;
   const uint64_t* first_src;
@@ -250,7 +251,10 @@ __global__ void __launch_bounds__(NT, 5) onesweep_kernel(const PassArgs a) {
   extern __shared__ __align__(16) unsigned char smraw[];
   PassSmem& S = *reinterpret_cast<PassSmem*>(smraw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (a.skip && a.pass < __ldg(a.skip + a.TB)) return;  // no tree needs this digit
+  if (a.skip) {
+    const uint32_t least = __ldg(a.skip + a.TB);
+    if (least && a.pass < 255u - least) return;  // no tree needs this digit
+  }
 
   if (tid == 0) S.tile = atomicAdd(a.ticket, 1u);
   for (int i = tid; i < WARPS * 256; i += NT) (&S.whist[0][0])[i] = 0;
@@ -983,8 +987,9 @@ int sort_batch(hf_forest* f, int t0, int tb, cudaStream_t s) {
   const int64_t hist_ts = (int64_t)K * 8 * 256;
   uint32_t* status = f->sort.status;
 
-  cudaMemsetAsync(f->sort.hist, 0, (size_t)tb * hist_ts * sizeof(uint32_t), s);
-  cudaMemsetAsync(status, 0, per_pass * passes * sizeof(uint32_t), s);
+  // the plan's words, the histograms and the look-back words are one run
+  cudaMemsetAsync(f->sort.skip, 0,
+                  (size_t)(status - f->sort.skip) * sizeof(uint32_t) + per_pass * passes * sizeof(uint32_t), s);
   const size_t hsm = (size_t)hist_ts * sizeof(uint32_t);
   set_attr((const void*)digit_hist_kernel, hsm);
   digit_hist_kernel<<<dim3(hf_blocks(n, 512, 152 * 8 / tb + 1), (unsigned)tb), 512, hsm, s>>>(f->pk, pk_ts, n, K,
@@ -1000,9 +1005,7 @@ int sort_batch(hf_forest* f, int t0, int tb, cudaStream_t s) {
   // first pass of each tree: the plan handles one or two words; the stall test
   // needs its first pass
   uint32_t* skip = f->sort.skip;
-  cudaMemsetAsync(skip, 0, (size_t)(tb + 1) * sizeof(uint32_t), s);
   if (K <= 2 && !f->test_stall) {
-    cudaMemsetAsync(skip + tb, 0xff, sizeof(uint32_t), s);
     if (n >= PLAN_LARGE)
       sort_plan_kernel<4096><<<(unsigned)tb, 1024, 0, s>>>(f->pk, pk_ts, n, K, tb, skip);
     else
