@@ -472,9 +472,9 @@ def keys_sort_hbm(a, ph):
     Algorithmic bytes per point and tree: keys read the permuted top bits of
     the point (d / 8 bytes of the bit-sliced top plane when the K-word prefix
     lies in the top bit level, d * L / 8 bytes of planes otherwise) and write
-    K 64-bit words; the sort makes 8 K passes of 8-bit digits, each reading
-    and writing one 64-bit key word and one 32-bit index per point
-    (24 bytes)."""
+    K 64-bit words; the sort is priced at 8 K passes of 8-bit digits, each
+    reading and writing one 64-bit key word and one 32-bit index per point
+    (24 bytes), also where its plan leaves low digits out."""
     K = min(2, -(-a.d * a.bits // 64))
     L = min(a.bits, -(-64 * K // a.d))
     kb = a.n * a.T * (a.d * L / 8 + 8 * K)
@@ -545,7 +545,7 @@ def window_roofline(a, launch_ms):
     flops = 3.0 * d * pairs
     achieved = flops / (launch_ms * 1e-3) / 1e12
     peak = SMS * FP32_LANES * MAX_SM_MHZ * 1e6 * 1.5 / 1e12
-    return {"bound": "alu", "kernel": "window_kernel (A5+A6, plain f32)",
+    return {"bound": "alu", "kernel": "pair_kernel + merge_kernel (A5+A6, plain f32)",
             "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
             "traffic": traffic_per_launch(WINDOW_TRAFFIC, n) if w == 32 else None, "launch_ms": launch_ms,
             "peak_note": "152 SMs x 128 FP32 lanes x 2070 MHz, 3 flops per FADD+FFMA pair"}

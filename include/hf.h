@@ -144,6 +144,12 @@ int hf_knn_graph(hf_forest* f, int32_t k, int32_t w, int32_t* out_idx, float* ou
  * query's position p is the lower bound of its full key among the data keys;
  * the candidates are the points at positions [p - w, p + w); the result is the
  * k nearest of their union by float32 squared distance.
+ * The first batch of 1024 queries or more that scores four rows per point or
+ * more makes a BF16 copy of the points (n x 64-padded d, plus n floats; at most
+ * a quarter of the free memory, else none), kept until hf_free; such batches
+ * screen their candidates against it before scoring them in float32. Results
+ * do not depend on it. Small batches, whose queries are shared by several
+ * warps, use 1.3 MB of scratch at most.
  * queries  : nq x d float32, row-major; nq >= 0 (0 returns HF_OK at once).
  * out_idx  : nq x k int32; out_dist : nq x k float32.
  */
@@ -204,8 +210,8 @@ int hf_build_segmented(const float* points, const int64_t* offsets, int32_t nset
  * mode 0, 1 or 2 when hf_graph_plan runs; a window the form cannot run is
  * HF_ENOTIMPL, never a change of form). hf_graph_plan keeps per-point lists
  * (and, for the Gram forms, the operand copies) in the forest for (k, w) and
- * the plain window kernel's block size `threads` (0: chosen per band, else
- * 256 or 512). hf_knn_graph_enqueue then enqueues the whole graph on
+ * the plain pair kernel's block size `threads` (0: chosen, else 256, for
+ * windows up to 480, or 512). hf_knn_graph_enqueue then enqueues the whole graph on
  * `stream` into DEVICE outputs (n x k) without allocating or synchronising,
  * so it can be captured; errors surface through hf_status, which synchronises
  * `stream` and reads and clears the device error word.

@@ -1213,9 +1213,9 @@ static int sketch_search(hf_forest* f, const float* q, const uint8_t* qc, int64_
 // Whether this search screens against the half-width copy of the points
 // (search.cu), which the first search that reads enough rows makes: copying
 // costs 1.5 reads of the matrix and saves half of every row scored, so four
-// rows scored per point pay for it within the same call. Without room for the
-// copy, or with rows that are not 16-byte aligned, the search reads the float32
-// rows as before. 10,000 queries, 3M x 384, T = 64, w = 50: 21 rows per point.
+// rows scored per point pay for it within the same call. Where the copy would
+// take more than a quarter of the free memory, or rows are not 16-byte aligned,
+// the search reads the float32 rows as before. 10,000 queries, 3M x 384, T = 64, w = 50: 21 rows per point.
 static bool search_uses16(hf_forest* f, const float* q, int64_t nq, int w, cudaStream_t s) {
   if (f->d % 4 || (reinterpret_cast<uintptr_t>(f->x) & 15) || (reinterpret_cast<uintptr_t>(q) & 15)) return false;
   // below 64 coordinates a row is two sectors or fewer, which halves save little of
@@ -1225,7 +1225,13 @@ static bool search_uses16(hf_forest* f, const float* q, int64_t nq, int w, cudaS
   if (f->x16) return true;
   void* x16 = nullptr;
   float* r16 = nullptr;
-  cudaError_t e = dalloc_bytes(&x16, (size_t)f->n * ((f->d + 63) / 64 * 64) * 2, s);
+  const size_t bytes = (size_t)f->n * ((f->d + 63) / 64 * 64) * 2;
+  size_t fr = 0, tot = 0;
+  if (cudaMemGetInfo(&fr, &tot) != cudaSuccess || bytes > fr / 4) {
+    cudaGetLastError();
+    return false;
+  }
+  cudaError_t e = dalloc_bytes(&x16, bytes, s);
   if (e == cudaSuccess) e = dalloc(&r16, (size_t)f->n, s);
   if (e == cudaSuccess) {
     launch_prepare16(f->x, f->n, f->d, x16, r16, s);
