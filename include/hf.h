@@ -247,7 +247,7 @@ int hf_exact_knn_rows(hf_forest* f, const int64_t* rows, int32_t nrows, int32_t 
  * limits) whose graph reaches target_recall on `sample` evenly spread rows
  * (recall against hf_exact_knn_rows; it grows with w because the candidate
  * sets grow), found by bisection, and at that w the faster block size of
- * the plain window kernel (256 or 512 threads; the Gram kernel is
+ * the plain pair kernel (256 or 512 threads; the Gram kernel is
  * persistent; the Gram forms are tried with 16 and with 32 list slots per
  * point, i.e. tensor_slack 16 - k and 32 - k, where they hold k + 1); then
  * the fastest variant that reaches the target (CUDA-event time of the whole
@@ -434,7 +434,7 @@ int hf_set_option(hf_forest* f, const char* key, int64_t value);
  * fix-up, [4] window distances + merge (all trees; the Gram kernels in mode
  * 1), [5] search, [6] number of kernel launches of the last build (as a
  * float), [7] re-rank (every form), [8] the form the last hf_knn_graph ran
- * (0 = plain float32 window kernel, 1 = BF16 tensor-core Gram bands, 2 = FP8
+ * (0 = plain float32 windows, 1 = BF16 tensor-core Gram bands, 2 = FP8
  * e4m3 Gram bands, 3 = sketch form), so a caller that asked for a tensor form can see whether
  * it fell back, [9] the time spent gathering each tree's rows into its
  * order (tensor forms; on a second stream, overlapping the previous tree's

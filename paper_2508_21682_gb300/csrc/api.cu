@@ -587,7 +587,7 @@ int knn_graph_impl(hf_forest* f, int32_t k, int32_t w, const int32_t* wpt, const
   cudaGetLastError();  // an earlier call's error was reported by that call
   const int64_t n = f->n;
   const bool budget = wpt != nullptr;
-  // Plain mode: the window kernel keeps the top kp >= k per point by exact
+  // Plain mode: the pair and merge kernels keep the top kp >= k per point by exact
   // float32 distance. Tensor mode: the Gram kernel keeps the top kp >= k + 1
   // (by default) by the BF16 expansion, then the re-rank orders them by exact
   // float32 distance. Either way the first k columns are the result.
@@ -702,7 +702,7 @@ int knn_graph_impl(hf_forest* f, int32_t k, int32_t w, const int32_t* wpt, const
   cudaEvent_t a1 = tm.mark();
   // every form's returned distances come from the re-rank's float32 exact
   // differences with the butterfly sum (relative error below 1.1e-6 at
-  // d = 384); the plain window kernel's sequential sums only select
+  // d = 384); the pair kernel's sequential sums only select
   if (rc == HF_OK)
     rc = launch_rerank(f->x, n, f->d, f->sigma, kp, sketchf ? (f->sketch_k2 > k ? f->sketch_k2 : k) : kp, li, ldd, s);
   cudaEvent_t a2 = tm.mark();

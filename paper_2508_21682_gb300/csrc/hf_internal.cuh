@@ -166,7 +166,7 @@ int segment_pass(hf_forest* f, const uint64_t* seg64, cudaStream_t s);
 int tie_fixup_big(hf_forest* f, int tree, uint32_t big_runs, cudaStream_t s);
 
 // window.cu
-int window_list_pitch(int k);  // list slots per point kept by the window kernel (>= k)
+int window_list_pitch(int k);  // list slots per point kept by the merge kernel (>= k)
 // scratch of a tree's pair distances (one row chunk of it)
 size_t window_band_bytes(int64_t n, int w);
 int launch_window_graph(const float* x, int64_t n, int d, const uint32_t* sigma, int w, int kp,

@@ -97,3 +97,31 @@ def test_pair_tiles_fp8(n, d, w):
         assert G.timings()["graph_form"] == 2.0
     oi, _ = O.knn_graph(F, 15, w)
     check_tensor_lists(x, gi.cpu().numpy(), gd.cpu().numpy(), oi, np.arange(n), min_hit=0.93)
+
+
+@pytest.mark.parametrize("mode,d,w", [(0, 40, 100), (1, 384, 40), (1, 384, 300), (2, 768, 300)])
+def test_captured_plan_equals_direct(mode, d, w):
+    """Pairs, the bound pass, single tiles and the plain band, replayed from a
+    captured graph after the direct call left other values in the outputs."""
+    import torch
+    import paper_2508_21682_gb300 as hf
+    x = torch.from_numpy(S.gaussian_mixture(6000, d, n_components=20, seed=4)).cuda()
+    with hf.build(x, T=3, bits=8, seed=5) as G:
+        G.set_option("mode", mode)
+        ri, rd = G.knn_graph(10, w)
+        assert G.timings()["graph_form"] == mode
+        G.graph_plan(10, w)
+        oi, od = torch.full_like(ri, -7), torch.full_like(rd, -7.0)
+        side = torch.cuda.Stream()
+        side.wait_stream(torch.cuda.current_stream())
+        graph = hf.CudaGraph(side.cuda_stream)
+        with graph:
+            G.knn_graph_enqueue(oi, od, side.cuda_stream)
+        for _ in range(2):
+            graph.launch()
+            G.status(side.cuda_stream)
+            assert torch.equal(oi, ri) and torch.equal(od, rd)
+            with torch.cuda.stream(side):
+                oi.fill_(-7)
+                od.fill_(-7.0)
+        graph.close()
