@@ -287,6 +287,7 @@ struct GramArgs {
   int nk;                  // K chunks of 128 bytes per row
   int elem_per_chunk;      // 64 (BF16) or 128 (FP8) elements per chunk
   int w;                   // window when tile_w is null
+  int w_max;               // wider windows are cut to this (the bounds' pass)
   int stages;              // B ring stages
   int box_rows;            // rows per TMA box
   int solo;                // no tile has more than one unit
@@ -296,6 +297,7 @@ struct GramArgs {
   float* ldist;
   float* thr;              // per position: a bound on the KP-th smallest estimate, or null
   int group;               // columns per group of the bound's pass
+  int w_bound;             // widest window of the bound's pass
   int* err;
   uint64_t spin_limit;
 };
@@ -453,6 +455,7 @@ __device__ __forceinline__ TileGeom tile_geom(const GramArgs& a, int64_t t) {
       g.w = __ldg(a.tile_w + t);
     }
   }
+  g.w = min(g.w, a.w_max);
   if (g.w <= 0) {
     g.w = g.W8 = g.ncol = g.J = 0;
     return g;
@@ -1269,8 +1272,11 @@ int launch_band(const GramArgs& a, const CUtensorMap& map, size_t smem, cudaStre
 template <int KP, bool F8, bool PAIR>
 int launch_tree(GramArgs a, bool bounds, const CUtensorMap& map, size_t smem, cudaStream_t s) {
   if (bounds) {
+    const int w_max = a.w_max;
+    a.w_max = a.w_bound;
     const int rc = launch_band<KP, F8, PAIR, true>(a, map, smem, s);
     if (rc != HF_OK) return rc;
+    a.w_max = w_max;
   } else {
     a.thr = nullptr;
   }
@@ -1357,11 +1363,19 @@ int launch_gram_window(int form, int64_t n, int d, const uint32_t* sigma, int w,
   a.spin_limit = 2000000000ull;  // 2 s per wait (globaltimer nanoseconds)
   // Bounds for a first tree: groups small enough for 4 KP of them in the
   // window, of 4 columns at least; not worth a pass below 2 KP groups, nor
-  // where a tile is one unit.
+  // where a tile is one unit. The middle of a wide window bounds the whole as
+  // well: 256 KP columns to each side. The pass pays by the insertions it
+  // spares, which grow with log w, and costs columns. First tree of 100,000,
+  // pass and band, us, without the pass / this rule / whole windows (KP = 16,
+  // d = 384): w = 2048: 1301 / 844 / 844; 8192: 2579 / 2004 / 2154; 100000:
+  // 13088 / 12379 / 21251; FP8 d = 768, KP = 32, w = 100000: 19128 / 16792 /
+  // 25131. Narrower: 1024 columns to each side: 951, 2164, 12650, 17940.
   a.thr = thr;
+  a.w_max = w;
+  a.w_bound = w < 256 * kp ? w : 256 * kp;
   a.group = 16;
-  while (a.group > 4 && 2 * w < 4 * kp * a.group) a.group >>= 1;
-  const bool bounds = thr && !p.solo && 2 * w >= 2 * kp * a.group;
+  while (a.group > 4 && a.w_bound < 2 * kp * a.group) a.group >>= 1;
+  const bool bounds = thr && !p.solo && a.w_bound >= kp * a.group;
   switch (kp * 4 + (f8 ? 2 : 0) + (p.pair ? 1 : 0)) {
     case 64: return launch_tree<16, false, false>(a, bounds, map, p.smem, s);
     case 65: return launch_tree<16, false, true>(a, bounds, map, p.smem, s);

@@ -52,6 +52,28 @@ def test_pair_tiles_equal_brute_force(n, d, w, k):
     assert np.array_equal(gi[rows], oi) and np.array_equal(gd[rows].astype(np.float64), od)
 
 
+@pytest.mark.parametrize("n,d,w,k", [(9001, 8, 4097, 10), (9001, 300, 9000, 15), (18000, 8, 8200, 20)])
+def test_windows_wider_than_the_bounds_pass(n, d, w, k):
+    import torch
+    import paper_2508_21682_gb300 as hf
+    x = S.small_integer_points(n, d, seed=n + d)
+    x[n // 2:n // 2 + 40] = x[:40]  # equal points far apart by index
+    with hf.build(torch.from_numpy(x).cuda(), T=2, bits=8, seed=5) as G:
+        orders = [G.order(t).astype(np.int64) for t in range(2)]
+        G.set_option("mode", 1)
+        gi, gd = G.knn_graph(k, w)
+        assert G.timings()["graph_form"] == 1.0
+        wp = torch.from_numpy(np.random.default_rng(1).integers(1, w + 1, n).astype(np.int32)).cuda()
+        bi, bd = G.knn_graph_budget(k, wp, torch.full((n,), 2, dtype=torch.int32, device="cuda"))
+        wp = wp.cpu().numpy()
+    rows = np.unique(np.concatenate([np.arange(0, n, 151), orders[0][:3], orders[0][-3:]]))
+    oi, od = _brute(x, orders, rows, k, lambda r, p, t: (max(0, p - w), min(n, p + w + 1)))
+    assert np.array_equal(gi.cpu().numpy()[rows], oi) and np.array_equal(gd.cpu().numpy()[rows].astype(np.float64), od)
+    oi, od = _brute(x, orders, rows, k, lambda r, p, t: (max(0, p - wp[r]), min(n, p + wp[r] + 1)))
+    bi, bd = bi.cpu().numpy()[rows], bd.cpu().numpy()[rows].astype(np.float64)
+    assert np.array_equal(bi, oi) and np.array_equal(bd, od)
+
+
 def test_pair_tiles_within_sets_and_budgets():
     import torch
     import paper_2508_21682_gb300 as hf
