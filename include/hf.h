@@ -214,7 +214,15 @@ int hf_build_segmented(const float* points, const int64_t* offsets, int32_t nset
  * windows up to 480, or 512). hf_knn_graph_enqueue then enqueues the whole graph on
  * `stream` into DEVICE outputs (n x k) without allocating or synchronising,
  * so it can be captured; errors surface through hf_status, which synchronises
- * `stream` and reads and clears the device error word.
+ * `stream` and reads and clears the device error word. The plan's buffers stay
+ * where they are until hf_free while later plans (hf_autotune's too) keep the
+ * form and the list slots per point (k, plus tensor_slack for the Gram forms,
+ * rounded up to 16, 32 or 64), whatever their window: graphs captured before
+ * can still be launched. A plan that changes either replaces buffers. Besides
+ * the lists a plain plan keeps the pair distances of a row chunk: about 4 w
+ * bytes per point, 256 MB at most, and as much as any window can need
+ * beside them from the first wider plan on. hf_knn_graph takes the former for
+ * the time of the call (modes 0 and 3).
  */
 int hf_graph_plan(hf_forest* f, int32_t k, int32_t w, int32_t threads, void* stream);
 int hf_knn_graph_enqueue(hf_forest* f, int32_t* out_idx, float* out_dist, void* stream);

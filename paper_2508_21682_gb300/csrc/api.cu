@@ -177,6 +177,7 @@ void destroy(hf_forest* f, cudaStream_t s) {
   dfree(f->plan_xs, s);
   dfree(f->plan_ms, s);
   dfree(f->plan_band, s);
+  dfree(f->plan_band_first, s);
   dfree(f->plan_thr, s);
   if (f->side) {
     cudaStreamSynchronize(s);  // the stream-ordered frees above run before the side stream goes
@@ -780,17 +781,21 @@ int hf_graph_plan(hf_forest* f, int32_t k, int32_t w, int32_t threads, void* str
   cudaGetLastError();
   const int64_t n = f->n;
   cudaError_t e = cudaSuccess;
+  // the band first: when there is no room for it, the earlier plan stands
+  if (!form && window_band_bytes(n, w) > f->plan_band_bytes) {
+    const size_t bytes = f->plan_band ? window_band_bytes_most(n) : window_band_bytes(n, w);
+    float* band = nullptr;
+    e = dalloc(&band, bytes / sizeof(float), s);
+    if (e != cudaSuccess) return map_cuda(e);
+    f->plan_band_first = f->plan_band;  // null, or the only band so far
+    f->plan_band = band;
+    f->plan_band_bytes = bytes;
+  }
   if (kp != f->plan_kp || !f->plan_li) {
     dfree(f->plan_li, s);
     dfree(f->plan_ld, s);
     e = dalloc(&f->plan_li, (size_t)n * kp, s);
     if (e == cudaSuccess) e = dalloc(&f->plan_ld, (size_t)n * kp, s);
-  }
-  if (e == cudaSuccess && !form && window_band_bytes(n, w) > f->plan_band_bytes) {
-    dfree(f->plan_band, s);
-    f->plan_band_bytes = 0;
-    e = dalloc(&f->plan_band, window_band_bytes(n, w) / sizeof(float), s);
-    if (e == cudaSuccess) f->plan_band_bytes = window_band_bytes(n, w);
   }
   if (e == cudaSuccess && form && (form != f->plan_form || !f->plan_xs)) {
     dfree(f->plan_xs, s);
@@ -817,8 +822,6 @@ int hf_graph_plan(hf_forest* f, int32_t k, int32_t w, int32_t threads, void* str
     dfree(f->plan_xs, s);
     dfree(f->plan_ms, s);
     dfree(f->plan_thr, s);
-    dfree(f->plan_band, s);
-    f->plan_band_bytes = 0;
     f->plan_kp = 0;
     return map_cuda(e);
   }

@@ -113,8 +113,14 @@ struct hf_forest {
   void* plan_xs = nullptr;     // tensor forms: operand rows in tree order
   float2* plan_ms = nullptr;
   float* plan_thr = nullptr;   // tensor forms: the first tree's bounds
-  float* plan_band = nullptr;  // plain form: pair distances of one row chunk
+  // plain form: pair distances of one row chunk. Enqueued and captured graphs
+  // hold the address, and a plan of another window with the same list width
+  // must leave them runnable: a band is kept until hf_free. The first plan takes
+  // what its window needs, the first wider one the most that any window can
+  // need, so there are two at most.
+  float* plan_band = nullptr;
   size_t plan_band_bytes = 0;
+  float* plan_band_first = nullptr;
   int plan_k = 0, plan_w = 0, plan_kp = 0, plan_nt = 0, plan_form = 0;
   int sketch_k2 = 60;     // candidates kept by Hamming distance (mode 3)
   int expand_h = 2;       // master-order neighbours per survivor (mode 3 search)
@@ -169,6 +175,7 @@ int tie_fixup_big(hf_forest* f, int tree, uint32_t big_runs, cudaStream_t s);
 int window_list_pitch(int k);  // list slots per point kept by the merge kernel (>= k)
 // scratch of a tree's pair distances (one row chunk of it)
 size_t window_band_bytes(int64_t n, int w);
+size_t window_band_bytes_most(int64_t n);  // the largest of them over all windows
 int launch_window_graph(const float* x, int64_t n, int d, const uint32_t* sigma, int w, int kp,
                         uint32_t* list_idx, float* list_dist, float* band, cudaStream_t s,
                         const uint32_t* segr = nullptr, const int64_t* segoff = nullptr, int nt = 0);

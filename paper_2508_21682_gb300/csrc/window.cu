@@ -416,6 +416,15 @@ int window_list_pitch(int k) { return k <= 16 ? 16 : (k <= 32 ? 32 : 64); }
 
 size_t window_band_bytes(int64_t n, int w) { return (size_t)band_geom(n, w).pitch * w * 4; }
 
+size_t window_band_bytes_most(int64_t n) {
+  size_t most = 0;
+  for (int w = 1; w <= HF_PLAIN_MAX_W; ++w) {
+    const size_t b = window_band_bytes(n, w);
+    if (b > most) most = b;
+  }
+  return most;
+}
+
 // w up to HF_PLAIN_MAX_W. Lists have window_list_pitch(k) slots per point;
 // band: window_band_bytes(n, w) of scratch.
 int launch_window_graph(const float* x, int64_t n, int d, const uint32_t* sigma, int w, int kp,
