@@ -618,13 +618,12 @@ void launch_merge(const SearchArgs& a, uint32_t* out_idx, float* out_dist, cudaS
 }
 
 // Parts per query. One warp walks all T trees of a query in T dependent steps
-// (key, probes, rows: about 30 us each at 200,000 x 384), which is the whole
-// time of a small batch; the trees, then the chunks of a window, go to as many
-// time of a small batch (5 queries, T = 32, w = 32: 1001 us a call, 107 split
-// into 64 parts each); the trees, then the chunks of a window, go to as many
-// warps as give the chip SPLIT_WARPS of them. From half that many queries on
-// the batch fills the chip by itself.
- int64_t SPLIT_WARPS = 152 * 16;
+// (key, probes, rows), which is the whole time of a small batch (5 queries, T =
+// 32, w = 32, 200,000 x 384: 1001 us a call, 107 split into 64 parts each). The
+// trees, then the chunks of a window, go to as many warps as give the chip
+// SPLIT_WARPS of them; from half that many queries on the batch fills the chip
+// by itself. search_parts sizes the part lists from the same split.
+constexpr int64_t SPLIT_WARPS = 152 * 16;
 
 void search_split(int64_t nq, int T, int w, int* tsplit, int* csplit) {
   const int64_t want = SPLIT_WARPS / nq;
