@@ -844,7 +844,6 @@ int hf_mlp_create(int32_t d, uint64_t seed, hf_mlp** out) {
   cudaMemset(m->b1, 0, H * 4);
   cudaMemset(m->b2, 0, H * 4);
   cudaMemset(m->b3, 0, hf_mlp::OUTP * 4);
-  cudaMemset(m->b3, 0, hf_mlp::OUTP * 4);
   cudaMemset(m->mom, 0, (size_t)2 * m->nparam * 4);
   cudaMemset(m->w3t, 0, (size_t)H * 64 * 2);
   cudaMemset(m->err, 0, 4);
