@@ -482,9 +482,10 @@ __device__ __forceinline__ uint32_t xor_scan_msb(uint32_t v) {
 //   tie_words  word K by the transform of the top Lf levels, for the rest;
 //   tie_rank   each member counts the members of its run that precede it.
 // Members that also tie on every word at hand form sub-runs of the ranked
-// order; tie_hard orders those by the full key. Runs longer than TIE_RUN_CAP
-// and sub-runs longer than tie_hard_cap go to the list of big runs, which the
-// host settles after the build's sync.
+// order; tie_hard orders those by the next words of the top bit level, where the
+// key has any, and then by the full key. Runs longer than TIE_RUN_CAP and
+// sub-runs longer than tie_hard_cap go to the list of big runs, which the host
+// settles after the build's sync.
 // The scratch is the sort's own, free after the last pass: words in keys_a,
 // sub-runs in keys_b, points in vals_a, listed positions in vals_b.
 // ---------------------------------------------------------------------------
@@ -492,8 +493,11 @@ __device__ __forceinline__ uint32_t xor_scan_msb(uint32_t v) {
 // the cap, about 20 us of the whole chip.
 constexpr int TIE_RUN_CAP = 8192;
 // Sub-run members whose full keys fit a block's scratch slice: 304 slices of
-// 256 x 48 words at d = 384 are 30 MB; rows of more than 64 words keep 64.
-__host__ __device__ constexpr int tie_hard_cap(int W) { return W <= 64 ? 256 : 64; }
+// 256 x 48 words at d = 384 are 30 MB, of 256 x 128 words at d = 1024 80 MB;
+// longer keys keep 64.
+__host__ __device__ constexpr int tie_hard_cap(int W) { return W <= 128 ? 256 : 64; }
+constexpr int TIE_HARD_WARPS = 8;
+constexpr int TIE_TOP_WORDS = 3;  // words past word K that tie_hard takes from the top bit level
 
 struct TieArgs {  // the first tree of the batch; strides below
   const uint64_t* prefix;  // [tb][K][n] sorted
@@ -512,7 +516,39 @@ struct TieArgs {  // the first tree of the batch; strides below
   const int* err;
   int64_t n, big_cap;
   int d, W32, bits, W, K, K2, Lf, tb, stride;
+  int top;   // words K + 1 .. K + top lie in the top bit level and tie_hard tries them first
+  int rows;  // coordinate rows of a tie_hard block's shared memory
 };
+
+// Key words w0 .. w0 + nw - 1 (nw <= N) of the point whose plane-0 row is `row`,
+// all in the top bit level (d >= 64 (w0 + nw)): the whole warp forms them with
+// ballots over the permuted, reflected top bits, carrying the parity of the
+// first 64 w0. Every lane gets them.
+template <int N>
+__device__ __forceinline__ void tie_top_words(const uint32_t* __restrict__ row, const int32_t* __restrict__ pi,
+                                              const uint32_t* __restrict__ rb, int w0, int nw, int lane,
+                                              uint64_t* out) {
+  auto ballot = [&](int h) {
+    const int c = __ldg(pi + 32 * h + lane);
+    const uint32_t bit = ((__ldg(row + (c >> 5)) >> (c & 31)) ^ (__ldg(rb + h) >> lane)) & 1u;
+    return __ballot_sync(0xffffffffu, bit);
+  };
+  uint32_t carry = 0;
+  for (int h = 0; h < 2 * w0; ++h) carry ^= __popc(ballot(h)) & 1u;
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    out[i] = 0;
+    if (i < nw) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        uint32_t v = xor_scan_msb(__brev(ballot(2 * (w0 + i) + h)));
+        if (carry) v = ~v;
+        carry = v & 1u;
+        out[i] = (out[i] << 32) | v;
+      }
+    }
+  }
+}
 
 // WORDS: where word K comes from. 0: the key kernel computed it (K2 > K); 1:
 // it lies in the top bit level (d >= 64 (K + 1)), a warp forms it per tied
@@ -556,22 +592,9 @@ __global__ void __launch_bounds__(256) tie_mark_kernel(const TieArgs a) {
       for (uint32_t rest = mask; rest; rest &= rest - 1) {
         const int src = __ffs(rest) - 1;
         const uint32_t q = __shfl_sync(0xffffffffu, p, src);
-        const uint32_t* row = a.planes + (size_t)q * a.W32;
-        uint32_t carry = 0, half[2] = {0, 0};
-        for (int h = 0; h < 2 * K + 2; ++h) {
-          const int c = __ldg(pi + 32 * h + lane);
-          const uint32_t bit = ((__ldg(row + (c >> 5)) >> (c & 31)) ^ (__ldg(rb + h) >> lane)) & 1u;
-          const uint32_t bal = __ballot_sync(0xffffffffu, bit);
-          if (h < 2 * K) {
-            carry ^= __popc(bal) & 1u;
-          } else {
-            uint32_t v = xor_scan_msb(__brev(bal));
-            if (carry) v = ~v;
-            carry = v & 1u;
-            half[h & 1] = v;
-          }
-        }
-        if (lane == src) word[m] = ((uint64_t)half[0] << 32) | half[1];
+        uint64_t wk;
+        tie_top_words<1>(a.planes + (size_t)q * a.W32, pi, rb, K, 1, lane, &wk);
+        if (lane == src) word[m] = wk;
       }
     }
   }
@@ -844,49 +867,149 @@ __global__ void __launch_bounds__(256) tie_rank_kernel(const TieArgs a) {
   }
 }
 
-// Sub-runs that tie on every word at hand: one block each (few: the next 64
-// bits settle all but near-duplicate points), ranked by (full key, index) from
-// full keys in the block's slice of global scratch. The time is that of one
-// member's key, a serial chain: 0.49 ms at d = 384 with the coordinates read
-// bit by bit through the permutation.
-__global__ void tie_hard_kernel(const TieArgs a, uint64_t* __restrict__ fk_scratch) {
+// -1 / 0 / +1 comparing the N words x and y.
+template <int N>
+__device__ __forceinline__ int cmp_words(const uint64_t (&x)[N], const uint64_t (&y)[N]) {
+  int c = 0;
+#pragma unroll
+  for (int i = N - 1; i >= 0; --i) c = x[i] < y[i] ? -1 : (x[i] > y[i] ? 1 : c);
+  return c;
+}
+
+// Sub-runs that tie on every word at hand, ranked by the next words of the top
+// bit level where there are any (a.top), and if some members tie on those too,
+// by (full key, index) from full keys in the block's slice of global scratch.
+// Sub-runs of few members (a warp's share of the block's rows) take a warp each,
+// eight at a time in a block, the others the whole block, one member per thread.
+// A member's full key is a serial chain of one thread, 60 us at d = 384, however
+// many lanes run beside it; its top-level words take a warp about 1 us. Near-
+// duplicates make sub-runs by the hundred thousand. Builds of 500,000 x 384, T =
+// 4, groups of 10 copies with 5 % / 1 % / 0.1 % noise: 2.5 / 40.2 / 32.8 ms; with
+// one block per sub-run and full keys at once 39.4 / 198 / 130; with one block
+// per run of equal prefixes, four words and then full keys for the whole run,
+// 9.6 / 287 / 294. 50,000 x 768, T = 1, in groups of 1,000 with 20 % noise, where
+// the few sub-runs' chain is a third of the build: 0.755 -> 0.48 ms.
+__global__ void __launch_bounds__(TIE_HARD_WARPS * 32) tie_hard_kernel(const TieArgs a,
+                                                                       uint64_t* __restrict__ fk_scratch) {
   extern __shared__ __align__(16) unsigned char smraw[];
   if (*(volatile const int*)a.err) return;
   const int64_t n = a.n;
-  const int d = a.d, W = a.W;
-  uint32_t* pt = reinterpret_cast<uint32_t*>(smraw);
-  const int cap = tie_hard_cap(W);
-  int32_t* inv = reinterpret_cast<int32_t*>(pt + cap);
-  uint8_t* Y = reinterpret_cast<uint8_t*>(inv + d) + (size_t)threadIdx.x * a.stride;
+  const int d = a.d, W = a.W, top = a.top, cap = tie_hard_cap(W);
+  const bool all = a.K + 1 + top >= W;  // the key has no words beyond those
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int share = a.rows / TIE_HARD_WARPS;  // members of a warp's sub-run, 32 at most
+  uint64_t* tw = reinterpret_cast<uint64_t*>(smraw);                        // [cap][TIE_TOP_WORDS]
+  uint32_t* pt = reinterpret_cast<uint32_t*>(tw + (size_t)cap * TIE_TOP_WORDS);  // [cap]
+  int32_t* inv = reinterpret_cast<int32_t*>(pt + cap);                      // [d]
+  uint8_t* Y = reinterpret_cast<uint8_t*>(inv + d);                         // [rows][stride]
   uint64_t* fk = fk_scratch + (size_t)blockIdx.x * cap * W;
+  auto full_key = [&](uint32_t p, int row, uint64_t* out) {
+    uint8_t* y = Y + (size_t)row * a.stride;
+    tie_load_row(a.planes, n, d, a.W32, a.bits, inv, p, y);
+    hf_skilling(y, d, a.bits);
+    for (int w = 0; w < W; ++w) out[w] = hf_pack_word(y, d, a.bits, w);
+  };
   for (int tr = 0; tr < a.tb; ++tr) {
     const uint32_t nruns = a.counters[(size_t)tr * 4 + 2];
     uint32_t* sigma = a.sigma + (size_t)tr * n;
+    const uint2* hard = a.hard + (size_t)tr * n;
+    const int32_t* pi = a.pi + (size_t)tr * d;
+    const uint32_t* rb = a.rbits + (size_t)tr * a.W32;
     // trees start at different blocks, so that a few sub-runs per tree spread
     const uint32_t first = (blockIdx.x + (uint32_t)tr * 37u) % gridDim.x;
     if (first >= nruns) continue;
-    tie_inverse(a.pi + (size_t)tr * d, a.rbits + (size_t)tr * a.W32, d, inv);
+    tie_inverse(pi, rb, d, inv);
     __syncthreads();
-    for (uint32_t r = first; r < nruns; r += gridDim.x) {
-      const uint2 run = a.hard[(size_t)tr * n + r];
-      const int len = (int)run.y;  // <= cap
-      for (int e = threadIdx.x; e < len; e += blockDim.x) {
-        const uint32_t p = sigma[run.x + e];
-        pt[e] = p;
-        if (p >= (uint64_t)n) continue;  // cannot happen for a valid order
-        tie_load_row(a.planes, n, d, a.W32, a.bits, inv, p, Y);
-        hf_skilling(Y, d, a.bits);
-        for (int w = 0; w < W; ++w) fk[(size_t)e * W + w] = hf_pack_word(Y, d, a.bits, w);
+    // short sub-runs, a warp each
+    for (uint64_t r = first + (uint64_t)warp * gridDim.x; r < nruns; r += (uint64_t)TIE_HARD_WARPS * gridDim.x) {
+      const uint2 run = hard[r];
+      const int len = (int)run.y;
+      if (len > share) continue;
+      const bool in = lane < len;
+      uint32_t p = in ? sigma[run.x + lane] : 0;
+      if (p >= (uint64_t)n) p = 0;  // cannot happen for a valid order
+      uint64_t own[TIE_TOP_WORDS] = {};
+      for (int e = 0; e < len && top; ++e) {
+        uint64_t w[TIE_TOP_WORDS];
+        tie_top_words<TIE_TOP_WORDS>(a.planes + (size_t)__shfl_sync(0xffffffffu, p, e) * a.W32, pi, rb, a.K + 1, top,
+                                     lane, w);
+#pragma unroll
+        for (int i = 0; i < TIE_TOP_WORDS; ++i)
+          if (lane == e) own[i] = w[i];
       }
-      __syncthreads();
-      for (int e = threadIdx.x; e < len; e += blockDim.x) {
-        uint32_t rk = 0;
-        for (int g = 0; g < len; ++g)
-          rk += full_less(fk + (size_t)g * W, pt[g], fk + (size_t)e * W, pt[e], W) ? 1u : 0u;
-        sigma[run.x + rk] = pt[e];
+      // members that tie on those stay in position order, which is index order
+      int rank = 0;
+      bool tie = false;
+      for (int g = 0; g < len; ++g) {
+        uint64_t o[TIE_TOP_WORDS];
+#pragma unroll
+        for (int i = 0; i < TIE_TOP_WORDS; ++i) o[i] = __shfl_sync(0xffffffffu, own[i], g);
+        const int c = cmp_words(o, own);
+        rank += c < 0 || (c == 0 && g < lane) ? 1 : 0;
+        tie |= in && c == 0 && g != lane;
       }
-      __syncthreads();
+      if (!all && __any_sync(0xffffffffu, tie)) {
+        uint64_t* wk = fk + (size_t)(warp * share) * W;
+        if (in) full_key(p, warp * share + lane, wk + (size_t)lane * W);
+        __syncwarp();
+        rank = 0;
+        for (int g = 0; g < len; ++g) {
+          const uint32_t pg = __shfl_sync(0xffffffffu, p, g);
+          if (in) rank += full_less(wk + (size_t)g * W, pg, wk + (size_t)lane * W, p, W) ? 1 : 0;
+        }
+        __syncwarp();  // the keys are read before the warp's next sub-run
+      }
+      if (in) sigma[run.x + rank] = p;
     }
+    __syncthreads();  // the rows and the scratch change hands
+    // the others, the whole block each (len <= cap <= the block's threads)
+    for (uint64_t r = first; r < nruns; r += gridDim.x) {
+      const uint2 run = hard[r];
+      const int len = (int)run.y;
+      if (len <= share) continue;
+      const bool in = tid < len;
+      uint32_t p = in ? sigma[run.x + tid] : 0;
+      if (p >= (uint64_t)n) p = 0;  // cannot happen for a valid order
+      if (in) pt[tid] = p;
+      __syncthreads();
+      for (int e = warp; e < len && top; e += TIE_HARD_WARPS) {
+        uint64_t w[TIE_TOP_WORDS];
+        tie_top_words<TIE_TOP_WORDS>(a.planes + (size_t)pt[e] * a.W32, pi, rb, a.K + 1, top, lane, w);
+        if (lane == 0)
+#pragma unroll
+          for (int i = 0; i < TIE_TOP_WORDS; ++i) tw[e * TIE_TOP_WORDS + i] = w[i];
+      }
+      __syncthreads();
+      int rank = 0;
+      bool tie = false;
+      if (in && top) {
+        uint64_t own[TIE_TOP_WORDS], o[TIE_TOP_WORDS];
+#pragma unroll
+        for (int i = 0; i < TIE_TOP_WORDS; ++i) own[i] = tw[tid * TIE_TOP_WORDS + i];
+        for (int g = 0; g < len; ++g) {
+#pragma unroll
+          for (int i = 0; i < TIE_TOP_WORDS; ++i) o[i] = tw[g * TIE_TOP_WORDS + i];
+          const int c = cmp_words(o, own);
+          rank += c < 0 || (c == 0 && g < tid) ? 1 : 0;
+          tie |= c == 0 && g != tid;
+        }
+      } else {
+        rank = tid;
+        tie = in;
+      }
+      if (!all && __syncthreads_or(tie)) {
+        if (tid < a.rows)
+          for (int e = tid; e < len; e += a.rows) full_key(pt[e], tid, fk + (size_t)e * W);
+        __syncthreads();
+        rank = 0;
+        if (in)
+          for (int g = 0; g < len; ++g)
+            rank += full_less(fk + (size_t)g * W, pt[g], fk + (size_t)tid * W, p, W) ? 1 : 0;
+      }
+      if (in) sigma[run.x + rank] = p;
+      __syncthreads();  // pt, tw and the keys are read before the next sub-run
+    }
+    __syncthreads();  // the table is read before the next tree's
   }
 }
 
@@ -958,9 +1081,16 @@ __global__ void iota_kernel(uint32_t* a, uint32_t m) {
 
 constexpr int TIE_BLOCKS = 152 * 2;
 
-// Threads of a tie_hard block: their coordinate rows (d bytes each) share the
-// block's shared memory.
-int tie_hard_threads(int d) { return d <= 2048 ? 64 : 32; }
+// Shared memory of a tie_hard block, and its coordinate rows (d bytes each): as
+// many as let two blocks share an SM, 32 at least (131 KB at d = 4096).
+size_t tie_hard_smem(int W, int d, int stride, int rows) {
+  return (size_t)tie_hard_cap(W) * (TIE_TOP_WORDS * 8 + 4) + (size_t)d * 4 + (size_t)rows * stride;
+}
+int tie_hard_rows(int W, int d, int stride) {
+  int rows = tie_hard_cap(W);
+  while (rows > 32 && tie_hard_smem(W, d, stride, rows) > 112 * 1024) rows >>= 1;
+  return rows;
+}
 
 // Levels that word K needs, and the row stride of tie_words.
 int tie_levels(int d, int bits, int K) {
@@ -1120,10 +1250,11 @@ int sort_batch(hf_forest* f, int t0, int tb, cudaStream_t s) {
     tie_rank_kernel<<<grid, 256, 0, s>>>(a);
     hf_after_launch("tie_rank_kernel", s);
     if ((K2 > K + 1 ? K2 : K + 1) < f->W) {
-      const int ht = tie_hard_threads(f->d);
-      const size_t sm = (size_t)(tie_hard_cap(f->W) + f->d) * 4 + (size_t)ht * a.stride;
+      a.rows = tie_hard_rows(f->W, f->d, a.stride);
+      if (K2 == K && f->d >= 64 * (K + 1)) a.top = std::min(TIE_TOP_WORDS, f->d / 64 - (K + 1));
+      const size_t sm = tie_hard_smem(f->W, f->d, a.stride, a.rows);
       set_attr((const void*)tie_hard_kernel, sm);
-      tie_hard_kernel<<<TIE_BLOCKS, ht, sm, s>>>(a, f->tie.fk);
+      tie_hard_kernel<<<TIE_BLOCKS, TIE_HARD_WARPS * 32, sm, s>>>(a, f->tie.fk);
       hf_after_launch("tie_hard_kernel", s);
     }
   }
