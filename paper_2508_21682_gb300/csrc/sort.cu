@@ -111,8 +111,13 @@ __global__ void hist_scan_kernel(uint32_t* __restrict__ hist) {
 // Prices in picoseconds (3M x 384, 4M x 64, 1.2M x 128): a pass 11 per point
 // (or its launch's latency, on small inputs), refining 24 per point and 60 per
 // point of a run that reaches past a warp's 32 positions, a compare 0.5,
-// fetching the first word again in the final order 9. A run that the sample
-// misses costs time, not order. Per sort: 3M x 384, T = 64: 33.2 -> 25.9 ms of
+// fetching the first word again in the final order 9. The members of the longest
+// run wait for a chain of as many compares, 120 ns each (40 where the first
+// words are equal and only the second ones are read), once for all trees of the
+// batch, which is the refining's time where it is above the rest (50,000 x 384
+// mixture data, T = 1, without this price: runs of up to 1,731, 207 us of
+// refining to save 104 us of passes). A run that the sample misses costs time,
+// not order. Per sort: 3M x 384, T = 64: 33.2 -> 25.9 ms of
 // kernels; 4M x 64, T = 16, where half of the points tie at 128 bits, keeps
 // every pass; 200,001 x 384, T = 16: 3.88 -> 3.74 ms, build and narrow graph.
 // A sample of 4096 takes 70 us, one block's sort, and one of 1024 24 us, which
@@ -127,6 +132,7 @@ __global__ void __launch_bounds__(1024) sort_plan_kernel(const uint64_t* __restr
   constexpr int E = PLAN_S / 1024;
   __shared__ uint64_t s[PLAN_S];
   __shared__ unsigned long long pairs[PLAN_LEVELS];
+  __shared__ uint32_t longest[PLAN_LEVELS];
   const uint64_t* word = pk + blockIdx.x * pk_ts;
   const int tid = threadIdx.x;
   const int S = n < PLAN_S ? (int)n : PLAN_S;
@@ -140,7 +146,7 @@ __global__ void __launch_bounds__(1024) sort_plan_kernel(const uint64_t* __restr
     const uint32_t h = (uint32_t)j * 0x9E3779B1u;
     v[e] = j < S ? __ldg(word + (int64_t)j * stride + (int64_t)((h >> 8) % (uint64_t)stride)) : ~0ull;
   }
-  if (tid < PLAN_LEVELS) pairs[tid] = 0;
+  if (tid < PLAN_LEVELS) pairs[tid] = longest[tid] = 0;
 #pragma unroll 1
   for (int kk = 2; kk <= PLAN_S; kk <<= 1)
 #pragma unroll 1
@@ -165,6 +171,7 @@ __global__ void __launch_bounds__(1024) sort_plan_kernel(const uint64_t* __restr
   __syncthreads();
   for (int l = 0; l < PLAN_LEVELS; ++l) {
     unsigned long long mine = 0;
+    uint32_t most = 0;  // points before one that share its top bits
     for (int i = tid; i < S; i += 1024) {  // (padding sorts last)
       const uint64_t v = s[i] >> (8 * l);
       int lo = 0, hi = i;  // first point with these top bits
@@ -174,10 +181,15 @@ __global__ void __launch_bounds__(1024) sort_plan_kernel(const uint64_t* __restr
         else hi = mid;
       }
       mine += (unsigned long long)(i - lo);
+      most = max(most, (uint32_t)(i - lo));
     }
+    most = __reduce_max_sync(0xffffffffu, most);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mine += __shfl_down_sync(0xffffffffu, mine, o);
-    if ((tid & 31) == 0 && mine) atomicAdd(&pairs[l], mine);
+    if ((tid & 31) == 0 && mine) {
+      atomicAdd(&pairs[l], mine);
+      atomicMax(&longest[l], most);
+    }
   }
   __syncthreads();
   if (tid == 0) {
@@ -190,8 +202,10 @@ __global__ void __launch_bounds__(1024) sort_plan_kernel(const uint64_t* __restr
       // mates per point; a run of m crosses a 32-position boundary with
       // probability about m / 32
       const double mates = compares / dn, cross = mates / (mates + 32.0);
+      // (two samples of one run may be all of it)
+      const double chain = longest[l] > 1 ? (l ? 120e3 : 40e3) * (longest[l] - 1) * (dn / S) / TB : 0.0;
       const double cost =
-          pass * (8 - l) + 24.0 * dn + cross * 60.0 * dn + 0.5 * cross * compares + (l ? 9.0 * dn : 0.0);
+          pass * (8 - l) + 24.0 * dn + fmax(cross * (60.0 * dn + 0.5 * compares), chain) + (l ? 9.0 * dn : 0.0);
       const uint32_t st = (uint32_t)(8 * (K - 1) + l);
       if (st && cost < best) {
         best = cost;
@@ -888,7 +902,7 @@ __device__ __forceinline__ int cmp_words(const uint64_t (&x)[N], const uint64_t 
 // one block per sub-run and full keys at once 39.4 / 198 / 130; with one block
 // per run of equal prefixes, four words and then full keys for the whole run,
 // 9.6 / 287 / 294. 50,000 x 768, T = 1, in groups of 1,000 with 20 % noise, where
-// the few sub-runs' chain is a third of the build: 0.755 -> 0.48 ms.
+// the few sub-runs' chain is a third of the build: 0.755 -> 0.45 ms.
 __global__ void __launch_bounds__(TIE_HARD_WARPS * 32) tie_hard_kernel(const TieArgs a,
                                                                        uint64_t* __restrict__ fk_scratch) {
   extern __shared__ __align__(16) unsigned char smraw[];
