@@ -332,8 +332,13 @@ __global__ void prepare16_kernel(const float* __restrict__ x, int64_t n, int d, 
   }
 }
 
+// Float32 rows: six blocks an SM, 80 registers, 16 rows' loads in flight. Left to
+// itself the compiler took the same number and issued the loads one after the
+// other (hf_search_static, 10,000 queries, T = 32, w = 8 to 128, d = 64 to 384: a
+// geometric mean of 12 % slower at k <= 32, 21 % at k = 64); five blocks (96
+// registers) are 9 % faster below 1,000 queries, 7 % slower from 10,000 on.
 template <int S, bool B16>
-__global__ void __launch_bounds__(SWARPS * 32) search_kernel(SearchArgs a) {
+__global__ void __launch_bounds__(SWARPS * 32, B16 ? 4 : 6) search_kernel(SearchArgs a) {
   extern __shared__ __align__(16) unsigned char smraw[];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const size_t per_warp = search_per_warp(a.K, a.d);
