@@ -147,9 +147,11 @@ int hf_knn_graph(hf_forest* f, int32_t k, int32_t w, int32_t* out_idx, float* ou
  * The first batch of 1024 queries or more that scores four rows per point or
  * more makes a BF16 copy of the points (n x 64-padded d, plus n floats; at most
  * a quarter of the free memory, else none), kept until hf_free; such batches
- * screen their candidates against it before scoring them in float32. Results
- * do not depend on it. Small batches, whose queries are shared by several
- * warps, use 1.3 MB of scratch at most.
+ * screen their candidates against it before scoring them in float32 (with k
+ * above 32 only where a query has enough candidates for it to pay). Results do
+ * not depend on it. Their scratch holds the positions of as many queries as fit
+ * 64 MB (8 T bytes each), or of 2048. Small batches, whose queries are shared by
+ * several warps, use 1.3 MB at most.
  * queries  : nq x d float32, row-major; nq >= 0 (0 returns HF_OK at once).
  * out_idx  : nq x k int32; out_dist : nq x k float32.
  */

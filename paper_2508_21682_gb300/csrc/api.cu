@@ -1201,7 +1201,7 @@ static int sketch_search(hf_forest* f, const float* q, const uint8_t* qc, int64_
   if (e == cudaSuccess) e = dalloc_bytes(&qb, (size_t)nq * dp * 2, s);
   if (e == cudaSuccess) e = dalloc(&qsk, (size_t)nq * words, s);
   int rc = map_cuda(e);
-  if (rc == HF_OK) rc = launch_search(f, q, qc, nq, k, w, nullptr, nullptr, pos, -2, s);
+  if (rc == HF_OK) rc = launch_positions(f, q, qc, nq, -1, pos, s);
   if (rc == HF_OK) {
     launch_f32_to_bf16(q, nq, d, dp, qb, s);
     rc = launch_sketch(qb, nq, dp, f->sketch_r, f->sketch_bits, qsk, f->err, s);
@@ -1218,12 +1218,19 @@ static int sketch_search(hf_forest* f, const float* q, const uint8_t* qc, int64_
 // costs 1.5 reads of the matrix and saves half of every row scored, so four
 // rows scored per point pay for it within the same call. Where the copy would
 // take more than a quarter of the free memory, or rows are not 16-byte aligned,
-// the search reads the float32 rows as before. 10,000 queries, 3M x 384, T = 64, w = 50: 21 rows per point.
-static bool search_uses16(hf_forest* f, const float* q, int64_t nq, int w, cudaStream_t s) {
+// the search reads the float32 rows as before. 10,000 queries, 3M x 384, T = 64,
+// w = 50: 21 rows per point.
+// Lists of more than 32 keep candidates that pass the screen coming for longer,
+// and each is scored on its own: from 6,500 k / d rows per query on the screen
+// has made up for them (10,000 queries, 2M points, T = 32, k = 64, with and
+// without: d = 128, 1,024 / 2,048 / 3,200 rows: 1.59 / 2.31 / 3.29 against 1.27 /
+// 2.01 / 3.08 ms; d = 384, 1,024: 2.98 against 2.69).
+static bool search_uses16(hf_forest* f, const float* q, int64_t nq, int k, int w, cudaStream_t s) {
   if (f->d % 4 || (reinterpret_cast<uintptr_t>(f->x) & 15) || (reinterpret_cast<uintptr_t>(q) & 15)) return false;
   // below 64 coordinates a row is two sectors or fewer, which halves save little of
-  const double rows = (double)nq * 2.0 * w * f->T;
+  const double per_query = 2.0 * w * f->T, rows = (double)nq * per_query;
   if (f->d < 64 || rows < 4.0 * (double)f->n || nq < 1024) return false;
+  if (k > 32 && per_query * f->d < 6500.0 * k) return false;
   std::lock_guard<std::mutex> lock(f->x16_mu);
   if (f->x16) return true;
   void* x16 = nullptr;
@@ -1275,6 +1282,7 @@ int hf_search(hf_forest* f, const float* queries, int64_t nq, int32_t k, int32_t
   const int64_t parts = f->mode == 3 ? 1 : search_parts(f, nq, w);
   uint32_t* part_i = nullptr;
   float* part_d = nullptr;
+  int64_t* pos16 = nullptr;  // positions, when the search screens against the half-width copy
   if (e == cudaSuccess && parts > 1) e = dalloc(&part_i, cnt * parts, s);
   if (e == cudaSuccess && parts > 1) e = dalloc(&part_d, cnt * parts, s);
   int rc = map_cuda(e);
@@ -1286,9 +1294,13 @@ int hf_search(hf_forest* f, const float* queries, int64_t nq, int32_t k, int32_t
     launch_quantize_codes(qsrc, nq, d, f->lo, f->scale, f->bits, qc, f->err, s);
     if (rc == HF_OK && f->mode == 3)
       rc = sketch_search(f, qsrc, qc, nq, k, w, li, ldd, s);
-    else if (rc == HF_OK)
-      rc = launch_search(f, qsrc, qc, nq, k, w, li, ldd, nullptr, -1, s, part_i, part_d,
-                         search_uses16(f, qsrc, nq, w, s));
+    else if (rc == HF_OK) {
+      // no room for the positions: no screen
+      if (search_uses16(f, qsrc, nq, k, w, s) &&
+          dalloc(&pos16, (size_t)f->T * search16_slice(nq, f->T), s) != cudaSuccess)
+        cudaGetLastError();
+      rc = launch_search(f, qsrc, qc, nq, k, w, li, ldd, s, part_i, part_d, pos16);
+    }
     cudaEvent_t a1 = tm.mark();
     tm.span(5, a0, a1);
     if (rc == HF_OK && !dev_i) rc = map_cuda(cudaMemcpyAsync(out_idx, li, cnt * 4, cudaMemcpyDeviceToHost, s));
@@ -1301,6 +1313,7 @@ int hf_search(hf_forest* f, const float* queries, int64_t nq, int32_t k, int32_t
   dfree(qc, s);
   dfree(part_i, s);
   dfree(part_d, s);
+  dfree(pos16, s);
   if (!dev_i) dfree(li, s);
   if (!dev_d) dfree(ldd, s);
   return rc;
@@ -1401,7 +1414,7 @@ int hf_debug_locate(hf_forest* f, int32_t tree, const float* queries, int64_t nq
     if (!dev_q) cudaMemcpyAsync(qd, queries, (size_t)nq * d * 4, cudaMemcpyHostToDevice, s);
     const float* qsrc = dev_q ? queries : qd;
     launch_quantize_codes(qsrc, nq, d, f->lo, f->scale, f->bits, qc, f->err, s);
-    rc = launch_search(f, qsrc, qc, nq, 1, 1, nullptr, nullptr, po, tree, s);
+    rc = launch_positions(f, qsrc, qc, nq, tree, po, s);
     if (rc == HF_OK && !dev_o) rc = map_cuda(cudaMemcpyAsync(out_pos, po, (size_t)nq * 8, cudaMemcpyDeviceToHost, s));
     int rc2 = finish(f, s);
     if (rc == HF_OK) rc = rc2;

@@ -227,9 +227,17 @@ int launch_sketch(const void* xb, int64_t n, int dp, const void* rb, int bits, u
 void launch_f32_to_bf16(const float* x, int64_t rows, int cols, int ld, void* out, cudaStream_t s);
 
 // search.cu
-int launch_search(const hf_forest* f, const float* q, const uint8_t* qcodes, int64_t nq, int k,
-                  int w, uint32_t* out_idx, float* out_dist, int64_t* out_pos, int only_tree,
-                  cudaStream_t s, uint32_t* part_idx = nullptr, float* part_dist = nullptr, bool use16 = false);
+// pos16: T x search16_slice(nq, T) positions of scratch for a search through the
+// half-width copy, or null
+int launch_search(const hf_forest* f, const float* q, const uint8_t* qcodes, int64_t nq, int k, int w,
+                  uint32_t* out_idx, float* out_dist, cudaStream_t s, uint32_t* part_idx = nullptr,
+                  float* part_dist = nullptr, int64_t* pos16 = nullptr);
+// queries that a screened search locates at a time (their positions take 64 MB,
+// or 2048 queries' worth)
+int64_t search16_slice(int64_t nq, int T);
+// positions of the queries in one tree (out_pos: nq), or in all (tree -1; T x nq)
+int launch_positions(const hf_forest* f, const float* q, const uint8_t* qcodes, int64_t nq, int tree, int64_t* out_pos,
+                     cudaStream_t s);
 // the search's half-width copy of the points: x16 n x 64-padded d BF16, r16 n
 void launch_prepare16(const float* x, int64_t n, int d, void* x16, float* r16, cudaStream_t s);
 // warps that share one query of a batch (1: no split); a split search keeps a

@@ -24,17 +24,20 @@
 //    (query, point) pair gets the same value in every tree.
 //  * Merge: the 32 scored candidates are sorted across the warp and inserted
 //    in ascending order until the first one that cannot enter.
-//  * Large batches read a half-width copy of the points first (B16 below):
-//    the distance to a point's BF16 copy, less the copy's distance from the
-//    point, bounds the point's distance from below, and only candidates whose
-//    bound does not exceed the list's last entry are scored, from the float32
-//    rows and in the arithmetic above. The lists are the same. 10,000 queries,
-//    3M x 384, T = 64, w = 50 (98 GB of float32 rows): 18.2 -> 12.4 ms, 13.5
-//    with the copy's making; bound by the screen's instructions (about 12 per
-//    row and four coordinates), no longer by HBM.
+//  * Large batches locate their queries in a launch of their own and read a
+//    half-width copy of the points first (search16_kernel): the distance to a
+//    point's BF16 copy, less the copy's distance from the point, bounds the
+//    point's distance from below, and only candidates whose bound does not
+//    exceed the list's last entry are scored, from the float32 rows and in the
+//    arithmetic above. The lists are the same. 10,000 queries, 3M x 384, T = 64,
+//    w = 50 (98 GB of float32 rows): 18.2 -> 11.1 ms, 12.3 with the copy's
+//    making; bound by the screen's instructions (about 12 per row and four
+//    coordinates), no longer by HBM.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math.h>
+
+#include <type_traits>
 
 #include "hf_internal.cuh"
 #include "hilbert_device.cuh"
@@ -99,13 +102,13 @@ struct SearchArgs {
   int k, w;
   uint32_t* out_idx;
   float* out_dist;
-  int64_t* out_pos;
-  int only_tree;
-  int pos_all;  // positions of every tree into out_pos[t * nq + query], no lists
+  int64_t* out_pos;  // locate_kernel: positions, of one tree [nq] or of all [T][nq]
+  int only_tree;     // locate_kernel: that tree, or -1 for all
   int vec4;  // d % 4 == 0 and both matrices 16-byte aligned
   int top;   // the K prefix words lie in the top bit level (d >= 64K)
-  // half-width screen, or null: the points in BF16 (row pitch dp) and an upper
-  // bound of each one's distance from its copy
+  // search16_kernel: positions [T][nq], the points in BF16 (row pitch dp) and an
+  // upper bound of each one's distance from its copy
+  const int64_t* pos;
   const __nv_bfloat16* x16;
   const float* r16;
   int dp;
@@ -167,6 +170,79 @@ __device__ __forceinline__ int64_t warp_bound(const uint64_t* __restrict__ pre, 
     }
   }
   return lo;
+}
+
+// Position of the query in tree t: the lower bound of its full key. qp: K words,
+// Yq, Yd: d bytes each, the warp's own.
+__device__ __forceinline__ int64_t warp_locate(const SearchArgs& a, int t, const uint8_t* __restrict__ qc,
+                                               uint64_t* qp, uint8_t* Yq, uint8_t* Yd, int lane) {
+  const int32_t* pi = a.pi + (size_t)t * a.d;
+  const uint32_t* rb = a.rbits + (size_t)t * a.W32;
+  const uint64_t* pre = a.prefix + (size_t)t * a.K * a.n;
+  const uint32_t* sig = a.sigma + (size_t)t * a.n;
+  if (a.top) {
+    warp_top_prefix(qc, a.bits, a.K, pi, rb, qp, lane);
+  } else if (lane == 0) {
+    hf_load_coords_codes(qc, a.d, a.bits, a.L, pi, rb, Yq);
+    hf_skilling(Yq, a.d, a.L);
+    for (int w = 0; w < a.K; ++w) qp[w] = hf_pack_word(Yq, a.d, a.L, w);
+  }
+  __syncwarp();
+  const int64_t lo = warp_bound(pre, a.n, a.K, qp, false, 0, lane);
+  int64_t pos = lo;
+  // [lo, lo2): positions whose prefix equals the query's
+  if (a.K < a.W && lo < a.n && cmp_prefix(pre, a.n, a.K, lo, qp) == 0) {
+    const int64_t lo2 = warp_bound(pre, a.n, a.K, qp, true, lo, lane);
+    if (lane == 0) {
+      // equal prefixes: lower bound by full key inside [lo, lo2)
+      hf_load_coords_codes(qc, a.d, a.bits, a.bits, pi, rb, Yq);
+      hf_skilling(Yq, a.d, a.bits);
+      int64_t l = lo, h = lo2;
+      while (l < h) {
+        const int64_t mid = (l + h) >> 1;
+        hf_load_coords_planes(a.planes, a.n, a.d, a.W32, a.bits, pi, rb, sig[mid], Yd);
+        hf_skilling(Yd, a.d, a.bits);
+        if (full_key_less(Yd, Yq, a.d, a.bits, a.W)) l = mid + 1;
+        else h = mid;
+      }
+      pos = l;
+    }
+    pos = __shfl_sync(FULL, pos, 0);
+  }
+  return pos;
+}
+
+// The warp's shared memory (search_per_warp).
+struct WarpScratch {
+  uint64_t* qp;
+  uint32_t* cpid;
+  uint8_t *Yq, *Yd;
+};
+__device__ __forceinline__ WarpScratch warp_scratch(unsigned char* base, int K, int d) {
+  WarpScratch w;
+  w.qp = reinterpret_cast<uint64_t*>(base);
+  w.cpid = reinterpret_cast<uint32_t*>(w.qp + K);
+  w.Yq = reinterpret_cast<uint8_t*>(w.cpid + 32);
+  w.Yd = w.Yq + d;
+  return w;
+}
+
+// Positions alone: warp (query, tp) takes trees tp, tp + tsplit, ..., or the one
+// tree asked for. Bound by latency (dependent probes of the prefixes, and for
+// equal prefixes one lane's keys), so by the warps an SM holds.
+__global__ void __launch_bounds__(SWARPS * 32) locate_kernel(SearchArgs a) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  const WarpScratch w = warp_scratch(smraw + search_per_warp(a.K, a.d) * wib, a.K, a.d);
+  const int64_t wi = (int64_t)blockIdx.x * SWARPS + wib;
+  const int64_t qi = wi / a.tsplit;
+  if (qi >= a.nq) return;
+  const bool one = a.only_tree >= 0;
+  const int t_end = one ? a.only_tree + 1 : a.T;
+  for (int t = one ? a.only_tree : (int)(wi - qi * a.tsplit); t < t_end; t += a.tsplit) {
+    const int64_t pos = warp_locate(a, t, a.qcodes + (size_t)qi * a.d, w.qp, w.Yq, w.Yd, lane);
+    if (lane == 0) a.out_pos[one ? (size_t)qi : (size_t)t * a.nq + qi] = pos;
+  }
 }
 
 // Bitonic sort of one (distance, index) pair per lane across the warp,
@@ -332,22 +408,18 @@ __global__ void prepare16_kernel(const float* __restrict__ x, int64_t n, int d, 
   }
 }
 
-// Float32 rows: six blocks an SM, 80 registers, 16 rows' loads in flight. Left to
-// itself the compiler took the same number and issued the loads one after the
-// other (hf_search_static, 10,000 queries, T = 32, w = 8 to 128, d = 64 to 384: a
+// Locates and scores: one warp per query, or per part of one.
+// Six blocks an SM: 80 registers, 16 rows' loads in flight. Left to itself the
+// compiler took the same number and issued the loads one after the other
+// (hf_search_static, 10,000 queries, T = 32, w = 8 to 128, d = 64 to 384: a
 // geometric mean of 12 % slower at k <= 32, 21 % at k = 64); five blocks (96
 // registers) are 9 % faster below 1,000 queries, 7 % slower from 10,000 on.
-template <int S, bool B16>
-__global__ void __launch_bounds__(SWARPS * 32, B16 ? 4 : 6) search_kernel(SearchArgs a) {
+template <int S>
+__global__ void __launch_bounds__(SWARPS * 32, 6) search_kernel(SearchArgs a) {
   extern __shared__ __align__(16) unsigned char smraw[];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const size_t per_warp = search_per_warp(a.K, a.d);
-  unsigned char* base = smraw + per_warp * wib;
-  uint64_t* qp = reinterpret_cast<uint64_t*>(base);
-  uint32_t* cpid = reinterpret_cast<uint32_t*>(qp + a.K);
-  uint8_t* Yq = reinterpret_cast<uint8_t*>(cpid + 32);
-  uint8_t* Yd = Yq + a.d;
-
+  const WarpScratch ws = warp_scratch(smraw + search_per_warp(a.K, a.d) * wib, a.K, a.d);
+  uint32_t* cpid = ws.cpid;
   const int parts = a.tsplit * a.csplit;
   const int64_t li = (int64_t)blockIdx.x * SWARPS + wib;  // this warp's list
   const int64_t qi = parts == 1 ? li : li / parts;
@@ -360,125 +432,15 @@ __global__ void __launch_bounds__(SWARPS * 32, B16 ? 4 : 6) search_kernel(Search
   WarpList<S> list;
   list.init();
 
-  const int t_begin = a.only_tree >= 0 ? a.only_tree : tp;
-  const int t_end = a.only_tree >= 0 ? a.only_tree + 1 : a.T;
-  for (int t = t_begin; t < t_end; t += a.tsplit) {
-    const int32_t* pi = a.pi + (size_t)t * a.d;
-    const uint32_t* rb = a.rbits + (size_t)t * a.W32;
-    const uint64_t* pre = a.prefix + (size_t)t * a.K * a.n;
+  for (int t = tp; t < a.T; t += a.tsplit) {
     const uint32_t* sig = a.sigma + (size_t)t * a.n;
-    if (a.top) {
-      warp_top_prefix(qc, a.bits, a.K, pi, rb, qp, lane);
-    } else if (lane == 0) {
-      hf_load_coords_codes(qc, a.d, a.bits, a.L, pi, rb, Yq);
-      hf_skilling(Yq, a.d, a.L);
-      for (int w = 0; w < a.K; ++w) qp[w] = hf_pack_word(Yq, a.d, a.L, w);
-    }
-    __syncwarp();
-    const int64_t lo = warp_bound(pre, a.n, a.K, qp, false, 0, lane);
-    int64_t pos = lo;
-    // [lo, lo2): positions whose prefix equals the query's
-    if (a.K < a.W && lo < a.n && cmp_prefix(pre, a.n, a.K, lo, qp) == 0) {
-      const int64_t lo2 = warp_bound(pre, a.n, a.K, qp, true, lo, lane);
-      if (lane == 0) {
-        // equal prefixes: lower bound by full key inside [lo, lo2)
-        hf_load_coords_codes(qc, a.d, a.bits, a.bits, pi, rb, Yq);
-        hf_skilling(Yq, a.d, a.bits);
-        int64_t l = lo, h = lo2;
-        while (l < h) {
-          const int64_t mid = (l + h) >> 1;
-          hf_load_coords_planes(a.planes, a.n, a.d, a.W32, a.bits, pi, rb, sig[mid], Yd);
-          hf_skilling(Yd, a.d, a.bits);
-          if (full_key_less(Yd, Yq, a.d, a.bits, a.W)) l = mid + 1;
-          else h = mid;
-        }
-        pos = l;
-      }
-      pos = __shfl_sync(FULL, pos, 0);
-    }
-    if (a.only_tree >= 0 || a.pos_all) {
-      if (lane == 0) a.out_pos[a.pos_all ? (size_t)t * a.nq + qi : (size_t)qi] = pos;
-      continue;
-    }
+    const int64_t pos = warp_locate(a, t, qc, ws.qp, ws.Yq, ws.Yd, lane);
     const int64_t c0 = pos - a.w > 0 ? pos - a.w : 0;
     const int64_t c1 = pos + a.w < a.n ? pos + a.w : a.n;
     for (int64_t cb = c0 + 32 * cp; cb < c1; cb += 32 * a.csplit) {
       const int64_t c = cb + lane;
       uint32_t pid = c < c1 ? __ldg(sig + c) : 0xffffffffu;
       float dist;
-      if (B16) {
-        cpid[lane] = pid;
-        const float res = pid != 0xffffffffu ? __ldg(a.r16 + pid) : 0.f;
-        __syncwarp();
-        const int cnt = (int)(c1 - cb < 32 ? c1 - cb : 32);
-        float part[32];
-        // 16 rows at a time (none for an empty half): their loads are issued
-        // before any is used (an empty slot reads row 0; its result is
-        // discarded), two coordinates to an instruction (f32x2), the even and
-        // the odd ones' sums apart until the end
-#pragma unroll
-        for (int u0 = 0; u0 < 32; u0 += 16) {
-          uint64_t acc[16];
-#pragma unroll
-          for (int u = 0; u < 16; ++u) acc[u] = 0;
-          if (u0 < cnt) {
-            for (int m = 4 * lane; m < a.d; m += 128) {
-              const ulonglong2 qa = __ldg(reinterpret_cast<const ulonglong2*>(qv + m));
-              uint2 xb[16];
-#pragma unroll
-              for (int u = 0; u < 16; ++u) {
-                const uint32_t p = cpid[u0 + u];
-                xb[u] = __ldg(reinterpret_cast<const uint2*>(a.x16 + (size_t)(p != 0xffffffffu ? p : 0u) * a.dp + m));
-              }
-#pragma unroll
-              for (int u = 0; u < 16; ++u) {
-                acc[u] = sq_diff2(qa.x, bf16_lo(xb[u].x), bf16_hi(xb[u].x), acc[u]);
-                acc[u] = sq_diff2(qa.y, bf16_lo(xb[u].y), bf16_hi(xb[u].y), acc[u]);
-              }
-            }
-          }
-#pragma unroll
-          for (int u = 0; u < 16; ++u) part[u0 + u] = pair_sum(acc[u]);
-        }
-        const float near = warp_transpose_sum(part, lane);
-        __syncwarp();
-        // |q - x| >= |q - copy| - |x - copy|; the sums are within 1e-5 of
-        // their values up to d = 4096, also the exact one. A sum that
-        // overflowed, or whose squares leave the float32 range, says nothing.
-        const float gap = sqrtf(near) * 0.99999f - res;
-        const float bound = gap > 1e-12f && near < 1e38f ? gap * gap * 0.99998f : 0.f;
-        float kd;
-        uint32_t ki;
-        list.last(a.k, kd, ki);
-        uint32_t todo = __ballot_sync(FULL, pid != 0xffffffffu && !(bound > kd));
-        while (todo) {
-          const int src = __ffs(todo) - 1;
-          todo &= todo - 1;
-          const uint32_t ci = __shfl_sync(FULL, pid, src);
-          if (__shfl_sync(FULL, bound, src) > kd || list.holds(ci, a.k, lane)) continue;
-          float cd = 0.f;
-          for (int m = 4 * lane; m < a.d; m += 128) {
-            const float4 qa = __ldg(reinterpret_cast<const float4*>(qv + m));
-            const float4 xv = __ldg(reinterpret_cast<const float4*>(a.x + (size_t)ci * a.d + m));
-            float e = qa.x - xv.x;
-            cd = fmaf(e, e, cd);
-            e = qa.y - xv.y;
-            cd = fmaf(e, e, cd);
-            e = qa.z - xv.z;
-            cd = fmaf(e, e, cd);
-            e = qa.w - xv.w;
-            cd = fmaf(e, e, cd);
-          }
-          // the lanes' partials in warp_transpose_sum's tree
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) cd += __shfl_xor_sync(FULL, cd, o);
-          if (lessp(cd, ci, kd, ki)) {
-            list.insert(cd, ci, a.k, lane);
-            list.last(a.k, kd, ki);
-          }
-        }
-        continue;
-      }
       if (a.vec4) {
         cpid[lane] = pid;
         __syncwarp();
@@ -540,7 +502,146 @@ __global__ void __launch_bounds__(SWARPS * 32, B16 ? 4 : 6) search_kernel(Search
       }
     }
   }
-  if (a.only_tree >= 0 || a.pos_all) return;
+#pragma unroll
+  for (int s = 0; s < S; ++s) {
+    const int e = 32 * s + lane;
+    if (e < a.k) {
+      a.out_idx[(size_t)li * a.k + e] = list.iv[s];
+      a.out_dist[(size_t)li * a.k + e] = list.dv[s];
+    }
+  }
+}
+
+// Scores through the half-width screen, the positions known (locate_kernel, in
+// a launch of its own: this kernel's registers leave an SM half of the warps
+// that hide the locate's latency, which cost batches with few rows per position,
+// 64 dimensions or near-duplicates 5 to 20 % of the whole search; 10,000 queries,
+// k = 30, both in one kernel and so: 3M x 384, T = 64, w = 50: 12.4, 11.1 ms; 1M
+// x 64, T = 64, w = 16: 6.4, 5.1; 300,000 x 384 near-duplicates, T = 64, w = 16:
+// 86.4, 57.1).
+template <int S>
+__global__ void __launch_bounds__(SWARPS * 32) search16_kernel(SearchArgs a) {
+  __shared__ uint32_t s_id[SWARPS][32];
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  uint32_t* cpid = s_id[wib];
+  const int parts = a.tsplit * a.csplit;
+  const int64_t li = (int64_t)blockIdx.x * SWARPS + wib;  // this warp's list
+  const int64_t qi = parts == 1 ? li : li / parts;
+  if (qi >= a.nq) return;
+  const int part = (int)(li - qi * parts);
+  const int tp = part / a.csplit, cp = part - tp * a.csplit;
+  const float* qv = a.q + (size_t)qi * a.d;
+
+  WarpList<S> list;
+  list.init();
+
+  int64_t next = tp < a.T ? __ldg(a.pos + (size_t)tp * a.nq + qi) : 0;
+  for (int t = tp; t < a.T; t += a.tsplit) {
+    const uint32_t* sig = a.sigma + (size_t)t * a.n;
+    const int64_t pos = next;
+    if (t + a.tsplit < a.T) next = __ldg(a.pos + (size_t)(t + a.tsplit) * a.nq + qi);
+    const int64_t c0 = pos - a.w > 0 ? pos - a.w : 0;
+    const int64_t c1 = pos + a.w < a.n ? pos + a.w : a.n;
+    for (int64_t cb = c0 + 32 * cp; cb < c1; cb += 32 * a.csplit) {
+      const int64_t c = cb + lane;
+      const uint32_t pid = c < c1 ? __ldg(sig + c) : 0xffffffffu;
+      cpid[lane] = pid;
+      const float res = pid != 0xffffffffu ? __ldg(a.r16 + pid) : 0.f;
+      __syncwarp();
+      const int cnt = (int)(c1 - cb < 32 ? c1 - cb : 32);
+      float part[32];
+      // 16 rows at a time (none for an empty half): their loads are issued
+      // before any is used (an empty slot reads row 0; its result is
+      // discarded), two coordinates to an instruction (f32x2), the even and
+      // the odd ones' sums apart until the end
+#pragma unroll
+      for (int u0 = 0; u0 < 32; u0 += 16) {
+        uint64_t acc[16];
+#pragma unroll
+        for (int u = 0; u < 16; ++u) acc[u] = 0;
+        if (u0 < cnt) {
+          for (int m = 4 * lane; m < a.d; m += 128) {
+            const ulonglong2 qa = __ldg(reinterpret_cast<const ulonglong2*>(qv + m));
+            uint2 xb[16];
+#pragma unroll
+            for (int u = 0; u < 16; ++u) {
+              const uint32_t p = cpid[u0 + u];
+              xb[u] = __ldg(reinterpret_cast<const uint2*>(a.x16 + (size_t)(p != 0xffffffffu ? p : 0u) * a.dp + m));
+            }
+#pragma unroll
+            for (int u = 0; u < 16; ++u) {
+              acc[u] = sq_diff2(qa.x, bf16_lo(xb[u].x), bf16_hi(xb[u].x), acc[u]);
+              acc[u] = sq_diff2(qa.y, bf16_lo(xb[u].y), bf16_hi(xb[u].y), acc[u]);
+            }
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < 16; ++u) part[u0 + u] = pair_sum(acc[u]);
+      }
+      const float near = warp_transpose_sum(part, lane);
+      __syncwarp();
+      // |q - x| >= |q - copy| - |x - copy|; the sums are within 1e-5 of
+      // their values up to d = 4096, also the exact one. A sum that
+      // overflowed, or whose squares leave the float32 range, says nothing.
+      const float gap = sqrtf(near) * 0.99999f - res;
+      const float bound = gap > 1e-12f && near < 1e38f ? gap * gap * 0.99998f : 0.f;
+      float kd;
+      uint32_t ki;
+      list.last(a.k, kd, ki);
+      uint32_t todo = __ballot_sync(FULL, pid != 0xffffffffu && !(bound > kd));
+      // scores the next NS survivors, their rows' loads in flight together
+      auto score = [&](auto count) {
+        constexpr int NS = decltype(count)::value;
+        uint32_t ci[NS];
+        float cd[NS];
+#pragma unroll
+        for (int u = 0; u < NS; ++u) {
+          const int src = todo ? __ffs(todo) - 1 : 0;
+          const bool some = todo != 0;
+          todo &= todo - 1;
+          const uint32_t id = __shfl_sync(FULL, pid, src);
+          const bool out = __shfl_sync(FULL, bound, src) > kd;
+          ci[u] = some && !out && !list.holds(id, a.k, lane) ? id : 0xffffffffu;
+          cd[u] = 0.f;
+        }
+        for (int m = 4 * lane; m < a.d; m += 128) {
+          const float4 qa = __ldg(reinterpret_cast<const float4*>(qv + m));
+          float4 xv[NS];
+#pragma unroll
+          for (int u = 0; u < NS; ++u)
+            xv[u] = ci[u] != 0xffffffffu ? __ldg(reinterpret_cast<const float4*>(a.x + (size_t)ci[u] * a.d + m)) : qa;
+#pragma unroll
+          for (int u = 0; u < NS; ++u) {
+            float e = qa.x - xv[u].x;
+            cd[u] = fmaf(e, e, cd[u]);
+            e = qa.y - xv[u].y;
+            cd[u] = fmaf(e, e, cd[u]);
+            e = qa.z - xv[u].z;
+            cd[u] = fmaf(e, e, cd[u]);
+            e = qa.w - xv[u].w;
+            cd[u] = fmaf(e, e, cd[u]);
+          }
+        }
+        // the lanes' partials in warp_transpose_sum's tree
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+          for (int u = 0; u < NS; ++u) cd[u] += __shfl_xor_sync(FULL, cd[u], o);
+#pragma unroll
+        for (int u = 0; u < NS; ++u)
+          if (ci[u] != 0xffffffffu && lessp(cd[u], ci[u], kd, ki)) {
+            list.insert(cd[u], ci[u], a.k, lane);
+            list.last(a.k, kd, ki);
+          }
+      };
+      // one at a time once they are few: the list's last distance, which each may
+      // lower, spares the next one its row
+      while (todo) {
+        if (__popc(todo) >= 3) score(std::integral_constant<int, 4>{});
+        else score(std::integral_constant<int, 1>{});
+      }
+    }
+  }
 #pragma unroll
   for (int s = 0; s < S; ++s) {
     const int e = 32 * s + lane;
@@ -605,13 +706,28 @@ merge_parts_kernel(const uint32_t* __restrict__ pidx, const float* __restrict__ 
   }
 }
 
-template <int S, bool B16>
+template <int S>
 int launch_s(const SearchArgs& a, size_t smem, cudaStream_t s) {
-  if (smem > 48 * 1024 && cudaFuncSetAttribute((const void*)search_kernel<S, B16>,
+  const unsigned blocks = hf_blocks(a.nq * a.tsplit * a.csplit, SWARPS);
+  if (a.pos) {
+    search16_kernel<S><<<blocks, SWARPS * 32, 0, s>>>(a);
+    hf_after_launch("search16_kernel", s);
+    return HF_OK;
+  }
+  if (smem > 48 * 1024 && cudaFuncSetAttribute((const void*)search_kernel<S>,
                                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return HF_ECUDA;
-  search_kernel<S, B16><<<hf_blocks(a.nq * a.tsplit * a.csplit, SWARPS), SWARPS * 32, smem, s>>>(a);
+  search_kernel<S><<<blocks, SWARPS * 32, smem, s>>>(a);
   hf_after_launch("search_kernel", s);
+  return HF_OK;
+}
+
+int launch_locate(const SearchArgs& a, size_t smem, cudaStream_t s) {
+  if (smem > 48 * 1024 && cudaFuncSetAttribute((const void*)locate_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)smem) != cudaSuccess)
+    return HF_ECUDA;
+  locate_kernel<<<hf_blocks(a.nq * a.tsplit, SWARPS), SWARPS * 32, smem, s>>>(a);
+  hf_after_launch("locate_kernel", s);
   return HF_OK;
 }
 
@@ -654,11 +770,10 @@ int64_t search_parts(const hf_forest* f, int64_t nq, int w) {
   return (int64_t)ts * cs;
 }
 
-int launch_search(const hf_forest* f, const float* q, const uint8_t* qcodes, int64_t nq, int k, int w,
-                  uint32_t* out_idx, float* out_dist, int64_t* out_pos, int only_tree, cudaStream_t s,
-                  uint32_t* part_idx, float* part_dist, bool use16) {
-  if (k < 1 || k > 64) return HF_EINVAL;
-  SearchArgs a;
+namespace {
+
+SearchArgs search_args(const hf_forest* f, const float* q, const uint8_t* qcodes, int64_t nq, int k, int w) {
+  SearchArgs a{};
   a.x = f->x;
   a.n = f->n;
   a.d = f->d;
@@ -678,39 +793,71 @@ int launch_search(const hf_forest* f, const float* q, const uint8_t* qcodes, int
   a.nq = nq;
   a.k = k;
   a.w = w;
-  a.out_idx = out_idx;
-  a.out_dist = out_dist;
-  a.out_pos = out_pos;
-  a.only_tree = only_tree >= 0 ? only_tree : -1;
-  a.pos_all = only_tree == -2;
-  if (a.pos_all && !out_pos) return HF_EINVAL;
+  a.only_tree = -1;
   a.vec4 = (f->d % 4 == 0) && ((reinterpret_cast<uintptr_t>(f->x) & 15) == 0) &&
            ((reinterpret_cast<uintptr_t>(q) & 15) == 0);
   a.top = f->d >= 64 * f->K;
+  a.dp = (f->d + 63) / 64 * 64;
   a.tsplit = a.csplit = 1;
-  if (a.pos_all) {
-    // positions only: trees are independent, nothing to merge
+  return a;
+}
+
+}  // namespace
+
+int launch_positions(const hf_forest* f, const float* q, const uint8_t* qcodes, int64_t nq, int tree, int64_t* out_pos,
+                     cudaStream_t s) {
+  SearchArgs a = search_args(f, q, qcodes, nq, 1, 1);
+  a.out_pos = out_pos;
+  a.only_tree = tree;
+  if (tree < 0) {
+    // trees are independent, nothing to merge
     int cs;
     search_split(nq, f->T, 1, &a.tsplit, &cs);
-  } else if (a.only_tree < 0 && part_idx) {
-    search_split(nq, f->T, w, &a.tsplit, &a.csplit);
   }
-  const bool parts = !a.pos_all && a.tsplit * a.csplit > 1;
-  if (parts) {
-    a.out_idx = part_idx;
-    a.out_dist = part_dist;
-  }
-  const size_t smem = search_per_warp(f->K, f->d) * SWARPS;
-  const bool b16 = a.vec4 && f->x16 && use16 && !a.pos_all && a.only_tree < 0;
-  a.x16 = b16 ? static_cast<const __nv_bfloat16*>(f->x16) : nullptr;
-  a.r16 = f->r16;
-  a.dp = (f->d + 63) / 64 * 64;
-  const int rc = b16 ? (k <= 32 ? launch_s<1, true>(a, smem, s) : launch_s<2, true>(a, smem, s))
-                     : (k <= 32 ? launch_s<1, false>(a, smem, s) : launch_s<2, false>(a, smem, s));
+  const int rc = launch_locate(a, search_per_warp(f->K, f->d) * SWARPS, s);
   if (rc != HF_OK) return rc;
-  if (parts) {
-    if (k <= 32) launch_merge<1>(a, out_idx, out_dist, s);
-    else launch_merge<2>(a, out_idx, out_dist, s);
+  return cudaGetLastError() == cudaSuccess ? HF_OK : HF_ECUDA;
+}
+
+int64_t search16_slice(int64_t nq, int T) {
+  int64_t slice = ((int64_t)64 << 20) / (8 * (int64_t)T);
+  if (slice < 2048) slice = 2048;
+  return slice < nq ? slice : nq;
+}
+
+int launch_search(const hf_forest* f, const float* q, const uint8_t* qcodes, int64_t nq, int k, int w,
+                  uint32_t* out_idx, float* out_dist, cudaStream_t s, uint32_t* part_idx, float* part_dist,
+                  int64_t* pos16) {
+  if (k < 1 || k > 64) return HF_EINVAL;
+  const size_t smem = search_per_warp(f->K, f->d) * SWARPS;
+  const int64_t slice = pos16 ? search16_slice(nq, f->T) : nq;
+  for (int64_t q0 = 0; q0 < nq; q0 += slice) {
+    const int64_t m = nq - q0 < slice ? nq - q0 : slice;
+    SearchArgs a = search_args(f, q + (size_t)q0 * f->d, qcodes + (size_t)q0 * f->d, m, k, w);
+    uint32_t* oi = a.out_idx = out_idx + (size_t)q0 * k;
+    float* od = a.out_dist = out_dist + (size_t)q0 * k;
+    int rc = HF_OK;
+    if (pos16 && a.vec4 && f->x16) {
+      a.out_pos = pos16;
+      a.tsplit = f->T;
+      rc = launch_locate(a, smem, s);
+      a.tsplit = 1;
+      a.pos = pos16;
+      a.x16 = static_cast<const __nv_bfloat16*>(f->x16);
+      a.r16 = f->r16;
+    }
+    if (part_idx) search_split(m, f->T, w, &a.tsplit, &a.csplit);
+    const bool parts = a.tsplit * a.csplit > 1;
+    if (parts) {
+      a.out_idx = part_idx;
+      a.out_dist = part_dist;
+    }
+    if (rc == HF_OK) rc = k <= 32 ? launch_s<1>(a, smem, s) : launch_s<2>(a, smem, s);
+    if (rc != HF_OK) return rc;
+    if (parts) {
+      if (k <= 32) launch_merge<1>(a, oi, od, s);
+      else launch_merge<2>(a, oi, od, s);
+    }
   }
   return cudaGetLastError() == cudaSuccess ? HF_OK : HF_ECUDA;
 }
@@ -1154,7 +1301,7 @@ extern "C" int hf_search_static(hf_forest* f, const float* queries, int64_t nq, 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   cudaGetLastError();  // an earlier call's error was reported by that call
   launch_quantize_codes(queries, nq, f->d, f->lo, f->scale, f->bits, qc, f->err, s);
-  rc = launch_search(f, queries, qc, nq, k, w, reinterpret_cast<uint32_t*>(out_idx), out_dist, nullptr, -1, s);
+  rc = launch_search(f, queries, qc, nq, k, w, reinterpret_cast<uint32_t*>(out_idx), out_dist, s);
   // the same synchronisation and status mapping as every other entry point
   const int rc2 = hf_finish(f, s);
   return rc != HF_OK ? rc : rc2;
