@@ -136,7 +136,6 @@ __global__ void __launch_bounds__(1024) sort_plan_kernel(const uint64_t* __restr
   const uint64_t* word = pk + blockIdx.x * pk_ts;
   const int tid = threadIdx.x;
   const int S = n < PLAN_S ? (int)n : PLAN_S;
-  const int64_t stride = n / S;
   // bitonic sort of element e * 1024 + tid in register e, padded with the
   // largest word: partners less than 32 apart by shuffles
   uint64_t v[E];
@@ -144,7 +143,8 @@ __global__ void __launch_bounds__(1024) sort_plan_kernel(const uint64_t* __restr
   for (int e = 0; e < E; ++e) {
     const int j = e * 1024 + tid;
     const uint32_t h = (uint32_t)j * 0x9E3779B1u;
-    v[e] = j < S ? __ldg(word + (int64_t)j * stride + (int64_t)((h >> 8) % (uint64_t)stride)) : ~0ull;
+    const int64_t a = n * j / S, b = n * (j + 1) / S;  // this sample's share of the points
+    v[e] = j < S ? __ldg(word + a + (int64_t)((h >> 8) % (uint64_t)(b - a))) : ~0ull;
   }
   if (tid < PLAN_LEVELS) pairs[tid] = longest[tid] = 0;
 #pragma unroll 1
