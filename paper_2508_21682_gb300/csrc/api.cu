@@ -46,6 +46,7 @@ int classify(const void* p) {
 // most) cached between calls; hf_trim_pool returns it.
 std::mutex g_pool_mu;
 cudaMemPool_t g_pools[64] = {};
+std::atomic<uint32_t> g_trims{1};  // counts hf_trim_pool calls
 
 cudaMemPool_t device_pool() {
   int dev = 0;
@@ -66,6 +67,23 @@ cudaMemPool_t device_pool() {
     g_pools[dev] = pool;
   }
   return g_pools[dev];
+}
+
+// Memory that an allocation can have: what the device has free and what the
+// library's pool holds without using it.
+size_t free_bytes() {
+  size_t fr = 0, tot = 0;
+  if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  uint64_t held = 0, used = 0;
+  cudaMemPool_t pool = device_pool();
+  if (pool && cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &held) == cudaSuccess &&
+      cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess && held > used)
+    fr += held - used;
+  cudaGetLastError();
+  return fr;
 }
 
 }  // namespace
@@ -533,6 +551,7 @@ int hf_free(hf_forest* f) {
 int hf_trim_pool(void) {
   cudaMemPool_t pool = device_pool();
   if (!pool) return HF_ECUDA;
+  g_trims.fetch_add(1, std::memory_order_relaxed);
   if (cudaDeviceSynchronize() != cudaSuccess || cudaMemPoolTrimTo(pool, 0) != cudaSuccess) {
     cudaGetLastError();
     return HF_ECUDA;
@@ -1217,9 +1236,9 @@ static int sketch_search(hf_forest* f, const float* q, const uint8_t* qc, int64_
 // (search.cu), which the first search that reads enough rows makes: copying
 // costs 1.5 reads of the matrix and saves half of every row scored, so four
 // rows scored per point pay for it within the same call. Where the copy would
-// take more than a quarter of the free memory, or rows are not 16-byte aligned,
-// the search reads the float32 rows as before. 10,000 queries, 3M x 384, T = 64,
-// w = 50: 21 rows per point.
+// take more than a quarter of the free memory (the pool's idle part counted in),
+// or rows are not 16-byte aligned, the search reads the float32 rows as before.
+// 10,000 queries, 3M x 384, T = 64, w = 50: 21 rows per point.
 // Lists of more than 32 keep candidates that pass the screen coming for longer,
 // and each is scored on its own: from 6,500 k / d rows per query on the screen
 // has made up for them (10,000 queries, 2M points, T = 32, k = 64, with and
@@ -1233,12 +1252,15 @@ static bool search_uses16(hf_forest* f, const float* q, int64_t nq, int k, int w
   if (k > 32 && per_query * f->d < 6500.0 * k) return false;
   std::lock_guard<std::mutex> lock(f->x16_mu);
   if (f->x16) return true;
+  // a copy that found no room is not asked for again (the question is a slow
+  // call) until the pool has been trimmed
+  const uint32_t trims = g_trims.load(std::memory_order_relaxed);
+  if (f->x16_refused == trims) return false;
   void* x16 = nullptr;
   float* r16 = nullptr;
   const size_t bytes = (size_t)f->n * ((f->d + 63) / 64 * 64) * 2;
-  size_t fr = 0, tot = 0;
-  if (cudaMemGetInfo(&fr, &tot) != cudaSuccess || bytes > fr / 4) {
-    cudaGetLastError();
+  if (bytes > free_bytes() / 4) {
+    f->x16_refused = trims;
     return false;
   }
   cudaError_t e = dalloc_bytes(&x16, bytes, s);
@@ -1251,6 +1273,7 @@ static bool search_uses16(hf_forest* f, const float* q, int64_t nq, int k, int w
     cudaGetLastError();
     dfree(x16, s);
     dfree(r16, s);
+    f->x16_refused = trims;
     return false;
   }
   f->r16 = r16;

@@ -84,6 +84,7 @@ struct hf_forest {
   std::mutex x16_mu;
   void* x16 = nullptr;
   float* r16 = nullptr;
+  uint32_t x16_refused = 0;   // hf_trim_pool calls there had been when the copy found no room, or 0
   float* xm = nullptr;        // master-ordered points (n x d), built on demand
   uint32_t* posm = nullptr;   // inverse of the master order
 
