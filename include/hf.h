@@ -212,8 +212,8 @@ int hf_build_segmented(const float* points, const int64_t* offsets, int32_t nset
  * mode 0, 1 or 2 when hf_graph_plan runs; a window the form cannot run is
  * HF_ENOTIMPL, never a change of form). hf_graph_plan keeps per-point lists
  * (and, for the Gram forms, the operand copies) in the forest for (k, w) and
- * the plain pair kernel's block size `threads` (0: chosen, else 256, for
- * windows up to 480, or 512). hf_knn_graph_enqueue then enqueues the whole graph on
+ * the plain pair kernel's block size `threads` (256 or 512; 0: 256).
+ * hf_knn_graph_enqueue then enqueues the whole graph on
  * `stream` into DEVICE outputs (n x k) without allocating or synchronising,
  * so it can be captured; errors surface through hf_status, which synchronises
  * `stream` and reads and clears the device error word. The plan's buffers stay

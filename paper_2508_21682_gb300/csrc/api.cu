@@ -1069,7 +1069,7 @@ int hf_autotune(hf_forest* f, int32_t k, double target_recall, int32_t sample, i
       if (hf_graph_plan(f, k, ladder[pick], nt, stream) != HF_OK) continue;
       float ms = 0.f;
       if (time_plan(&ms) != HF_OK) {
-        cudaGetLastError();  // a block size whose blocks cannot hold 32 positions is skipped
+        cudaGetLastError();  // a variant that cannot be run is skipped
         continue;
       }
       // a form that reaches the target beats one that does not; then time

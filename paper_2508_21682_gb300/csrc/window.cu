@@ -357,8 +357,10 @@ int launch_pairs(PairArgs a, int dlo, int ytiles, int64_t cols, cudaStream_t s) 
 
 // Offsets 1 .. w in tiles of 64 (256 rows; the fewest staged rows per pair),
 // the rest in tiles of 32 (512 rows) and 16 (512 rows of 128 threads), so that
-// at most 15 offsets are computed beyond w. nt = 512: 64-offset tiles of 512
-// rows, one block per SM.
+// at most 15 offsets are computed beyond w. nt = 512, for plans that ask for it
+// (the tuner tries both): 64-offset tiles of 512 rows, one block per SM; at
+// windows from 64 to 704 between 3 % faster (20,000 x 384, w = 128) and 12 %
+// slower (100,003 x 100, w = 64) than nt = 256, 50 % on 20,000 x 384 at w = 64.
 template <bool HAM>
 int launch_band(const PairArgs& a, int64_t cols, int nt, cudaStream_t s) {
   int full = a.w / 64, rest = a.w % 64;
@@ -431,7 +433,6 @@ int launch_window_graph(const float* x, int64_t n, int d, const uint32_t* sigma,
                         uint32_t* list_idx, float* list_dist, float* band, cudaStream_t s, const uint32_t* segr,
                         const int64_t* segoff, int nt) {
   if (nt != 0 && nt != 256 && nt != 512) return HF_EINVAL;
-  if (nt == 256 && w > 480) return HF_ENOTIMPL;  // widest window a plan may ask of this block size
   return launch_tree<false>(x, n, d, sigma, w, kp, list_idx, list_dist, band, s, segr, segoff, nt);
 }
 

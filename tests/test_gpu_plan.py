@@ -51,3 +51,19 @@ def test_replay_after_another_plan(n, later):
             o.close()
         for _, graph in graphs:
             graph.close()
+
+
+@pytest.mark.parametrize("w", [480, 481, 520, 704])
+@pytest.mark.parametrize("threads", [0, 256, 512])
+def test_block_sizes_at_wide_windows(threads, w):
+    """Every block size that a plan accepts runs at every window of the form."""
+    import torch
+    import paper_2508_21682_gb300 as hf
+    x = torch.from_numpy(S.gaussian_mixture(3000, 24, n_components=20, seed=3)).cuda()
+    with hf.build(x, T=2, bits=8, seed=5) as G:
+        ri, rd = G.knn_graph(10, w)
+        oi, od = torch.empty_like(ri), torch.empty_like(rd)
+        G.graph_plan(10, w, threads)
+        G.knn_graph_enqueue(oi, od)
+        G.status()
+        assert torch.equal(ri, oi) and torch.equal(rd, od)
