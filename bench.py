@@ -472,19 +472,29 @@ def keys_sort_hbm(a, ph):
     Algorithmic bytes per point and tree: keys read the permuted top bits of
     the point (d / 8 bytes of the bit-sliced top plane when the K-word prefix
     lies in the top bit level, d * L / 8 bytes of planes otherwise) and write
-    K 64-bit words; the sort is priced at 8 K passes of 8-bit digits, each
-    reading and writing one 64-bit key word and one 32-bit index per point
-    (24 bytes), also where its plan leaves low digits out."""
+    K 64-bit words. The sort reads the K words for its histograms (8 K bytes),
+    makes the passes that its plan keeps (sort_passes of the timings; each reads
+    and writes one 64-bit key word and one 32-bit index, 24 bytes), reads the
+    first word of the partial order to refine it where passes were left out (8),
+    and gathers the words that were not sorted last (4 bytes of index and 16 a
+    word: K - 1 words, K where the first one was not sorted by all its digits).
+    all_digits is the rate at which the work of all 8 K passes was done, whatever
+    the plan left out: no share of the bandwidth."""
     K = min(2, -(-a.d * a.bits // 64))
     L = min(a.bits, -(-64 * K // a.d))
+    passes = ph.get("sort_passes") or 8.0 * K
+    left_out = passes < 8 * K
     kb = a.n * a.T * (a.d * L / 8 + 8 * K)
-    sb = a.n * a.T * 8 * K * 24
+    words = K - 1 + (1 if passes < 8 else 0)
+    sb = a.n * a.T * (8 * K + 24 * passes + (8 if left_out else 0) + (4 + 16 * words if words else 0))
     peaks, src = measured_peaks()
     peak = float(peaks["hbm_gbs"])
     out = {"peak": peak, "unit": "GB/s", "peak_note": f"hbm_gbs {src} (MEASURED_PEAKS.json)"}
     for name, b, ms in (("keys", kb, ph["keys"]), ("sort", sb, ph["sort"])):
         ach = b / (ms * 1e-3) / 1e9 if ms > 0 else None
         out[name] = {"bytes": b, "ms": ms, "achieved": ach, "frac": ach / peak if ach else None}
+    out["sort"]["passes_per_tree"] = passes
+    out["sort"]["all_digits"] = a.n * a.T * 8 * K * 24 / (ph["sort"] * 1e-3) / 1e9 if ph["sort"] > 0 else None
     return out
 
 

@@ -449,7 +449,8 @@ int hf_set_option(hf_forest* f, const char* key, int64_t value);
  * it fell back, [9] the time spent gathering each tree's rows into its
  * order (tensor forms; on a second stream, overlapping the previous tree's
  * Gram band, so it is not a part of [4]), [10] the Gram band launches alone
- * (tensor forms), [11] reserved (0). Writes min(cap, 12).
+ * (tensor forms), [11] digit passes per tree that the last build's sort ran (a
+ * mean; at most 8 per sorted key word). Writes min(cap, 12).
  */
 int hf_get_timings(const hf_forest* f, float* out_ms, int32_t cap);
 

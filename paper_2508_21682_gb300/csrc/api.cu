@@ -425,7 +425,9 @@ static int build_impl(const float* points, int64_t n, int32_t d, int32_t T, int3
   keep.add(&f->pi, (size_t)T * (d + W32));  // the reflection masks behind the axes: one upload
   keep.add(&f->prefix, (size_t)T * K * n);
   keep.add(&f->sigma, (size_t)T * n);
-  keep.add(&f->err, 4 + (size_t)T * 4);  // the tie counters behind the error word: one read
+  // the tie counters and each tree's first sort pass behind the error word: one read
+  const size_t read_words = 4 + (size_t)T * 5;
+  keep.add(&f->err, read_words);
   tmp.add(&f->pk, (size_t)TB * f->K2 * n);
   const bool sliced = prefix_top_path(d, f->K2, f->L);
   if (sliced) tmp.add(&f->p0t, (size_t)((n + 31) / 32) * d);
@@ -450,9 +452,10 @@ static int build_impl(const float* points, int64_t n, int32_t d, int32_t T, int3
   }
   f->rbits = reinterpret_cast<uint32_t*>(f->pi) + (size_t)T * d;
   f->tie.counters = reinterpret_cast<uint32_t*>(f->err) + 4;
+  f->sort.first = f->tie.counters + (size_t)T * 4;
   f->sort.hist = f->sort.skip + skip_words;
   f->sort.status = f->sort.hist + hist_words;
-  cudaMemsetAsync(f->err, 0, (4 + (size_t)T * 4) * sizeof(uint32_t), s);
+  cudaMemsetAsync(f->err, 0, read_words * sizeof(uint32_t), s);
   if (nseg > 1) {
     cudaMemcpyAsync(f->seg_off, f->seg_off_h.data(), (size_t)(nseg + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s);
     launch_seg_of_row(f->seg_off, nseg, n, f->seg, seg64, s);
@@ -489,8 +492,7 @@ static int build_impl(const float* points, int64_t n, int32_t d, int32_t T, int3
     tm.span(1, k0, k1);
     tm.span(2, k1, k2);
   }
-  // the error word and the tie counters in one read
-  std::vector<uint32_t> ctr(4 + (size_t)T * 4);
+  std::vector<uint32_t> ctr(read_words);
   if (rc == HF_OK) rc = finish(f, s, ctr.data(), ctr.size());
   // runs of equal prefixes longer than the on-device cap
   if (rc == HF_OK) {
@@ -516,6 +518,9 @@ static int build_impl(const float* points, int64_t n, int32_t d, int32_t T, int3
     // keys, histogram, scan, 8K passes, prefix gather and tie kernels per batch
     const int nb = (T + TB - 1) / TB;
     f->timings[6] = (float)(nb * (4 + 8 * K + (K <= 2 ? 3 : 0) + (K < f->W ? 3 : 0)));
+    double skipped = 0.0;
+    for (int t = 0; t < T; ++t) skipped += ctr[4 + (size_t)T * 4 + t];
+    f->timings[11] = (float)(8 * K - skipped / T);
   }
   free_build_scratch(f, s);
   if (rc != HF_OK) {

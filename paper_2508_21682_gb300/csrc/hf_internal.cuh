@@ -37,6 +37,7 @@ struct SortScratch {  // for a batch of TB trees
   uint32_t* hist = nullptr;    // [TB][K*8][256] digit counts -> exclusive offsets
   uint32_t* skip = nullptr;    // [TB + 1] first pass of each tree, 255 less the least of them (0: none);
                                // hist and status follow in the same run of words
+  uint32_t* first = nullptr;   // [T] first pass of each tree, for the host (behind the error word)
 };
 
 struct TieScratch {

@@ -128,7 +128,8 @@ constexpr int PLAN_LEVELS = 5;
 
 template <int PLAN_S>
 __global__ void __launch_bounds__(1024) sort_plan_kernel(const uint64_t* __restrict__ pk, int64_t pk_ts, int64_t n,
-                                                         int K, int TB, uint32_t* __restrict__ skip) {
+                                                         int K, int TB, uint32_t* __restrict__ skip,
+                                                         uint32_t* __restrict__ first) {
   constexpr int E = PLAN_S / 1024;
   __shared__ uint64_t s[PLAN_S];
   __shared__ unsigned long long pairs[PLAN_LEVELS];
@@ -212,7 +213,7 @@ __global__ void __launch_bounds__(1024) sort_plan_kernel(const uint64_t* __restr
         s0 = st;
       }
     }
-    skip[blockIdx.x] = s0;
+    skip[blockIdx.x] = first[blockIdx.x] = s0;
     atomicMax(&skip[TB], 255u - s0);
   }
 }
@@ -1151,9 +1152,9 @@ int sort_batch(hf_forest* f, int t0, int tb, cudaStream_t s) {
   uint32_t* skip = f->sort.skip;
   if (K <= 2 && !f->test_stall) {
     if (n >= PLAN_LARGE)
-      sort_plan_kernel<4096><<<(unsigned)tb, 1024, 0, s>>>(f->pk, pk_ts, n, K, tb, skip);
+      sort_plan_kernel<4096><<<(unsigned)tb, 1024, 0, s>>>(f->pk, pk_ts, n, K, tb, skip, f->sort.first + t0);
     else
-      sort_plan_kernel<1024><<<(unsigned)tb, 1024, 0, s>>>(f->pk, pk_ts, n, K, tb, skip);
+      sort_plan_kernel<1024><<<(unsigned)tb, 1024, 0, s>>>(f->pk, pk_ts, n, K, tb, skip, f->sort.first + t0);
     hf_after_launch("sort_plan_kernel", s);
   }
 
