@@ -16,6 +16,7 @@
 size_t sort_status_words(int64_t n, int K, int tb);
 int tie_big_min(int W);
 size_t tie_scratch_words(int W);
+int tie_launches(const hf_forest* f);
 
 namespace {
 
@@ -515,9 +516,10 @@ static int build_impl(const float* points, int64_t n, int32_t d, int32_t T, int3
   }
   if (rc == HF_OK) {
     tm.collect({0, 1, 2, 3});
-    // keys, histogram, scan, 8K passes, prefix gather and tie kernels per batch
+    // keys, histogram, scan, 8K passes, prefix gather, plan, refining and tie
+    // kernels per batch
     const int nb = (T + TB - 1) / TB;
-    f->timings[6] = (float)(nb * (4 + 8 * K + (K <= 2 ? 3 : 0) + (K < f->W ? 3 : 0)));
+    f->timings[6] = (float)(nb * (4 + 8 * K + (K <= 2 ? 3 : 0) + tie_launches(f)));
     double skipped = 0.0;
     for (int t = 0; t < T; ++t) skipped += ctr[4 + (size_t)T * 4 + t];
     f->timings[11] = (float)(8 * K - skipped / T);

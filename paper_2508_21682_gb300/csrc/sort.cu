@@ -1392,6 +1392,14 @@ int tie_fixup_big(hf_forest* f, int t, uint32_t nbig, cudaStream_t s) {
 // Words of the sub-runs' full-key scratch.
 size_t tie_scratch_words(int W) { return (size_t)TIE_BLOCKS * tie_hard_cap(W) * W; }
 
+// Launches of the fix-up per batch (sort_batch's own conditions).
+int tie_launches(const hf_forest* f) {
+  if (f->K >= f->W) return 0;
+  const bool words = f->K2 == f->K && f->d < 64 * (f->K + 1);
+  const bool hard = (f->K2 > f->K + 1 ? f->K2 : f->K + 1) < f->W;
+  return 2 + (words ? 1 : 0) + (hard ? 1 : 0);
+}
+
 // Runs and sub-runs on the big list are longer than this.
 int tie_big_min(int W) { return tie_hard_cap(W); }
 
