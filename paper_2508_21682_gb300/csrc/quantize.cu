@@ -279,87 +279,99 @@ __device__ __forceinline__ float rank_float(uint32_t r) {
   return __uint_as_float((r & 0x80000000u) ? r & 0x7fffffffu : ~r);
 }
 
-// Range of every set of a segmented matrix. Block (row chunk, column chunk): a
+// Range of every set of a segmented matrix. Block (row range, column chunk): a
 // warp takes 32 / cg rows at a time, cg lanes of VEC consecutive columns each
-// (16-byte loads when VEC = 4), four rows per lane in flight; the chunk's part
-// of each set is reduced over the block's warps and folded into the set's
-// running range (kept as float_rank values in lo / scale) by atomics. The row
-// chunks cut the matrix evenly whatever the sets' sizes: one block per set and
-// 32 columns left a 200,000-row set to 8 warps (1.2M x 128 in 23 sets: 3.35
-// ms; the segmented build + graph went from 19.5 to 16.6 ms with this split).
-// Bound by HBM: the points are read once.
+// (16-byte loads when VEC = 4), four rows per lane in flight; the range's minima
+// and maxima are reduced over the block's warps and folded into its set's
+// running range (kept as float_rank values in lo / scale) by atomics. The first
+// rpb rows of every set are a block's, and every chunk of rpb rows of the matrix
+// is another's, for what it holds past the first rpb rows of the set it starts
+// in: each block has rows of one set, whatever the sets' sizes. One block per
+// set and 32 columns left a 200,000-row set to 8 warps (1.2M x 128 in 23 sets:
+// 3.35 ms; the segmented build + graph went from 19.5 to 16.6 ms with an even
+// split), and chunks alone, their sets one after the other, took 0.32 ms for 256
+// sets of 2 x 16 (SMALL_SETS). Bound by HBM: the points are read once.
 constexpr int SR_WARPS = 8;
 template <int VEC>
 __global__ void __launch_bounds__(SR_WARPS * 32)
-seg_range_kernel(const float* __restrict__ x, int64_t n, int d, const int64_t* __restrict__ off,
-                 const uint32_t* __restrict__ seg, int64_t rows_per_block, int cg, uint32_t* __restrict__ lo,
+seg_range_kernel(const float* __restrict__ x, int64_t n, int d, const int64_t* __restrict__ off, int nseg,
+                 const uint32_t* __restrict__ seg, int64_t rpb, int cg, uint32_t* __restrict__ lo,
                  uint32_t* __restrict__ hi, int* __restrict__ err) {
   __shared__ float smn[SR_WARPS][32 * VEC], smx[SR_WARPS][32 * VEC];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int c0 = (int)blockIdx.y * cg * VEC;             // first column of the block
   const int c = c0 + (lane % cg) * VEC, sub = lane / cg;  // this lane's columns and row within the warp's group
   const int rstep = SR_WARPS * (32 / cg);
-  const int64_t r0 = (int64_t)blockIdx.x * rows_per_block;
-  const int64_t r1 = r0 + rows_per_block < n ? r0 + rows_per_block : n;
+  // rows [a, b) of one set
+  uint32_t set;
+  int64_t a, b;
+  if ((int)blockIdx.x < nseg) {
+    set = blockIdx.x;
+    a = __ldg(off + set);
+    b = a + rpb;
+  } else {
+    const int64_t r0 = (int64_t)(blockIdx.x - nseg) * rpb;
+    set = __ldg(seg + r0);
+    a = __ldg(off + set) + rpb;
+    if (a < r0) a = r0;
+    b = r0 + rpb;
+  }
+  const int64_t end = __ldg(off + set + 1);
+  if (b > end) b = end;
+  if (a >= b) return;
   bool bad = false;
-  for (int64_t a = r0; a < r1;) {  // one set's part of the chunk at a time
-    const uint32_t set = __ldg(seg + a);
-    const int64_t e = __ldg(off + set + 1), b = e < r1 ? e : r1;
-    float mn[VEC], mx[VEC];
+  float mn[VEC], mx[VEC];
+#pragma unroll
+  for (int v = 0; v < VEC; ++v) {
+    mn[v] = INFINITY;
+    mx[v] = -INFINITY;
+  }
+  auto take = [&](const float* q) {
 #pragma unroll
     for (int v = 0; v < VEC; ++v) {
-      mn[v] = INFINITY;
-      mx[v] = -INFINITY;
+      bad |= !isfinite(q[v]);
+      mn[v] = fminf(mn[v], q[v]);
+      mx[v] = fmaxf(mx[v], q[v]);
     }
-    auto take = [&](const float* q) {
+  };
+  if (c < d) {
+    int64_t r = a + warp * (32 / cg) + sub;
+    constexpr int UN = 4;
+    for (; r + (UN - 1) * rstep < b; r += UN * rstep) {
+      float q[UN][VEC];
 #pragma unroll
-      for (int v = 0; v < VEC; ++v) {
-        bad |= !isfinite(q[v]);
-        mn[v] = fminf(mn[v], q[v]);
-        mx[v] = fmaxf(mx[v], q[v]);
+      for (int u = 0; u < UN; ++u) {
+        const float* src = x + (size_t)(r + u * rstep) * d + c;
+        if (VEC == 4) *reinterpret_cast<float4*>(q[u]) = __ldg(reinterpret_cast<const float4*>(src));
+        else q[u][0] = __ldg(src);
       }
-    };
-    if (c < d) {
-      int64_t r = a + warp * (32 / cg) + sub;
-      constexpr int UN = 4;
-      for (; r + (UN - 1) * rstep < b; r += UN * rstep) {
-        float q[UN][VEC];
 #pragma unroll
-        for (int u = 0; u < UN; ++u) {
-          const float* src = x + (size_t)(r + u * rstep) * d + c;
-          if (VEC == 4) *reinterpret_cast<float4*>(q[u]) = __ldg(reinterpret_cast<const float4*>(src));
-          else q[u][0] = __ldg(src);
-        }
+      for (int u = 0; u < UN; ++u) take(q[u]);
+    }
+    for (; r < b; r += rstep) {
+      float q[VEC];
+      const float* src = x + (size_t)r * d + c;
+      if (VEC == 4) *reinterpret_cast<float4*>(q) = __ldg(reinterpret_cast<const float4*>(src));
+      else q[0] = __ldg(src);
+      take(q);
+    }
+  }
 #pragma unroll
-        for (int u = 0; u < UN; ++u) take(q[u]);
+  for (int v = 0; v < VEC; ++v) {
+    smn[warp][lane * VEC + v] = mn[v];
+    smx[warp][lane * VEC + v] = mx[v];
+  }
+  __syncthreads();
+  for (int j = threadIdx.x; j < cg * VEC; j += SR_WARPS * 32) {
+    if (c0 + j >= d) break;
+    float m0 = INFINITY, m1 = -INFINITY;
+    for (int w = 0; w < SR_WARPS; ++w)
+      for (int q = j; q < 32 * VEC; q += cg * VEC) {
+        m0 = fminf(m0, smn[w][q]);
+        m1 = fmaxf(m1, smx[w][q]);
       }
-      for (; r < b; r += rstep) {
-        float q[VEC];
-        const float* src = x + (size_t)r * d + c;
-        if (VEC == 4) *reinterpret_cast<float4*>(q) = __ldg(reinterpret_cast<const float4*>(src));
-        else q[0] = __ldg(src);
-        take(q);
-      }
-    }
-#pragma unroll
-    for (int v = 0; v < VEC; ++v) {
-      smn[warp][lane * VEC + v] = mn[v];
-      smx[warp][lane * VEC + v] = mx[v];
-    }
-    __syncthreads();
-    for (int j = threadIdx.x; j < cg * VEC; j += SR_WARPS * 32) {
-      if (c0 + j >= d) break;
-      float m0 = INFINITY, m1 = -INFINITY;
-      for (int w = 0; w < SR_WARPS; ++w)
-        for (int q = j; q < 32 * VEC; q += cg * VEC) {
-          m0 = fminf(m0, smn[w][q]);
-          m1 = fmaxf(m1, smx[w][q]);
-        }
-      atomicMin(lo + (size_t)set * d + c0 + j, float_rank(m0));
-      atomicMax(hi + (size_t)set * d + c0 + j, float_rank(m1));
-    }
-    __syncthreads();
-    a = b;
+    atomicMin(lo + (size_t)set * d + c0 + j, float_rank(m0));
+    atomicMax(hi + (size_t)set * d + c0 + j, float_rank(m1));
   }
   if (bad) hf_raise(err, HF_ERRBIT_NONFINITE);
 }
@@ -444,11 +456,11 @@ void launch_seg_range(const float* x, int64_t n, int d, const int64_t* off, cons
   int64_t rpb = (n * ychunks + 152 * 8 - 1) / (152 * 8);
   const int64_t least = (int64_t)SR_WARPS * (32 / cg) * 4;
   if (rpb < least) rpb = least;
-  const dim3 grid(hf_blocks(n, (int)rpb), (unsigned)ychunks);
+  const dim3 grid((unsigned)nseg + hf_blocks(n, (int)rpb), (unsigned)ychunks);
   if (v4)
-    seg_range_kernel<4><<<grid, SR_WARPS * 32, 0, s>>>(x, n, d, off, seg, rpb, cg, ulo, uhi, err);
+    seg_range_kernel<4><<<grid, SR_WARPS * 32, 0, s>>>(x, n, d, off, nseg, seg, rpb, cg, ulo, uhi, err);
   else
-    seg_range_kernel<1><<<grid, SR_WARPS * 32, 0, s>>>(x, n, d, off, seg, rpb, cg, ulo, uhi, err);
+    seg_range_kernel<1><<<grid, SR_WARPS * 32, 0, s>>>(x, n, d, off, nseg, seg, rpb, cg, ulo, uhi, err);
   hf_after_launch("seg_range_kernel", s);
   seg_range_final_kernel<<<hf_blocks(count, 256), 256, 0, s>>>(count, bits, lo, scale);
   hf_after_launch("seg_range_final_kernel", s);
