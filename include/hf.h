@@ -200,8 +200,9 @@ int hf_search_static(hf_forest* f, const float* queries, int64_t nq, int32_t k, 
  * lists set 0's points first (in their own Hilbert order), then set 1's, ...
  * hf_knn_graph then gives, for every row, exactly the lists hf_build +
  * hf_knn_graph give on that set alone (plain and sketch forms), with row
- * indices of the stacked matrix (subtract offsets[s]). Tensor forms, the
- * budgeted graph and search return HF_ENOTIMPL on a segmented forest.
+ * indices of the stacked matrix (subtract offsets[s]); the tensor forms take
+ * their candidates from the row's own set too. The budgeted graph and search
+ * return HF_ENOTIMPL on a segmented forest.
  */
 #define HF_MAX_SETS 256
 int hf_build_segmented(const float* points, const int64_t* offsets, int32_t nsets, int32_t d, int32_t T,
