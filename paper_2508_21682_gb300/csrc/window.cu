@@ -38,6 +38,7 @@ namespace {
 constexpr int DC = 16;          // coordinates per staged chunk
 constexpr int UR = 8;           // rows per unit
 constexpr int UC = 8;           // offsets per unit
+constexpr int kSms = 152;
 // Memory of one chunk's band.
 constexpr size_t BAND_BYTES = (size_t)256 << 20;
 
@@ -357,14 +358,20 @@ int launch_pairs(PairArgs a, int dlo, int ytiles, int64_t cols, cudaStream_t s) 
 
 // Offsets 1 .. w in tiles of 64 (256 rows; the fewest staged rows per pair),
 // the rest in tiles of 32 (512 rows) and 16 (512 rows of 128 threads), so that
-// at most 15 offsets are computed beyond w. nt = 512, for plans that ask for it
-// (the tuner tries both): 64-offset tiles of 512 rows, one block per SM; at
-// windows from 64 to 704 between 3 % faster (20,000 x 384, w = 128) and 12 %
-// slower (100,003 x 100, w = 64) than nt = 256, 50 % on 20,000 x 384 at w = 64.
+// at most 15 offsets are computed beyond w. A launch that leaves SMs idle lasts
+// as long as one block, and rows that are not 16-byte aligned are staged in 4-byte
+// copies, fewer per thread in the tiles of 64: they take such a launch's rest too
+// (200 x 33, T = 8, w = 2: 0.30 -> 0.24 ms the graph; aligned rows are bound by
+// the arithmetic, which the wider tile has more of: 200 x 384: 0.75 -> 0.86).
+// nt = 512, for plans that ask for it (the tuner tries both): 64-offset tiles of
+// 512 rows, one block per SM; at windows from 64 to 704 between 3 % faster
+// (20,000 x 384, w = 128) and 12 % slower (100,003 x 100, w = 64) than nt = 256,
+// 50 % on 20,000 x 384 at w = 64.
 template <bool HAM>
 int launch_band(const PairArgs& a, int64_t cols, int nt, cudaStream_t s) {
   int full = a.w / 64, rest = a.w % 64;
-  if (rest > 48) {
+  const bool vec = a.d % 4 == 0 && (reinterpret_cast<uintptr_t>(a.x) & 15) == 0;
+  if (rest > 48 || (rest > 0 && !vec && nt != 512 && (cols + 255) / 256 * (full + 1) <= kSms)) {
     ++full;
     rest = 0;
   }
