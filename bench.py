@@ -52,7 +52,7 @@ MODES = {"plain": 0, "tensor": 1, "fp8": 2}
 # DRAM traffic of the dominant kernels from one ncu capture of a 1M-point
 # launch (bytes per point, scaled by n here) and the source file it was taken
 # on; a figure is dropped (null) once its source differs.
-WINDOW_TRAFFIC = {"bytes_per_point": 2065, "source_sha": "194a8354b9341b42", "file": "window.cu"}   # w = 32, pair_kernel + merge_kernel
+WINDOW_TRAFFIC = {"bytes_per_point": 2065, "source_sha": "4a28b09c422b9770", "file": "window.cu"}   # w = 32, pair_kernel + merge_kernel
 GRAM_TRAFFIC = {"bytes_per_point": 1139, "source_sha": "23ffe7e70668a4e5", "file": "gram.cu", "w": 1024}
 
 # GB300: 152 SMs x 128 FP32 lanes; one pair-coordinate update of the exact-
