@@ -196,7 +196,7 @@ void destroy(hf_forest* f, cudaStream_t s) {
   dfree(f->plan_xs, s);
   dfree(f->plan_ms, s);
   dfree(f->plan_band, s);
-  dfree(f->plan_band_first, s);
+  for (float* b : f->plan_bands_before) dfree(b, s);
   dfree(f->plan_thr, s);
   if (f->side) {
     cudaStreamSynchronize(s);  // the stream-ordered frees above run before the side stream goes
@@ -809,11 +809,17 @@ int hf_graph_plan(hf_forest* f, int32_t k, int32_t w, int32_t threads, void* str
   cudaError_t e = cudaSuccess;
   // the band first: when there is no room for it, the earlier plan stands
   if (!form && window_band_bytes(n, w) > f->plan_band_bytes) {
-    const size_t bytes = f->plan_band ? window_band_bytes_most(n) : window_band_bytes(n, w);
+    const size_t need = window_band_bytes(n, w);
+    size_t bytes = f->plan_band ? window_band_bytes_most(n) : need;
     float* band = nullptr;
     e = dalloc(&band, bytes / sizeof(float), s);
+    if (e != cudaSuccess && bytes > need) {
+      cudaGetLastError();
+      bytes = need;
+      e = dalloc(&band, bytes / sizeof(float), s);
+    }
     if (e != cudaSuccess) return map_cuda(e);
-    f->plan_band_first = f->plan_band;  // null, or the only band so far
+    if (f->plan_band) f->plan_bands_before.push_back(f->plan_band);
     f->plan_band = band;
     f->plan_band_bytes = bytes;
   }

@@ -119,10 +119,10 @@ struct hf_forest {
   // hold the address, and a plan of another window with the same list width
   // must leave them runnable: a band is kept until hf_free. The first plan takes
   // what its window needs, the first wider one the most that any window can
-  // need, so there are two at most.
+  // need, so there are two at most (more only where that much finds no room).
   float* plan_band = nullptr;
   size_t plan_band_bytes = 0;
-  float* plan_band_first = nullptr;
+  std::vector<float*> plan_bands_before;
   int plan_k = 0, plan_w = 0, plan_kp = 0, plan_nt = 0, plan_form = 0;
   int sketch_k2 = 60;     // candidates kept by Hamming distance (mode 3)
   int expand_h = 2;       // master-order neighbours per survivor (mode 3 search)
